@@ -12,7 +12,7 @@
 //       nodes and the radial current K_c of each cell (pass_currents);
 //   P2  E_z = d_xi psi (Eq. 7) by a block-wide inward scan of the cell currents; Q = P + E_z U;
 //       B_theta from Eq. 6 differentiated in r (Helmholtz form, shift chi), a tridiagonal
-//       system solved by block-wide parallel cyclic reduction on row sums (solve_fields);
+//       system solved on row sums by one warp (solve_fields);
 //   P3  per ring: the Cartesian radial force (gamma/Gamma) psi' - B_theta (Eqs. 4-5 with the
 //       centrifugal term carried by the local frame), the move to the next stage's position,
 //       and that position's charge deposit (linear hats).
@@ -77,6 +77,26 @@ __device__ __forceinline__ double wide_of<double, double>(double x) { return x; 
 template <>
 __device__ __forceinline__ FF wide_of<FF, float>(float x) { return FF{x, 0.f}; }
 
+// 64-bit fixed point (the mixed forms' charge): the prefix sums are integer and exact
+__device__ __forceinline__ long long wide_add(long long a, long long b) { return a + b; }
+__device__ __forceinline__ long long wide_shfl_up(long long a, int o) { return __shfl_up_sync(kFull, a, o); }
+__device__ __forceinline__ long long wide_shfl_down(long long a, int o) { return __shfl_down_sync(kFull, a, o); }
+__device__ __forceinline__ long long wide_shfl_idx(long long a, int l) { return __shfl_sync(kFull, a, l); }
+template <>
+__device__ __forceinline__ long long wide_zero<long long>() { return 0; }
+
+// 1/x.  FP32: the unit's division (a reciprocal instruction in the fast units).  FP64: the
+// hardware's approximation (about 20 bits) and one third-order Newton step r (1 + e + e^2),
+// e = 1 - x r, which leaves about an ulp: three FP64 instructions after the seed, where GB300's
+// narrow FP64 pipe makes an IEEE division cost three times as many.
+__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_of(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // exclusive prefix over the lanes of one warp of per-lane totals (lane 0 gets 0)
 template <class W>
 __device__ __forceinline__ W warp_excl_prefix(W v, int lane) {
@@ -127,7 +147,6 @@ struct PolFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kWarpPCR = false;      // the tridiagonal solve finished per warp
   static constexpr int kScanE = 3;  // nodes per thread in the block scans: n1 <= kScanE * NT
 };
 struct PolMixed {
@@ -144,7 +163,6 @@ struct PolMixed {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kWarpPCR = true;      // the tridiagonal solve finished per warp
   static constexpr int kScanE = 3;
 };
 // The precision split in which only the particle arithmetic is FP32: each ring's push and its
@@ -165,7 +183,6 @@ struct PolMixed64 {
   static constexpr bool kWinGlobal = true;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kWarpPCR = true;      // the tridiagonal solve finished per warp
   static constexpr int kScanE = 3;
 };
 // The mixed arithmetic for boxes too large for one CTA's shared memory to hold the rings
@@ -185,7 +202,6 @@ struct PolWide {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kWarpPCR = false;      // the tridiagonal solve finished per warp
   static constexpr int kScanE = 5;
 };
 
@@ -206,7 +222,6 @@ struct PolWideFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kWarpPCR = false;      // the tridiagonal solve finished per warp
   static constexpr int kScanE = 5;
 };
 // The slab geometry (x, xi) of a policy (Sec. I: WAKE handles slab and cylindrical geometry):
@@ -218,6 +233,10 @@ template <class P>
 struct SlabOf : P {
   static constexpr bool kSlab = true;
 };
+
+// Rows per lane of the tridiagonal solve (tri_solve_warp) of n rows, and the length of its arrays.
+__host__ __device__ constexpr int tri_per_lane(int n) { return (n + 31) >> 5; }
+__host__ __device__ constexpr int tri_len(int n) { return 33 * ((n + 31) >> 5); }
 
 // Ring slot arrays: cell index, offset in the cell, u_r, the constants l_z, Gamma_0, w, and
 // the stage-1 Gamma and radial force kept for the full step; with ids, each slot also carries
@@ -264,7 +283,7 @@ struct MarchSmem {
 
   __host__ __device__ static size_t bytes(int n1, int slots, bool ids = false) {
     size_t b = sizeof(typename Pol::W) * 64 + sizeof(typename Pol::Q) * 2 * (size_t)n1 + sizeof(Acc) * 6 * (size_t)n1 +
-               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + sizeof(N) * 4 * ((size_t)n1 + 32) + 256;
+               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + sizeof(N) * 4 * (size_t)tri_len(n1) + 256;
     b += sizeof(N) * (Pol::kTables ? 6 : 2) * (size_t)n1;
     if (Pol::kSortEvery > 0) b += sizeof(int) * ((size_t)n1 + 32);
     if (Pol::kSmemRings) b += RingSoA<R>::bytes(slots, ids) + 32;
@@ -287,10 +306,10 @@ struct MarchSmem {
     dpsi = rp; rp += n1;
     ez = rp; rp += n1;
     bth = rp; rp += n1;
-    ta = rp; rp += n1 + 32;
-    tb = rp; rp += n1 + 32;
-    tc = rp; rp += n1 + 32;
-    td = rp; rp += n1 + 32;
+    ta = rp; rp += tri_len(n1);
+    tb = rp; rp += tri_len(n1);
+    tc = rp; rp += tri_len(n1);
+    td = rp; rp += tri_len(n1);
     invR = invV = alpha = ga = gb = gc = nullptr;
     invR = rp; rp += n1;
     ga = rp; rp += n1;
@@ -316,7 +335,7 @@ struct MarchSmem {
   // The out-of-window ring queue: slot ids in the tridiagonal rows, which are free from the end
   // of one solve to the start of the next (a ring pass and the deposits that follow it)
   __device__ __forceinline__ int *queue() const { return (int *)ta; }
-  __device__ __forceinline__ int queue_cap(int n1) const { return (int)(4 * ((size_t)n1 + 32) * sizeof(N) / sizeof(int)); }
+  __device__ __forceinline__ int queue_cap(int n1) const { return (int)(4 * (size_t)tri_len(n1) * sizeof(N) / sizeof(int)); }
 };
 
 // ---------------------------------------------------------------------------------------
@@ -463,122 +482,101 @@ __device__ __forceinline__ FF q_to_wide<long long, FF>(long long d) {
   return FF{x.h * s, x.l * s};
 }
 
-// Block-wide parallel cyclic reduction on the row-sum form (see pcr_rowsum_solve below), every
-// doubling over the block with a barrier.  Double-buffered; returns the buffer holding the
-// result (x_q = d_q / s_q there).  Ends with a barrier.
-template <int NT, class S>
-__device__ __forceinline__ int pcr_rowsum(S *a0, S *s0, S *c0, S *d0, S *a1, S *s1, S *c1, S *d1, int n) {
-  int cur = 0;
-  for (int k = 1; k < n; k <<= 1) {
-    const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
-    S *an = cur ? a0 : a1, *sn = cur ? s0 : s1, *cn = cur ? c0 : c1, *dn = cur ? d0 : d1;
-    for (int q = threadIdx.x; q < n; q += NT) {
-      const S aq = a[q], cq = c[q];
-      S sq = sm_[q], dq = d[q], na = (S)0, nc = (S)0;
-      if (q - k >= 0) {
-        const S bm = sm_[q - k] - a[q - k] - c[q - k];
-        const S k1 = aq / bm;
-        sq -= k1 * sm_[q - k];
-        dq -= k1 * d[q - k];
-        na = -a[q - k] * k1;
-      }
-      if (q + k < n) {
-        const S bp = sm_[q + k] - a[q + k] - c[q + k];
-        const S k2 = cq / bp;
-        sq -= k2 * sm_[q + k];
-        dq -= k2 * d[q + k];
-        nc = -c[q + k] * k2;
-      }
-      an[q] = na;
-      sn[q] = sq;
-      cn[q] = nc;
-      dn[q] = dq;
-    }
-    __syncthreads();
-    cur ^= 1;
-  }
-  return cur;
-}
-
-// Parallel cyclic reduction (Hockney) on rows a_q x_{q-1} + b_q x_q + c_q x_{q+1} = d_q
-// stored as (a, s = a + b + c, c, d).  For this M-matrix (a, c >= 0, s < 0) the eliminated
-// row sum s' = s - k1 s_{q-k} - k2 s_{q+k} (k1 = a_q/b_{q-k}, k2 = c_q/b_{q+k}, both <= 0)
-// adds terms of one sign, so the margin of diagonal dominance is never lost to cancellation;
-// b = s - a - c likewise.  After ceil(log2 n) doublings a = c = 0 and x_q = d_q / s_q.
+// Tridiagonal rows a_q x_{q-1} + b_q x_q + c_q x_{q+1} = d_q, q = 0..n-1, given as (a, s = a + b +
+// c, c, d).  For this M-matrix (a, c >= 0, s < 0) an eliminated row's sum s' = s - k s_e (k = its
+// coupling / the eliminated row's b, k <= 0) adds terms of one sign, so the margin of diagonal
+// dominance is never lost to cancellation; b = s - a - c likewise.
 //
-// The first doublings (strides 1 .. ns/2) run over the block, double-buffered, one barrier
-// each.  They leave ns independent systems, rows r, r + ns, r + 2 ns, ... (ns the smallest
-// power of two >= NT/32 with n <= 32 ns); each is finished by one warp, lane l holding row
-// r + ns l, with the remaining doublings (lane strides 1 .. 16) done by shuffles.  The
-// arithmetic is that of the block form, stride for stride.  out(q, x_q) receives the solution.
-template <int NT, class S, class Out>
-__device__ __forceinline__ void pcr_rowsum_solve(S *a0, S *s0, S *c0, S *d0, S *a1, S *s1, S *c1, S *d1, int n,
-                                                 Out &&out) {
-  constexpr int W = NT / 32;
-  int ns = W;
-  while (32 * ns < n) ns <<= 1;
-  int cur = 0;
-  for (int k = 1; k < ns && k < n; k <<= 1) {
-    const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
-    S *an = cur ? a0 : a1, *sn = cur ? s0 : s1, *cn = cur ? c0 : c1, *dn = cur ? d0 : d1;
-    for (int q = threadIdx.x; q < n; q += NT) {
-      const S aq = a[q], cq = c[q];
-      S sq = sm_[q], dq = d[q], na = (S)0, nc = (S)0;
-      if (q - k >= 0) {
-        const S bm = sm_[q - k] - a[q - k] - c[q - k];
-        const S k1 = aq / bm;
-        sq -= k1 * sm_[q - k];
-        dq -= k1 * d[q - k];
-        na = -a[q - k] * k1;
-      }
-      if (q + k < n) {
-        const S bp = sm_[q + k] - a[q + k] - c[q + k];
-        const S k2 = cq / bp;
-        sq -= k2 * sm_[q + k];
-        dq -= k2 * d[q + k];
-        nc = -c[q + k] * k2;
-      }
-      an[q] = na;
-      sn[q] = sq;
-      cn[q] = nc;
-      dn[q] = dq;
-    }
-    __syncthreads();
-    cur ^= 1;
+// One warp solves the system.  Lane l holds the E = ceil(n / 32) consecutive rows l E .. l E + E - 1;
+// the last is its separator.  Two eliminations run side by side through the lane's rows: downwards
+// (each row left with the separator before, itself and the row after; the separator row with the
+// separators on its left and the next lane's first row) and upwards (which leaves the first row with
+// the two separators around it).  The 32 separators then form a tridiagonal system, solved by
+// parallel cyclic reduction over the lanes (Hockney), and the downward rows give the lane's other
+// unknowns.  The work is ~25 operations per row, against ~30 per row and doubling for a cyclic
+// reduction of all rows; the chain is E reciprocals and five doublings, without a block barrier.
+//
+// Row q lies at tri_at(q) of each array: rows of the same index in consecutive lanes are adjacent,
+// 33 entries apart from the next index's, so the lanes' reads and the rows' writers (consecutive q)
+// both spread over the shared-memory banks.
+struct TriAt {
+  int E;
+  unsigned m;  // ceil(2^32 / E): q / E for q < 2^16
+  __device__ __forceinline__ explicit TriAt(int n) : E(tri_per_lane(n)), m(0xffffffffu / (unsigned)tri_per_lane(n) + 1u) {}
+  __device__ __forceinline__ int operator()(int q) const {
+    const int lane = E == 1 ? q : (int)__umulhi((unsigned)q, m);
+    return (q - lane * E) * 33 + lane;
   }
-  const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
-  const int lane = threadIdx.x & 31;
-  for (int r = threadIdx.x >> 5; r < ns; r += W) {
-    const int q = r + ns * lane;
-    const bool on = q < n;  // rows past n: the identity (their neighbours' couplings to them are zero)
-    S aq = on ? a[q] : (S)0, sq = on ? sm_[q] : (S)1, cq = on ? c[q] : (S)0, dq = on ? d[q] : (S)0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const S am = __shfl_up_sync(kFull, aq, o), smm = __shfl_up_sync(kFull, sq, o);
-      const S cm = __shfl_up_sync(kFull, cq, o), dm = __shfl_up_sync(kFull, dq, o);
-      const S ap = __shfl_down_sync(kFull, aq, o), spp = __shfl_down_sync(kFull, sq, o);
-      const S cp = __shfl_down_sync(kFull, cq, o), dp = __shfl_down_sync(kFull, dq, o);
-      S s2 = sq, d2 = dq, na = (S)0, nc = (S)0;
-      if (lane >= o) {
-        const S bm = smm - am - cm;
-        const S k1 = aq / bm;
-        s2 -= k1 * smm;
-        d2 -= k1 * dm;
-        na = -am * k1;
+};
+
+// Called by one warp.  ta, ts, tc, td: the rows, 32 E of them (rows past n: a = c = d = 0, s = -1);
+// w: 3 tri_len(n) entries of scratch when E > 1.  out(q, x_q) receives the solution for q < n.
+template <class S, class Out>
+__device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S *tc, const S *td, S *w, int n, Out &&out) {
+  const int lane = threadIdx.x & 31, E = tri_per_lane(n), L = 33 * E;
+  S *wl = w, *wr = w + L, *wd = w + 2 * L;  // the downward rows: left coupling, 1/b, right-hand side
+  S aq = ta[lane], sq = ts[lane], cq = tc[lane], dq = td[lane];
+  if (E > 1) {
+    int u = (E - 2) * 33 + lane;  // the upward elimination starts at row E - 2
+    S ua = ta[u], us = ts[u], ur = tc[u], ud = td[u], urb = rcp_of(us - ua - ur);
+    S rb = rcp_of(sq - aq - cq);
+    wl[lane] = aq;
+    wr[lane] = rb;
+    wd[lane] = dq;
+    int v = lane;
+#pragma unroll 2
+    for (int e = 1; e < E; ++e) {
+      v += 33;
+      const S k = ta[v] * rb;
+      sq = ts[v] - k * sq;
+      dq = td[v] - k * dq;
+      aq = -k * aq;
+      cq = tc[v];
+      rb = rcp_of(sq - aq - cq);
+      wl[v] = aq;
+      wr[v] = rb;
+      wd[v] = dq;
+      if (e < E - 1) {
+        u -= 33;
+        const S ku = tc[u] * urb;
+        us = ts[u] - ku * us;
+        ud = td[u] - ku * ud;
+        ur = -ku * ur;
+        ua = ta[u];
+        urb = rcp_of(us - ua - ur);
       }
-      if (lane + o < 32) {
-        const S bp = spp - ap - cp;
-        const S k2 = cq / bp;
-        s2 -= k2 * spp;
-        d2 -= k2 * dp;
-        nc = -cp * k2;
-      }
-      aq = na;
-      sq = s2;
-      cq = nc;
-      dq = d2;
     }
-    if (on) out(q, dq / sq);
+    // the next lane's first row replaces its unknown in this separator row
+    const S ns = __shfl_down_sync(kFull, us, 1), nr = __shfl_down_sync(kFull, ur, 1);
+    const S nd = __shfl_down_sync(kFull, ud, 1), nrb = __shfl_down_sync(kFull, urb, 1);
+    const S k = lane < 31 ? cq * nrb : (S)0;
+    sq -= k * ns;
+    dq -= k * nd;
+    cq = -k * nr;
+  }
+  if (lane == 31) cq = (S)0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const S rb = rcp_of(sq - aq - cq);
+    const S am = __shfl_up_sync(kFull, aq, o), sm = __shfl_up_sync(kFull, sq, o);
+    const S dm = __shfl_up_sync(kFull, dq, o), rm = __shfl_up_sync(kFull, rb, o);
+    const S cp = __shfl_down_sync(kFull, cq, o), sp = __shfl_down_sync(kFull, sq, o);
+    const S dp = __shfl_down_sync(kFull, dq, o), rp = __shfl_down_sync(kFull, rb, o);
+    const S k1 = lane >= o ? aq * rm : (S)0, k2 = lane + o < 32 ? cq * rp : (S)0;
+    sq = sq - k1 * sm - k2 * sp;
+    dq = dq - k1 * dm - k2 * dp;
+    aq = -am * k1;
+    cq = -cp * k2;
+  }
+  S x = dq * rcp_of(sq);
+  const S up = __shfl_up_sync(kFull, x, 1), zl = lane == 0 ? (S)0 : up;
+  const int q0 = lane * E;
+  if (q0 + E - 1 < n) out(q0 + E - 1, x);
+#pragma unroll 2
+  for (int e = E - 2; e >= 0; --e) {
+    const int v = e * 33 + lane;
+    x = (wd[v] - wl[v] * zl - tc[v] * x) * wr[v];
+    if (q0 + e < n) out(q0 + e, x);
   }
 }
 
@@ -642,12 +640,15 @@ __device__ __forceinline__ void solve_psi(MarchSmem<Pol> &sm, const NodeGeo<Pol>
   using R = typename Pol::N;
   using W = typename Pol::W;
   const int nr = geo.nr, n1 = nr + 1;
-  block_scan_fused<NT, Pol::kScanE, false, W>(
-      n1, wtot, [&](int m) { return q_to_wide<typename Pol::Q, W>(sm.rho[m] - sm.rho0[m]); },
-      [&](int m, W incl) {
+  using Q = typename Pol::Q;
+  static_assert(sizeof(Q) <= sizeof(W), "the charge scan's totals lie in wtot");
+  block_scan_fused<NT, Pol::kScanE, false, Q>(
+      n1, (Q *)wtot, [&](int m) { return sm.rho[m] - sm.rho0[m]; },
+      [&](int m, Q sum) {
         R dp = (R)0;
         if (m > 0) {
-          const R v = (R)wide_value(q_to_wide<typename Pol::Q, W>(sm.rho[m] - sm.rho0[m]));
+          const W incl = q_to_wide<Q, W>(sum);
+          const R v = (R)wide_value(q_to_wide<Q, W>(sm.rho[m] - sm.rho0[m]));
           dp = (R)wide_value(wide_add(incl, wide_of<W, R>(-((R)1 - geo.alpha(m)) * v))) * geo.metric(m);
         }
         sm.dpsi[m] = dp;
@@ -683,37 +684,38 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
   // rows) read where the rows need them
   auto dens = [&](const Acc *v, int m) -> R { return (R)v[m] * geo.invV(m); };
   auto jz_node = [&](int m) -> R { return (R)sm.jz[m] * geo.invV(m) - (R)0.5 * ((R)nbA[m] + (R)nbB[m]); };
-  // rows q = 0..nr-1 (node i = q + 1): central differences, a half cell at the wall
+  // rows q = 0..nr-1 (node i = q + 1): central differences, a half cell at the wall; the rows
+  // past them up to whole lanes are -x = 0
   const R i2dr = (R)0.5 * inv_dr;
-  for (int q = tid; q < nr; q += NT) {
-    const int i = q + 1;
-    const R Qi = dens(sm.P, i) + sm.ez[i] * dens(sm.U, i);
-    const R Ti = dens(sm.T, i);
-    R a, c, sgeo;
-    geo.row(q, a, c, sgeo);
-    R rhs;
-    if (i < nr)
-      rhs = (jz_node(i + 1) - jz_node(i - 1)) * i2dr + Qi + (dens(sm.T, i + 1) - dens(sm.T, i - 1)) * i2dr +
-            Ti * geo.curv(i);
-    else
-      rhs = Qi + (Ti - dens(sm.T, i - 1)) * inv_dr + Ti * geo.curv(i) - (jz_node(i - 1) + jz_node(i)) * inv_dr;
-    sm.ta[q] = a;
-    sm.tb[q] = sgeo - dens(sm.chi, i);  // row sum a + b + c (both terms negative)
-    sm.tc[q] = c;
-    sm.td[q] = rhs;
+  const TriAt at(nr);
+  const int nrows = 32 * at.E;
+  for (int q = tid; q < nrows; q += NT) {
+    R a = (R)0, c = (R)0, s = (R)-1, rhs = (R)0;
+    if (q < nr) {
+      const int i = q + 1;
+      const R Qi = dens(sm.P, i) + sm.ez[i] * dens(sm.U, i);
+      const R Ti = dens(sm.T, i);
+      geo.row(q, a, c, s);
+      s -= dens(sm.chi, i);  // row sum a + b + c (both terms negative)
+      if (i < nr)
+        rhs = (jz_node(i + 1) - jz_node(i - 1)) * i2dr + Qi + (dens(sm.T, i + 1) - dens(sm.T, i - 1)) * i2dr +
+              Ti * geo.curv(i);
+      else
+        rhs = Qi + (Ti - dens(sm.T, i - 1)) * inv_dr + Ti * geo.curv(i) - (jz_node(i - 1) + jz_node(i)) * inv_dr;
+    }
+    const int r = at(q);
+    sm.ta[r] = a;
+    sm.tb[r] = s;
+    sm.tc[r] = c;
+    sm.td[r] = rhs;
   }
   __syncthreads();
-  // parallel cyclic reduction (on row sums); the second buffer reuses the deposit arrays J_z, chi, T, P,
-  // which are dead once the rows are set up (they are zeroed before the next pass B)
-  static_assert(sizeof(Acc) == sizeof(R), "PCR buffer reuses deposit arrays");
-  if constexpr (Pol::kWarpPCR) {
-    pcr_rowsum_solve<NT, R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, (R *)sm.chi, (R *)sm.T, (R *)sm.P, nr,
-                            [&](int q, R x) { sm.bth[q + 1] = x; });  // row q is node q + 1
+  // one warp solves; its scratch reuses the six deposit arrays (contiguous, dead once the rows are
+  // set up, zeroed before the next pass B): 3 tri_len(nr) <= 6 (nr + 1) whenever nr > 32
+  static_assert(sizeof(Acc) == sizeof(R), "the solver's scratch reuses the deposit arrays");
+  if (tid < 32) {
+    tri_solve_warp<R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, nr, [&](int q, R x) { sm.bth[q + 1] = x; });
     if (tid == 0) sm.bth[0] = (R)0;
-  } else {
-    const int cur = pcr_rowsum<NT, R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, (R *)sm.chi, (R *)sm.T, (R *)sm.P, nr);
-    const R *bb = cur ? (const R *)sm.chi : sm.tb, *dd = cur ? (const R *)sm.P : sm.td;  // row sum = diagonal now
-    for (int m = tid; m < n1; m += NT) sm.bth[m] = m > 0 ? dd[m - 1] / bb[m - 1] : (R)0;
   }
   __syncthreads();
 }
@@ -1269,7 +1271,7 @@ __device__ __forceinline__ void resort_rings(MarchSmem<Pol> &sm, const RingSoA<t
 
 // The march of one simulation by one CTA.  Hooks supply the beam-density rows and receive
 // each slice's fields (see PlainHooks; the pipelined beam step adds its own):
-//   bool wait_rows(int k)           rows k, k+1 may be read (false: give up, block-uniform)
+//   bool wait_row(int row)          rows up to this one may be read (false: give up, block-uniform)
 //   R    nb_row(int row, int m)     beam density at node m of a row
 //   void slice_done(int k, sm)      stage-1 fields of slice k are in sm (psi, dpsi, ez, bth)
 //   void finish(sm)                 after the last slice
@@ -1400,25 +1402,12 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
   for (int k = 0; k <= nxi; ++k) {
     if (Pol::kSortEvery > 0 && k > 0 && k % Pol::kSortEvery == 0) resort_rings<Pol, NT, PPT, kIds>(sm, rs, np, nr);
     const R *nbk = (k & 1) ? sm.nb1 : sm.nb0, *nbk1 = (k & 1) ? sm.nb0 : sm.nb1;
-    if (!hk.wait_rows(k)) break;
-    if (k == 0)  // row 0 is first read in P2, after two barriers
+    if (k == 0) {  // row 0 is first read in P2, after two barriers
+      if (!hk.wait_row(0)) break;
       for (int m = tid; m < n1; m += NT) sm.nb0[m] = hk.nb_row(0, m);
-    // prefetch beam-density row k+1 (stored in phase P1); n1 <= 3 NT
-    R pre[3] = {(R)0, (R)0, (R)0};
-    if (k < nxi) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (tid + q * NT < n1) pre[q] = hk.nb_row(k + 1, tid + q * NT);
     }
     // ======== stage 1 at xi_k ========
     solve_psi<Pol, NT>(sm, geo, sm.wtot);  // P0
-    __syncthreads();
-    if (k < nxi) {  // P1
-      R *dst = (k & 1) ? sm.nb0 : sm.nb1;
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (tid + q * NT < n1) dst[tid + q * NT] = pre[q];
-    }
     for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
     {
       R Gs[PPT], gqs[PPT];
@@ -1437,7 +1426,6 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     drain_queue<NT>(sm, n1, cur_miss1);
     if constexpr (kTrap) hk.template trap_rings<NT, PPT>(k, rs, np);  // after every stage-1 deposit
     solve_fields<Pol, NT>(sm, geo, nbk, nbk, sm.wtot);  // P2
-    __syncthreads();
     // P3: fields of slice k, then the move to the midpoint and its charge deposit
     hk.slice_done(k, sm);
     if (k == nxi) break;
@@ -1481,9 +1469,22 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     }
     __syncthreads();
     // ======== stage 2 at xi_k + dxi/2 ========
+    // beam-density row k+1, first read by this stage: fetched here, stored in P1 (n1 <= 3 NT).
+    // (Waiting for it only here, not at the start of the slice, lets a pipelined step follow the
+    // step before it by two slices and two pushes instead of two and a half and three.)
+    if (!hk.wait_row(k + 1)) break;
+    R pre[3] = {(R)0, (R)0, (R)0};
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (tid + q * NT < n1) pre[q] = hk.nb_row(k + 1, tid + q * NT);
     solve_psi<Pol, NT>(sm, geo, sm.wtot);  // P0
-    __syncthreads();
-    for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;  // P1
+    {  // P1
+      R *dst = (k & 1) ? sm.nb0 : sm.nb1;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (tid + q * NT < n1) dst[tid + q * NT] = pre[q];
+    }
+    for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
     pass_currents<Pol, NT, PPT, kTrap>(sm, rs, np, nr, dR, d.status,
                                 [&](int p, int, int &c, R &f, R &u_r, R &u_t) {
                                   c = MC[p];
@@ -1495,7 +1496,6 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     __syncthreads();
     drain_queue<NT>(sm, n1, cur_miss2);
     solve_fields<Pol, NT>(sm, geo, nbk, nbk1, sm.wtot);  // P2
-    __syncthreads();
     // P3: full step from the slice-k state with the midpoint derivative, and the charge
     // deposit of the new slice
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
@@ -1559,7 +1559,7 @@ struct PlainHooks {
   G *opsi, *oez, *oer, *obth;
   int n1;
   int *status;
-  __device__ __forceinline__ bool wait_rows(int) { return true; }
+  __device__ __forceinline__ bool wait_row(int) { return true; }
   __device__ __forceinline__ R nb_row(int row, int m) const { return (R)nb[(size_t)row * n1 + m]; }
   __device__ __forceinline__ void slice_done(int k, MarchSmem<Pol> &sm) {
     if (!opsi) return;  // a timing probe of the tile autotuner keeps no output

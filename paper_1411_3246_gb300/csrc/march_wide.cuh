@@ -201,26 +201,12 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
   for (int k = 0; k <= nxi; ++k) {
     if (Pol::kSortEvery > 0 && k > 0 && k % Pol::kSortEvery == 0) resort_rings_wide<Pol, NT, PPT>(sm, wr, np, nr, nch);
     const R *nbk = (k & 1) ? sm.nb1 : sm.nb0, *nbk1 = (k & 1) ? sm.nb0 : sm.nb1;
-    if (!hk.wait_rows(k)) break;
-    if (k == 0)
+    if (k == 0) {
+      if (!hk.wait_row(0)) break;
       for (int m = tid; m < n1; m += NT) sm.nb0[m] = hk.nb_row(0, m);
-    R pre[PRE];
-#pragma unroll
-    for (int q = 0; q < PRE; ++q) pre[q] = (R)0;
-    if (k < nxi) {
-#pragma unroll
-      for (int q = 0; q < PRE; ++q)
-        if (tid + q * NT < n1) pre[q] = hk.nb_row(k + 1, tid + q * NT);
     }
     // ======== stage 1 at xi_k ========
     solve_psi<Pol, NT>(sm, geo, sm.wtot);
-    __syncthreads();
-    if (k < nxi) {
-      R *dst = (k & 1) ? sm.nb0 : sm.nb1;
-#pragma unroll
-      for (int q = 0; q < PRE; ++q)
-        if (tid + q * NT < n1) dst[tid + q * NT] = pre[q];
-    }
     for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
     for (int ch = 0; ch < nch; ++ch) {
       base = ch * SLOTS;
@@ -239,7 +225,6 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     }
     __syncthreads();
     solve_fields<Pol, NT>(sm, geo, nbk, nbk, sm.wtot);
-    __syncthreads();
     hk.slice_done(k, sm);
     if (k == nxi) break;
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
@@ -270,8 +255,20 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     }
     __syncthreads();
     // ======== stage 2 at xi_k + dxi/2 ========
+    if (!hk.wait_row(k + 1)) break;  // row k+1 is first read by this stage
+    R pre[PRE];
+#pragma unroll
+    for (int q = 0; q < PRE; ++q) {
+      pre[q] = (R)0;
+      if (tid + q * NT < n1) pre[q] = hk.nb_row(k + 1, tid + q * NT);
+    }
     solve_psi<Pol, NT>(sm, geo, sm.wtot);
-    __syncthreads();
+    {
+      R *dst = (k & 1) ? sm.nb0 : sm.nb1;
+#pragma unroll
+      for (int q = 0; q < PRE; ++q)
+        if (tid + q * NT < n1) dst[tid + q * NT] = pre[q];
+    }
     for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
     for (int ch = 0; ch < nch; ++ch) {
       base = ch * SLOTS;
@@ -291,7 +288,6 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     }
     __syncthreads();
     solve_fields<Pol, NT>(sm, geo, nbk, nbk1, sm.wtot);
-    __syncthreads();
     // full step from the slice-k state with the midpoint derivative; charge of the new slice
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     for (int ch = 0; ch < nch; ++ch) {

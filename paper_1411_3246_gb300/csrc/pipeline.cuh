@@ -92,12 +92,12 @@ struct PipeHooks {
 
   __device__ __forceinline__ const G *grid(int s) const { return (const G *)a.grids + (size_t)s * a.ng; }
 
-  // rows <= k+1 of this step's grid are final once progress[t-1] >= min(nxi, k + 2).  Thread 0
-  // polls (bounded; it also gives up as soon as another CTA has timed out), every thread then
-  // meets at one barrier, so the decision is uniform.
-  __device__ __forceinline__ bool wait_rows(int k) {
+  // rows up to `row` of this step's grid are final once progress[t-1] >= min(nxi, row + 1).
+  // Thread 0 polls (bounded; it also gives up as soon as another CTA has timed out), every thread
+  // then meets at one barrier, so the decision is uniform.
+  __device__ __forceinline__ bool wait_row(int row) {
     if (t == 0) return true;
-    const int need = min(nxi, k + 2);
+    const int need = min(nxi, row + 1);
     if (threadIdx.x == 0 && ctl[1] < need) {
       long long it = 0;
       int v = ld_acquire(&a.progress[t - 1]);
