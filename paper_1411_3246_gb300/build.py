@@ -15,7 +15,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # flush denormals; every other translation unit keeps IEEE division and sqrt
 _FAST = ["--prec-div=false", "--prec-sqrt=false", "--ftz=true"]
 EXTRA = {"march_mixed.cu": _FAST, "march_mixed_small.cu": _FAST, "march_wide.cu": _FAST, "march_ext_mixed.cu": _FAST,
-         "march_mixed64.cu": _FAST}
+         "march_mixed64.cu": _FAST, "march_cluster_mixed.cu": _FAST}
 
 
 def sources():

@@ -50,8 +50,16 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
   const float h = s + e;
   return FF{h, e - (h - s)};
 }
+// The scans' sum: the rounding error of the high parts (two-sum) joins the low parts, without a
+// renormalisation at each level, so a level's chain is a shuffle and two adds instead of nine (the
+// error is formed beside the next level's shuffle).  The low part stays below n ulp of the high one.
+__device__ __forceinline__ FF ff_sum(FF a, FF b) {
+  const float s = a.h + b.h;
+  const float bb = s - a.h;
+  return FF{s, (a.l + b.l) + ((a.h - (s - bb)) + (b.h - bb))};
+}
 __device__ __forceinline__ double wide_add(double a, double b) { return a + b; }
-__device__ __forceinline__ FF wide_add(FF a, FF b) { return ff_add(a, b); }
+__device__ __forceinline__ FF wide_add(FF a, FF b) { return ff_sum(a, b); }
 __device__ __forceinline__ double wide_shfl_up(double a, int o) { return __shfl_up_sync(kFull, a, o); }
 __device__ __forceinline__ FF wide_shfl_up(FF a, int o) {
   return FF{__shfl_up_sync(kFull, a.h, o), __shfl_up_sync(kFull, a.l, o)};
@@ -97,6 +105,39 @@ __device__ __forceinline__ double rcp_of(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// 1/sqrt(x) (x > 0) and sqrt(x).  FP32: the unit's square root and division.  FP64: the
+// hardware's approximation y and one third-order Newton step y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2;
+// the root x y is corrected once.
+__device__ __forceinline__ void root_of(float x, float &r, float &ir) {
+  r = sqrtf(x);
+  ir = 1.0f / r;
+}
+__device__ __forceinline__ void root_of(double x, double &r, double &ir) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  y = fma(fma(0.375, e, 0.5), e * y, y);
+  const double g = x * y;
+  r = fma(fma(-g, g, x), 0.5 * y, g);
+  ir = y;
+}
+// The smallest square, and the smallest radius, that the reciprocals above take (FP64: the
+// approximations flush what is near the underflow; smaller counts as the axis).
+template <class R>
+__device__ __forceinline__ constexpr R tiny_r2() { return sizeof(R) == 8 ? (R)1e-290 : (R)0; }
+template <class R>
+__device__ __forceinline__ constexpr R tiny_r() { return sizeof(R) == 8 ? (R)1e-145 : (R)0; }
+// 1/a and 1/b: in FP64 from one reciprocal of the product (the FP64 pipe is the march's bound).
+__device__ __forceinline__ void rcp_pair(float a, float b, float &ia, float &ib) {
+  ia = rcp_of(a);
+  ib = rcp_of(b);
+}
+__device__ __forceinline__ void rcp_pair(double a, double b, double &ia, double &ib) {
+  const double t = rcp_of(a * b);
+  ia = t * b;
+  ib = t * a;
+}
+
 // exclusive prefix over the lanes of one warp of per-lane totals (lane 0 gets 0)
 template <class W>
 __device__ __forceinline__ W warp_excl_prefix(W v, int lane) {
@@ -120,6 +161,60 @@ __device__ __forceinline__ W warp_excl_suffix(W v, int lane) {
   }
   const W ex = wide_shfl_down(incl, 1);
   return lane == 31 ? wide_zero<W>() : ex;
+}
+
+// ---------------------------------------------------------------------------------------
+// thread-block clusters: one simulation marched by several CTAs (Hooks::kCluster).  Each CTA
+// holds a share of the rings and deposits them into its own node arrays; the arrays are summed
+// over the cluster through distributed shared memory, and every CTA then solves the fields for
+// itself from the same sums.
+// ---------------------------------------------------------------------------------------
+constexpr int kMaxCluster = 8;
+__device__ __forceinline__ int cl_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ int cl_size() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cl_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// this CTA's shared address p in the CTA of the given rank
+template <class T>
+__device__ __forceinline__ T *cl_peer(T *p, int rank) {
+  unsigned long long q;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(p), "r"(rank));
+  return reinterpret_cast<T *>(q);
+}
+__device__ __forceinline__ long long cl_add(long long a, long long b) { return a + b; }
+__device__ __forceinline__ double cl_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 cl_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+// a[0..n-1] of every CTA of the cluster replaced by the sum over the CTAs, in place.  CTA r sums
+// the r-th share of the elements (in rank order, so every CTA holds the same bits) and writes the
+// sums to all: nobody else touches that share between the two barriers.  n elements cross the
+// cluster twice, and a CTA may change its array freely before the first and after the second.
+template <int NT, class V>
+__device__ __forceinline__ void cluster_sum(V *a, int n, int cn, int cr) {
+  cl_barrier();
+  const int per = (n + cn - 1) / cn, beg = cr * per, end = min(n, beg + per);
+  for (int i = beg + threadIdx.x; i < end; i += NT) {
+    V v[kMaxCluster];
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r)
+      if (r < cn) v[r] = *cl_peer(a + i, r);
+    V s = v[0];
+#pragma unroll
+    for (int r = 1; r < kMaxCluster; ++r)
+      if (r < cn) s = cl_add(s, v[r]);
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r)
+      if (r < cn) *cl_peer(a + i, r) = s;
+  }
+  cl_barrier();
 }
 
 // ---------------------------------------------------------------------------------------
@@ -222,6 +317,11 @@ struct PolWideFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
+  static constexpr int kScanE = 5;
+};
+// A policy marched by clusters of narrower CTAs (march_cluster_*.cu).
+template <class P>
+struct ClusterOf : P {
   static constexpr int kScanE = 5;
 };
 // The slab geometry (x, xi) of a policy (Sec. I: WAKE handles slab and cylindrical geometry):
@@ -447,20 +547,15 @@ __device__ __forceinline__ FF two_prod(float a, float b) {
   const float p = a * b;
   return FF{p, __fmaf_rn(a, b, -p)};
 }
-// x rounded to the nearest integer (ties to even), as a 64-bit integer, from 32-bit
-// instructions only (the 64-bit conversions run on the slow FP64 pipe): below 2^31 in
-// magnitude the 32-bit conversion rounds it; above, x has 24 significant bits and is an
-// integer, given exactly by its significand shifted by its exponent.  |x| < 2^63.
+// x rounded to the nearest integer (ties to even), as a 64-bit integer, from 32-bit instructions
+// only (the 64-bit conversions run on the slow FP64 pipe): x = h 2^31 + l with h the nearest
+// integer to x 2^-31; the remainder l, at most 2^30, is exact.  |x| < 2^62.  (One path without a
+// branch: selecting between a short and a long form by the size of x made the charge passes slower
+// than the long form alone, the 200-step blowout run 191 ms against 175.)
 __device__ __forceinline__ long long f2q(float x) {
-  const int b = __float_as_int(x);
-  int e = ((b >> 23) & 0xff) - 150;  // x = m 2^e
-  e = e < 0 ? 0 : (e > 40 ? 40 : e);
-  const long long m = (long long)((b & 0x7fffff) | 0x800000) << e;
-  const bool small = fabsf(x) < 2147483648.f;
-  const long long r = (long long)__float2int_rn(small ? x : 0.f);
-  return small ? r : (b < 0 ? -m : m);
+  const float h = rintf(x * 0x1p-31f);
+  return (long long)__float2int_rn(h) * (1ll << 31) + __float2int_rn(fmaf(-h, 0x1p31f, x));
 }
-__device__ __forceinline__ long long ff_to_q(FF x) { return f2q(x.h * (float)kQScale) + f2q(x.l * (float)kQScale); }
 template <class Q, class W>
 __device__ __forceinline__ W q_to_wide(Q d);
 template <>
@@ -607,21 +702,29 @@ __device__ __forceinline__ void block_scan_fused(int n, W *wtot, In &&in, Out &&
       tot = wide_add(tot, v[j]);
     }
   }
+  const bool on = warp * 32 * E < n;  // a warp past the data takes the barriers only
   W incl = tot;
+  if (on) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const W t = wide_shfl_up(incl, o);
-    if (lane >= o) incl = wide_add(incl, t);
+    for (int o = 1; o < 32; o <<= 1) {
+      const W t = wide_shfl_up(incl, o);
+      if (lane >= o) incl = wide_add(incl, t);
+    }
+    if (lane == 31) wtot[warp] = incl;
   }
-  if (lane == 31) wtot[warp] = incl;
   __syncthreads();
-  // this warp's offset: the sum of the totals of the warps before it
-  W t = lane < warp ? wtot[lane] : wide_zero<W>();
+  W run = wide_zero<W>();
+  if (on) {
+    // this warp's offset: the sum of the totals of the warps before it
+    if (warp > 0) {
+      W t = lane < warp ? wtot[lane] : wide_zero<W>();
 #pragma unroll
-  for (int o = 1; o < NW; o <<= 1) t = wide_add(t, wide_shfl_down(t, o));
-  W run = wide_shfl_idx(t, 0);
-  const W below = wide_shfl_up(incl, 1);
-  if (lane > 0) run = wide_add(run, below);
+      for (int o = 1; o < NW; o <<= 1) t = wide_add(t, wide_shfl_down(t, o));
+      run = wide_shfl_idx(t, 0);
+    }
+    const W below = wide_shfl_up(incl, 1);
+    if (lane > 0) run = wide_add(run, below);
+  }
 #pragma unroll
   for (int j = 0; j < EMAX; ++j) {
     const int q = beg + j;
@@ -728,23 +831,46 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
 // and give it the Cartesian momentum (ux, uy).  The new radius is formed as the exact
 // increment r' - r = (dx (2r + dx) + dy^2) / (r' + r), applied to the cell offset, so no
 // precision is lost to the size of r.  Returns the new cell (cn, fn), the radius rn, and the
-// radial / azimuthal momenta; a ring beyond the wall r = nr dr is reflected specularly.
+// radial / azimuthal momenta and the direction (ex, ey) of its new position in the frame; a ring
+// beyond the wall r = nr dr is reflected specularly.
 template <class R>
 __device__ __forceinline__ void move_ring(int c, R f, R r, R dx, R dy, R ux, R uy, R inv_dr, R dr, int nr,
-                                          int &cn, R &fn, R &rn, R &urn, R &utn) {
-  const R xn = r + dx, yn = dy;
-  const R rr = sqrt(xn * xn + yn * yn);
-  const R den = rr + r;
-  const R delta = den > (R)0 ? (dx * ((R)2 * r + dx) + dy * dy) / den : (R)0;
-  R s = f + delta * inv_dr;  // offset from node c, in cells
-  if (rr > (R)0) {
-    const R irr = (R)1 / rr;
-    urn = (xn * ux + yn * uy) * irr;
-    utn = (xn * uy - yn * ux) * irr;
+                                          int &cn, R &fn, R &rn, R &urn, R &utn, R &ex, R &ey) {
+  const R xn = r + dx, yn = dy, r2 = xn * xn + yn * yn;
+  R delta = (R)0;
+  ex = (R)1;  // the direction of the new position in the frame
+  ey = (R)0;
+  // the momentum by one division of the products, not through ex: x (1/x) falls short of 1 by a
+  // rounding, the same way every slice (the mixed linear march's error against 64 bits doubled)
+  if constexpr (sizeof(R) == 8) {
+    if (r2 > tiny_r2<R>()) {
+      R rr, irr;
+      root_of(r2, rr, irr);
+      delta = (dx * ((R)2 * r + dx) + dy * dy) * rcp_of(rr + r);
+      ex = xn * irr;
+      ey = yn * irr;
+      urn = (xn * ux + yn * uy) * irr;
+      utn = (xn * uy - yn * ux) * irr;
+    } else {
+      if (r > tiny_r<R>()) delta = (dx * ((R)2 * r + dx) + dy * dy) * rcp_of(r);
+      urn = sqrt(ux * ux + uy * uy);
+      utn = (R)0;
+    }
   } else {
-    urn = sqrt(ux * ux + uy * uy);
-    utn = (R)0;
+    const R rr = sqrt(r2), den = rr + r;
+    delta = den > (R)0 ? (dx * ((R)2 * r + dx) + dy * dy) / den : (R)0;
+    if (rr > (R)0) {
+      const R irr = (R)1 / rr;
+      ex = xn * irr;
+      ey = yn * irr;
+      urn = (xn * ux + yn * uy) * irr;
+      utn = (xn * uy - yn * ux) * irr;
+    } else {
+      urn = sqrt(ux * ux + uy * uy);
+      utn = (R)0;
+    }
   }
+  R s = f + delta * inv_dr;  // offset from node c, in cells
   if ((R)c + s > (R)nr) {  // specular reflection at the wall: r'/dr -> 2 nr - r'/dr
     s = (R)(2 * (nr - c)) - s;
     urn = -urn;
@@ -765,16 +891,21 @@ __device__ __forceinline__ void move_ring(int c, R f, R r, R dx, R dy, R ux, R u
   rn = ((R)ci + fo) * dr;
 }
 
-// Window of three cells c0..c0+2 (four nodes) summed in registers; a ring outside the
+// Cells of a thread's deposit window: a thread of one ring needs that ring's cell only, a thread
+// of two rarely more than two.  Every cell less is a node less to sum over the warp and to add:
+// 11, 17 or 23 sums per thread of a current pass.
+__host__ __device__ constexpr int win_cells(int ppt) { return ppt == 1 ? 1 : ppt == 2 ? 2 : 3; }
+
+// Window of three (or NC) cells c0..c0+2 (NC + 1 nodes) summed in registers; a ring outside the
 // window deposits directly.
-template <class R, int NV>
+template <class R, int NV, int NC>
 struct WindowAcc {
   int c0 = -1;
-  R n[4][NV];
+  R n[NC + 1][NV];
   __device__ __forceinline__ void init(int c) {
     c0 = c;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a <= NC; ++a)
 #pragma unroll
       for (int q = 0; q < NV; ++q) n[a][q] = (R)0;
   }
@@ -782,16 +913,13 @@ struct WindowAcc {
   // multiply-add per node and value
   __device__ __forceinline__ bool add(int c, R f, const R (&v)[NV]) {
     const int o = c - c0;
-    if (o < 0 || o > 2) return false;
+    if (o < 0 || o >= NC) return false;
     const R g = (R)1 - f;
-    const R w0 = o == 0 ? g : (R)0, w1 = o == 0 ? f : (o == 1 ? g : (R)0);
-    const R w2 = o == 1 ? f : (o == 2 ? g : (R)0), w3 = o == 2 ? f : (R)0;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      n[0][q] += v[q] * w0;
-      n[1][q] += v[q] * w1;
-      n[2][q] += v[q] * w2;
-      n[3][q] += v[q] * w3;
+    for (int a = 0; a <= NC; ++a) {
+      const R w = (a < NC && o == a) ? g : (a > 0 && o == a - 1 ? f : (R)0);
+#pragma unroll
+      for (int q = 0; q < NV; ++q) n[a][q] += v[q] * w;
     }
     return true;
   }
@@ -833,114 +961,85 @@ struct WarpSeg {
   }
 };
 
-// A ring's charge contributions to the node pair (c, c+1) in the form's charge-window type.
-template <class Pol>
-struct ChargeWin;
-template <>
-struct ChargeWin<PolFP64> {
-  int c0 = -1;
-  double n[4];
-  __device__ __forceinline__ void init(int c) {
-    c0 = c;
-    n[0] = n[1] = n[2] = n[3] = 0.0;
-  }
-  __device__ __forceinline__ bool add(int c, double f, double w) {
-    const int o = c - c0;
-    if (o < 0 || o > 2) return false;
-    const double lo = w * (1.0 - f), hi = w * f;
-    n[0] += o == 0 ? lo : 0.0;
-    n[1] += o == 0 ? hi : (o == 1 ? lo : 0.0);
-    n[2] += o == 1 ? hi : (o == 2 ? lo : 0.0);
-    n[3] += o == 2 ? hi : 0.0;
-    return true;
-  }
-  __device__ __forceinline__ static void direct(double *rho, int c, double f, double w) {
-    atomicAdd(&rho[c], w * (1.0 - f));
-    atomicAdd(&rho[c + 1], w * f);
-  }
-  __device__ __forceinline__ double node(int a) const { return n[a]; }
-};
-template <>
-struct ChargeWin<PolMixed> {
-  int c0 = -1;
-  long long n[4];
-  __device__ __forceinline__ void init(int c) {
-    c0 = c;
-    n[0] = n[1] = n[2] = n[3] = 0;
-  }
-  // w f as an exact float-float product, w and w f in fixed point, w (1 - f) = w - w f there
-  __device__ __forceinline__ static void split(float f, float w, long long &qlo, long long &qhi) {
-    const FF hi = two_prod(w, f);
-    qhi = ff_to_q(hi);
-    qlo = f2q(w * (float)kQScale) - qhi;
-  }
-  __device__ __forceinline__ bool add(int c, float f, float w) {
-    const int o = c - c0;
-    if (o < 0 || o > 2) return false;
-    long long lo, hi;
-    split(f, w, lo, hi);
-    n[0] += o == 0 ? lo : 0ll;
-    n[1] += o == 0 ? hi : (o == 1 ? lo : 0ll);
-    n[2] += o == 1 ? hi : (o == 2 ? lo : 0ll);
-    n[3] += o == 2 ? hi : 0ll;
-    return true;
-  }
-  __device__ __forceinline__ static void direct(long long *rho, int c, float f, float w) {
-    long long lo, hi;
-    split(f, w, lo, hi);
-    atomicAdd((unsigned long long *)&rho[c], (unsigned long long)lo);
-    atomicAdd((unsigned long long *)&rho[c + 1], (unsigned long long)hi);
-  }
-  __device__ __forceinline__ long long node(int a) const { return n[a]; }
-};
-
-template <>
-struct ChargeWin<PolWide> : ChargeWin<PolMixed> {};
-template <>
-struct ChargeWin<PolMixed64> : ChargeWin<PolMixed> {};
-template <>
-struct ChargeWin<PolWideFP64> : ChargeWin<PolFP64> {};
-template <class P>
-struct ChargeWin<SlabOf<P>> : ChargeWin<P> {};
-
-
+// A ring's charge in the form's deposit type: its shares w (1 - f) and w f of the nodes c, c + 1.
+// FP64: doubles.  Mixed forms: w f as the exact float-float product (two-product by FMA) rounded
+// to the fixed-point grid, and w in fixed point minus it.
+__device__ __forceinline__ void charge_split(double f, double w, double &lo, double &hi) {
+  lo = w * (1.0 - f);
+  hi = w * f;
+}
+__device__ __forceinline__ void charge_split(float f, float w, long long &lo, long long &hi) {
+  const FF p = two_prod(w, f);
+  hi = f2q(p.h * (float)kQScale) + f2q(p.l * (float)kQScale);
+  lo = f2q(w * (float)kQScale) - hi;
+}
 __device__ __forceinline__ void q_atomic_add(double *p, double v) { atomicAdd(p, v); }
 __device__ __forceinline__ void q_atomic_add(long long *p, long long v) {
   atomicAdd((unsigned long long *)p, (unsigned long long)v);
 }
+// Charge deposit of one ring straight into rho (shared atomics).
+template <class Q, class R>
+__device__ __forceinline__ void charge_direct(Q *rho, int c, R f, R w) {
+  Q lo, hi;
+  charge_split(f, w, lo, hi);
+  q_atomic_add(&rho[c], lo);
+  q_atomic_add(&rho[c + 1], hi);
+}
+// The charge window: the rings' shares summed over NC cells (NC + 1 nodes) in registers.
+template <class Pol, int NC>
+struct ChargeWin {
+  using Q = typename Pol::Q;
+  using R = typename Pol::R;
+  int c0 = -1;
+  Q n[NC + 1];
+  __device__ __forceinline__ void init(int c) {
+    c0 = c;
+#pragma unroll
+    for (int a = 0; a <= NC; ++a) n[a] = (Q)0;
+  }
+  __device__ __forceinline__ bool add(int c, R f, R w) {
+    const int o = c - c0;
+    if (o < 0 || o >= NC) return false;
+    Q lo, hi;
+    charge_split(f, w, lo, hi);
+#pragma unroll
+    for (int a = 0; a <= NC; ++a) n[a] += (a < NC && o == a) ? lo : ((a > 0 && o == a - 1) ? hi : (Q)0);
+    return true;
+  }
+};
 
 // Flush a charge window into rho over the warp.  All lanes of the warp call it.
-template <class Pol>
-__device__ __forceinline__ void flush_charge(MarchSmem<Pol> &sm, const ChargeWin<Pol> &acc, int nr) {
+template <class Pol, int NC>
+__device__ __forceinline__ void flush_charge(MarchSmem<Pol> &sm, const ChargeWin<Pol, NC> &acc, int nr) {
   using Q = typename Pol::Q;
   const WarpSeg seg(acc.c0);
-  Q t[4];
+  Q t[NC + 1];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) t[a] = acc.node(a);
+  for (int a = 0; a <= NC; ++a) t[a] = acc.n[a];
   seg.sum_n(t);
 #pragma unroll
-  for (int a = 0; a < 4; ++a)  // a node no ring of the segment touched is not added to
+  for (int a = 0; a <= NC; ++a)  // a node no ring of the segment touched is not added to
     if (seg.is_tail && acc.c0 >= 0 && acc.c0 + a <= nr && t[a] != (Q)0) q_atomic_add(&sm.rho[acc.c0 + a], t[a]);
 }
 
 // Charge deposit of one ring through a window (direct atomics outside it).
-template <class Pol>
-__device__ __forceinline__ void add_charge(MarchSmem<Pol> &sm, ChargeWin<Pol> &acc, int p, int c,
+template <class Pol, int NC>
+__device__ __forceinline__ void add_charge(MarchSmem<Pol> &sm, ChargeWin<Pol, NC> &acc, int p, int c,
                                            typename Pol::R f, typename Pol::R w) {
   if (p == 0) acc.init(c);
-  if (!acc.add(c, f, w)) ChargeWin<Pol>::direct(sm.rho, c, f, w);
+  if (!acc.add(c, f, w)) charge_direct(sm.rho, c, f, w);
 }
 // Charge deposit of ring p through the window; a ring outside it is marked in miss (bit p) and
 // left to warp_misses.
-template <class Pol>
-__device__ __forceinline__ void add_charge_mark(MarchSmem<Pol> &sm, ChargeWin<Pol> &acc, int p, int c,
+template <class Pol, int NC>
+__device__ __forceinline__ void add_charge_mark(MarchSmem<Pol> &sm, ChargeWin<Pol, NC> &acc, int p, int c,
                                                 typename Pol::R f, typename Pol::R w, unsigned &miss) {
   if (p == 0) acc.init(c);
   if (!acc.add(c, f, w)) {
     if constexpr (Pol::kDeferMisses)
       miss |= 1u << p;
     else
-      ChargeWin<Pol>::direct(sm.rho, c, f, w);  // the policy deposits in the loop
+      charge_direct(sm.rho, c, f, w);  // the policy deposits in the loop
   }
 }
 
@@ -1033,8 +1132,9 @@ __device__ __forceinline__ void drain_queue(MarchSmem<Pol> &sm, int n1, Fn &&fn)
 }
 
 // One ring's current-type deposit values (the source terms of Eqs. 4-7: J_z, chi, T, P, U and
-// the K share), its Gamma and (gamma/Gamma) psi', at cell c, offset f, momenta (u_r, u_theta).
-template <class Pol>
+// the K share), its Gamma and (gamma/Gamma) psi', at cell c, offset f, momenta (u_r, u_theta);
+// kFromL: u_theta is formed here, l_z / r, from the reciprocal of r that the centrifugal term needs.
+template <bool kFromL, class Pol>
 __device__ __forceinline__ void current_values(const MarchSmem<Pol> &sm, const RingSoA<typename Pol::R> &rs, int sl,
                                                int c, typename Pol::R f, typename Pol::R u_r, typename Pol::R u_t,
                                                typename Pol::R dr, int *status, typename Pol::R (&v)[5],
@@ -1044,13 +1144,22 @@ __device__ __forceinline__ void current_values(const MarchSmem<Pol> &sm, const R
   const R rp = ((R)c + f) * dr;
   G = rs.G0[sl] + interp(sm.psi, c, f);
   if (!(G > (R)0)) flag(status, ST_NUMERIC);
-  const R iG = (R)1 / G;
+  R iG, ir = (R)0;
+  if (slab) {
+    iG = rcp_of(G);
+    if (kFromL) u_t = rs.lz[sl];
+  } else {
+    const bool off = rp > tiny_r<R>();
+    rcp_pair(G, off ? rp : (R)1, iG, ir);
+    ir = off ? ir : (R)0;
+    if (kFromL) u_t = rs.lz[sl] * ir;
+  }
   const R up2 = u_r * u_r + u_t * u_t;
   const R gam = ((R)1 + up2 + G * G) * (R)0.5 * iG;
   const R uz = gam - G;
   const R a = u_r * iG;
   const R dp = interp(sm.dpsi, c, f);
-  const R cent = (!slab && rp > (R)0) ? u_t * u_t * iG / rp : (R)0;  // Eq. 4's centrifugal term (cylinder)
+  const R cent = slab ? (R)0 : u_t * u_t * iG * ir;  // Eq. 4's centrifugal term (cylinder)
   g = gam * iG * dp;
   const R w = rs.w[sl];
   v[0] = -w * uz * iG;
@@ -1078,14 +1187,14 @@ __device__ __forceinline__ void current_direct(MarchSmem<Pol> &sm, int c, typena
 
 // A ring outside the window, at slot sl, through the position functor pos_slot: its values
 // formed again by the same arithmetic and deposited straight into the node arrays.
-template <class Pol, class PosSlot>
+template <bool kFromL, class Pol, class PosSlot>
 __device__ __forceinline__ void current_miss(MarchSmem<Pol> &sm, const RingSoA<typename Pol::R> &rs, int sl,
                                              typename Pol::R dr, int *status, PosSlot &&pos_slot) {
   using R = typename Pol::R;
   int c;
   R f, u_r, u_t, v[5], ka, G, g;
   pos_slot(sl, c, f, u_r, u_t);
-  current_values<Pol>(sm, rs, sl, c, f, u_r, u_t, dr, status, v, ka, G, g);
+  current_values<kFromL, Pol>(sm, rs, sl, c, f, u_r, u_t, dr, status, v, ka, G, g);
   current_direct<Pol>(sm, c, f, v, ka);
 }
 
@@ -1094,16 +1203,19 @@ __device__ __forceinline__ void current_miss(MarchSmem<Pol> &sm, const RingSoA<t
 // A ring outside the thread's window is only marked in the loop (an atomic there would order
 // every later ring's loads behind it); on_miss(mask) receives the thread's marks after the loop
 // (all lanes call it) and sees to those rings' deposits (current_miss).
-template <class Pol, int NT, int PPT, bool kTrap = false, class Pos, class OnMiss>
+template <bool kFromL, class Pol, int NT, int PPT, bool kTrap = false, class Pos, class OnMiss>
 __device__ __forceinline__ void pass_currents(MarchSmem<Pol> &sm, const RingSoA<typename Pol::R> &rs, int np,
                                               int nr, typename Pol::R dr, int *status, Pos &&pos, OnMiss &&on_miss,
                                               typename Pol::R (&Gam)[PPT], typename Pol::R (&gq)[PPT]) {
   using R = typename Pol::R;
   using Acc = typename Pol::Acc;
   const int t = threadIdx.x;
-  WindowAcc<R, 5> acc;
+  constexpr int NC = win_cells(PPT);
+  WindowAcc<R, 5, NC> acc;
   acc.init(-8);
-  R kw[3] = {(R)0, (R)0, (R)0};
+  R kw[NC];
+#pragma unroll
+  for (int a = 0; a < NC; ++a) kw[a] = (R)0;
   unsigned miss = 0u;
 #pragma unroll
   for (int p = 0; p < PPT; ++p) {
@@ -1121,12 +1233,11 @@ __device__ __forceinline__ void pass_currents(MarchSmem<Pol> &sm, const RingSoA<
       if constexpr (kTrap)
         if (rs.w[sl] == (R)0) continue;  // promoted to a beam particle: no longer in the plasma
       R v[5], ka, G, g;
-      current_values<Pol>(sm, rs, sl, c, f, u_r, u_t, dr, status, v, ka, G, g);
+      current_values<kFromL, Pol>(sm, rs, sl, c, f, u_r, u_t, dr, status, v, ka, G, g);
       if (acc.add(c, f, v)) {
         const int o = c - acc.c0;
-        kw[0] += o == 0 ? ka : (R)0;
-        kw[1] += o == 1 ? ka : (R)0;
-        kw[2] += o == 2 ? ka : (R)0;
+#pragma unroll
+        for (int a = 0; a < NC; ++a) kw[a] += o == a ? ka : (R)0;
       } else if constexpr (Pol::kDeferMisses) {
         miss |= 1u << p;
       } else {
@@ -1140,13 +1251,13 @@ __device__ __forceinline__ void pass_currents(MarchSmem<Pol> &sm, const RingSoA<
   const WarpSeg seg(acc.c0);
   const int c = acc.c0;
   const bool emit = seg.is_tail && c >= 0;
-  Acc tot[23];  // the thread's window sums, then summed across rings in the deposit type
+  Acc tot[6 * NC + 5];  // the thread's window sums, then summed across rings in the deposit type
 #pragma unroll
   for (int q = 0; q < 5; ++q)
 #pragma unroll
-    for (int a = 0; a < 4; ++a) tot[q * 4 + a] = (Acc)acc.n[a][q];
+    for (int a = 0; a <= NC; ++a) tot[q * (NC + 1) + a] = (Acc)acc.n[a][q];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) tot[20 + a] = (Acc)kw[a];
+  for (int a = 0; a < NC; ++a) tot[5 * (NC + 1) + a] = (Acc)kw[a];
   seg.sum_n(tot);
   // The window's last nodes are often untouched (a thread's rings span one or two cells where
   // the plasma is dense), and the shared-memory adds are the pass's costliest part: zero sums
@@ -1155,11 +1266,15 @@ __device__ __forceinline__ void pass_currents(MarchSmem<Pol> &sm, const RingSoA<
 #pragma unroll
   for (int q = 0; q < 5; ++q)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-      if (emit && c + a <= nr && tot[q * 4 + a] != (Acc)0) atomicAdd(&arr[q][c + a], (Acc)tot[q * 4 + a]);
+    for (int a = 0; a <= NC; ++a) {
+      const Acc v = tot[q * (NC + 1) + a];
+      if (emit && c + a <= nr && v != (Acc)0) atomicAdd(&arr[q][c + a], v);
+    }
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    if (emit && c + a < nr && tot[20 + a] != (Acc)0) atomicAdd(&sm.K[c + a], (Acc)tot[20 + a]);
+  for (int a = 0; a < NC; ++a) {
+    const Acc v = tot[5 * (NC + 1) + a];
+    if (emit && c + a < nr && v != (Acc)0) atomicAdd(&sm.K[c + a], v);
+  }
 }
 
 // Re-sort the rings of the CTA by cell (counting sort) so that each thread's rings are
@@ -1275,6 +1390,13 @@ __device__ __forceinline__ void resort_rings(MarchSmem<Pol> &sm, const RingSoA<t
 //   R    nb_row(int row, int m)     beam density at node m of a row
 //   void slice_done(int k, sm)      stage-1 fields of slice k are in sm (psi, dpsi, ez, bth)
 //   void finish(sm)                 after the last slice
+//   kCluster                        (true) the march is shared by the CTAs of a cluster, each
+//                                   calling this with the same descriptor; wait_row may then give up
+//                                   in one CTA alone, and given_up(row), called by all after a
+//                                   cluster barrier that follows wait_row(row), gives the answer for
+//                                   the cluster; between_pushes() is called between two slice_done
+//                                   where every CTA has returned from the first and none has
+//                                   entered the second
 //   kTraj, ring_state<NT, PPT>(k, rs, np)
 //                                   (kTraj true only) the slice-k state of the thread's own
 //                                   rings, with their stage-1 Gamma in rs.G1; the slots carry
@@ -1288,17 +1410,34 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
   using R = typename Pol::R;
   using G = typename Pol::G;
   using Acc = typename Pol::Acc;
-  const int tid = threadIdx.x, nr = d.nr, n1 = nr + 1, np = d.np, nxi = d.nxi;
   constexpr int SLOTS = NT * PPT;
   constexpr bool kTrap = Hooks::kTrap;
   constexpr bool kIds = Hooks::kTraj || kTrap;
+  constexpr bool kCl = Hooks::kCluster;
+  // the CTA's rings j0 .. j0 + np - 1: all, or its share of them (consecutive in radius at first)
+  const int cn = kCl ? cl_size() : 1, cr = kCl ? cl_rank() : 0;
+  const int share = kCl ? (d.np + cn - 1) / cn : d.np, j0 = cr * share;
+  const int tid = threadIdx.x, nr = d.nr, n1 = nr + 1, np = kCl ? max(0, min(share, d.np - j0)) : d.np, nxi = d.nxi;
   MarchSmem<Pol> sm;
   sm.carve(smem_raw, n1, SLOTS, kIds);
   RingSoA<R> rs;
   if (Pol::kSmemRings)
     rs = sm.rings;
   else
-    rs.carve(d.ring_buf, SLOTS, kIds);
+    rs.carve((unsigned char *)d.ring_buf + (kCl ? (size_t)cr * RingSoA<R>::bytes(SLOTS, kIds) : 0), SLOTS, kIds);
+  // the end of a deposit pass: a barrier, and the cluster's sums in every CTA's arrays
+  auto sum_charge = [&]() {
+    if constexpr (kCl)
+      cluster_sum<NT>(sm.rho, n1, cn, cr);
+    else
+      __syncthreads();
+  };
+  auto sum_currents = [&]() {  // after the pass's own barrier; jz, chi, T, P, U, K are contiguous
+    if constexpr (kCl) {
+      using V = std::conditional_t<sizeof(Acc) == 4, float2, double>;
+      cluster_sum<NT>((V *)sm.jz, (int)(6 * n1 * sizeof(Acc) / sizeof(V)), cn, cr);
+    }
+  };
   const double drd = d.dr;
   const R h = (R)d.dxi, R_wall = (R)d.rmax, dR = (R)drd, inv_dr = (R)(1.0 / drd);
   using N = typename Pol::N;
@@ -1320,8 +1459,8 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
   // position resolution is uniform over the box; moves are exact radial displacements.
 #pragma unroll
   for (int p = 0; p < PPT; ++p) {
-    const int j = tid * PPT + p, sl = p * NT + tid;
-    if (j < np) {
+    const int jl = tid * PPT + p, sl = p * NT + tid, j = j0 + jl;
+    if (jl < np) {
       const double s = d.r0[j] / drd;
       int c = (int)floor(s);
       c = c < 0 ? 0 : (c > nr - 1 ? nr - 1 : c);
@@ -1343,48 +1482,61 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
   // u_theta = l_z / r; in the slab, lz holds the conserved u_y, which enters gamma only and
   // moves nothing (d/dy = 0): the Cartesian frame below is then the x line, and r = |x| puts a
   // sheet that crosses x = 0 in place of its mirror image
-  auto state_pos = [&](int sl, int &c, R &f, R &u_r, R &u_t) {
+  auto state_pos = [&](int sl, int &c, R &f, R &u_r, R &) {  // u_theta: current_values<true>
     c = rs.c[sl];
     f = rs.f[sl];
     u_r = rs.ur[sl];
-    const R r = ((R)c + f) * dR;
-    u_t = slab ? rs.lz[sl] : (r > (R)0 ? rs.lz[sl] / r : (R)0);
   };
-  auto midpoint = [&](int sl, int &c, R &f, R &u_r, R &u_t) -> R {
+  // 1/Gamma of stage 1 and the frame's y momentum of the slice's state
+  auto frame_of = [&](int sl, R r, R &iG, R &ut) {
+    if (slab) {
+      iG = rcp_of(rs.G1[sl]);
+      ut = (R)0;
+    } else {
+      const bool off = r > tiny_r<R>();
+      R ir;
+      rcp_pair(rs.G1[sl], off ? r : (R)1, iG, ir);
+      ut = off ? rs.lz[sl] * ir : (R)0;
+    }
+  };
+  auto midpoint = [&](int sl, int &c, R &f, R &u_r, R &u_t, R &ex, R &ey) -> R {
     const int c0 = rs.c[sl];
     const R f0 = rs.f[sl], ur0 = rs.ur[sl];
     const R r = ((R)c0 + f0) * dR;
-    const R ut = slab ? (R)0 : (r > (R)0 ? rs.lz[sl] / r : (R)0);  // the frame's y momentum
-    const R iG = (R)1 / rs.G1[sl];
+    R iG, ut;
+    frame_of(sl, r, iG, ut);
     const R dx = (R)0.5 * h * ur0 * iG, dy = (R)0.5 * h * ut * iG;
     const R uxh = ur0 + (R)0.5 * h * rs.F1[sl];
     R rr;
-    move_ring<R>(c0, f0, r, dx, dy, uxh, ut, inv_dr, dR, nr, c, f, rr, u_r, u_t);
+    move_ring<R>(c0, f0, r, dx, dy, uxh, ut, inv_dr, dR, nr, c, f, rr, u_r, u_t, ex, ey);
     if (slab) u_t = rs.lz[sl];
     return rr;
   };
-  auto mid_slot = [&](int sl, int &c, R &f, R &u_r, R &u_t) { midpoint(sl, c, f, u_r, u_t); };
+  auto mid_slot = [&](int sl, int &c, R &f, R &u_r, R &u_t) {
+    R ex, ey;
+    midpoint(sl, c, f, u_r, u_t, ex, ey);
+  };
   // out-of-window rings: those of the current passes queued and drained by the CTA after the
   // pass, those of the charge passes (two atomics each) deposited by their own warp
-  auto cur_miss1 = [&](int sl) { current_miss<Pol>(sm, rs, sl, dR, d.status, state_pos); };
-  auto cur_miss2 = [&](int sl) { current_miss<Pol>(sm, rs, sl, dR, d.status, mid_slot); };
+  auto cur_miss1 = [&](int sl) { current_miss<true, Pol>(sm, rs, sl, dR, d.status, state_pos); };
+  auto cur_miss2 = [&](int sl) { current_miss<false, Pol>(sm, rs, sl, dR, d.status, mid_slot); };
   auto chg_miss_mid = [&](int sl) {
     const R w = rs.w[sl];
     if (kTrap && w == (R)0) return;  // a promoted ring deposits nothing
     int c;
     R f, u_r, u_t;
-    midpoint(sl, c, f, u_r, u_t);
-    ChargeWin<Pol>::direct(sm.rho, c, f, w);
+    mid_slot(sl, c, f, u_r, u_t);
+    charge_direct(sm.rho, c, f, w);
   };
   auto chg_miss_full = [&](int sl) {  // the new positions are in the slots
     const R w = rs.w[sl];
-    if (w != (R)0) ChargeWin<Pol>::direct(sm.rho, rs.c[sl], rs.f[sl], w);
+    if (w != (R)0) charge_direct(sm.rho, rs.c[sl], rs.f[sl], w);
   };
 
   // charge of the initial slice; it is also the ion background (the deposit of the
   // unperturbed electrons), so psi starts exactly at zero
   {
-    ChargeWin<Pol> acc;
+    ChargeWin<Pol, win_cells(PPT)> acc;
     acc.init(-8);
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
@@ -1394,7 +1546,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
       }
     flush_charge<Pol>(sm, acc, nr);
   }
-  __syncthreads();
+  sum_charge();
   for (int m = tid; m < n1; m += NT) sm.rho0[m] = sm.rho[m];
   __syncthreads();
 
@@ -1411,7 +1563,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
     {
       R Gs[PPT], gqs[PPT];
-      pass_currents<Pol, NT, PPT, kTrap>(
+      pass_currents<true, Pol, NT, PPT, kTrap>(
           sm, rs, np, nr, dR, d.status, state_pos,
           [&](unsigned miss) { queue_misses<NT, PPT>(sm, n1, miss, cur_miss1); }, Gs, gqs);
 #pragma unroll
@@ -1424,22 +1576,25 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     }
     __syncthreads();
     drain_queue<NT>(sm, n1, cur_miss1);
+    sum_currents();
     if constexpr (kTrap) hk.template trap_rings<NT, PPT>(k, rs, np);  // after every stage-1 deposit
     solve_fields<Pol, NT>(sm, geo, nbk, nbk, sm.wtot);  // P2
     // P3: fields of slice k, then the move to the midpoint and its charge deposit
     hk.slice_done(k, sm);
     if (k == nxi) break;
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
-    // the midpoint of each ring, kept in registers for stage 2 and the full step
+    // the midpoint of each ring, kept in registers for stage 2 and the full step (its direction too
+    // where a thread has few rings; more would spill)
+    constexpr bool kKeepDir = PPT <= 2;
     int MC[PPT];
-    R MF[PPT], MUR[PPT], MUT[PPT];
+    R MF[PPT], MUR[PPT], MUT[PPT], MEX[kKeepDir ? PPT : 1], MEY[kKeepDir ? PPT : 1];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
       MC[p] = 0;
       MF[p] = MUR[p] = MUT[p] = (R)0;
     }
     {
-      ChargeWin<Pol> acc;
+      ChargeWin<Pol, win_cells(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -1448,13 +1603,17 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
           const int sl = p * NT + tid;
           rs.F1[sl] = rs.F1[sl] - interp(sm.bth, rs.c[sl], rs.f[sl]);
           int c;
-          R f, u_r, u_t;
+          R f, u_r, u_t = (R)0, ex = (R)1, ey = (R)0;
           R rr;
           if (kTrap && rs.w[sl] == (R)0) {  // a promoted ring stays where it is
             state_pos(sl, c, f, u_r, u_t);
             rr = ((R)c + f) * dR;
           } else {
-            rr = midpoint(sl, c, f, u_r, u_t);
+            rr = midpoint(sl, c, f, u_r, u_t, ex, ey);
+          }
+          if constexpr (kKeepDir) {
+            MEX[p] = ex;
+            MEY[p] = ey;
           }
           if (!(rr >= (R)0 && rr <= R_wall)) flag(d.status, ST_ESCAPE);
           MC[p] = c;
@@ -1467,25 +1626,25 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
       warp_misses<NT, PPT>(miss, chg_miss_mid);
       flush_charge<Pol>(sm, acc, nr);
     }
-    __syncthreads();
+    sum_charge();
+    if constexpr (kCl) hk.between_pushes();
     // ======== stage 2 at xi_k + dxi/2 ========
-    // beam-density row k+1, first read by this stage: fetched here, stored in P1 (n1 <= 3 NT).
+    // beam-density row k+1, first read by this stage: fetched here, stored in P1.
     // (Waiting for it only here, not at the start of the slice, lets a pipelined step follow the
     // step before it by two slices and two pushes instead of two and a half and three.)
     if (!hk.wait_row(k + 1)) break;
-    R pre[3] = {(R)0, (R)0, (R)0};
+    R pre[Pol::kScanE];
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
-      if (tid + q * NT < n1) pre[q] = hk.nb_row(k + 1, tid + q * NT);
+    for (int q = 0; q < Pol::kScanE; ++q) pre[q] = tid + q * NT < n1 ? hk.nb_row(k + 1, tid + q * NT) : (R)0;
     solve_psi<Pol, NT>(sm, geo, sm.wtot);  // P0
     {  // P1
       R *dst = (k & 1) ? sm.nb0 : sm.nb1;
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
+      for (int q = 0; q < Pol::kScanE; ++q)
         if (tid + q * NT < n1) dst[tid + q * NT] = pre[q];
     }
     for (int i = tid; i < n1; i += NT) sm.rho[i] = (typename Pol::Q)0;
-    pass_currents<Pol, NT, PPT, kTrap>(sm, rs, np, nr, dR, d.status,
+    pass_currents<false, Pol, NT, PPT, kTrap>(sm, rs, np, nr, dR, d.status,
                                 [&](int p, int, int &c, R &f, R &u_r, R &u_t) {
                                   c = MC[p];
                                   f = MF[p];
@@ -1495,12 +1654,15 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
                                 [&](unsigned miss) { queue_misses<NT, PPT>(sm, n1, miss, cur_miss2); }, G2, F2);
     __syncthreads();
     drain_queue<NT>(sm, n1, cur_miss2);
+    sum_currents();
+    if constexpr (kCl)
+      if (hk.given_up(k + 1)) break;  // the same answer in every CTA of the cluster
     solve_fields<Pol, NT>(sm, geo, nbk, nbk1, sm.wtot);  // P2
     // P3: full step from the slice-k state with the midpoint derivative, and the charge
     // deposit of the new slice
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     {
-      ChargeWin<Pol> acc;
+      ChargeWin<Pol, win_cells(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -1513,26 +1675,29 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
           }
           const R F2b = F2[p] - interp(sm.bth, MC[p], MF[p]);  // at the midpoint
           const int c0 = rs.c[sl];
-          const R f0 = rs.f[sl], ur0 = rs.ur[sl], G1v = rs.G1[sl], F1v = rs.F1[sl];
+          const R f0 = rs.f[sl], ur0 = rs.ur[sl], F1v = rs.F1[sl];
           const R r = ((R)c0 + f0) * dR;
-          const R ut = slab ? (R)0 : (r > (R)0 ? rs.lz[sl] / r : (R)0);  // the frame's y momentum
-          const R iG1 = (R)1 / G1v;
-          const R xh = r + (R)0.5 * h * ur0 * iG1;
-          const R yh = (R)0.5 * h * ut * iG1;
+          R iG1, ut, ex = (R)1, ey = (R)0;
+          frame_of(sl, r, iG1, ut);
           const R uxh = ur0 + (R)0.5 * h * F1v;
-          const R rh = sqrt(xh * xh + yh * yh);
-          R ex = (R)1, ey = (R)0;
-          if (rh > (R)0) {
-            const R irh = (R)1 / rh;
-            ex = xh * irh;
-            ey = yh * irh;
+          if constexpr (kKeepDir) {
+            ex = MEX[p];
+            ey = MEY[p];
+          } else {
+            const R xh = r + (R)0.5 * h * ur0 * iG1, yh = (R)0.5 * h * ut * iG1, h2 = xh * xh + yh * yh;
+            if (h2 > tiny_r2<R>()) {
+              R rh, irh;
+              root_of(h2, rh, irh);
+              ex = xh * irh;
+              ey = yh * irh;
+            }
           }
-          const R iG2 = (R)1 / G2[p];
+          const R iG2 = rcp_of(G2[p]);
           const R dx = h * uxh * iG2, dy = h * ut * iG2;
           const R uxn = ur0 + h * F2b * ex, uyn = ut + h * F2b * ey;
           int cn;
-          R fn, rn, urn, utn;
-          move_ring<R>(c0, f0, r, dx, dy, uxn, uyn, inv_dr, dR, nr, cn, fn, rn, urn, utn);
+          R fn, rn, urn, utn, nx, ny;
+          move_ring<R>(c0, f0, r, dx, dy, uxn, uyn, inv_dr, dR, nr, cn, fn, rn, urn, utn, nx, ny);
           if (!(rn >= (R)0 && rn <= R_wall) || !isfinite(urn)) flag(d.status, ST_ESCAPE);
           rs.c[sl] = cn;
           rs.f[sl] = fn;
@@ -1543,18 +1708,21 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
       warp_misses<NT, PPT>(miss, chg_miss_full);
       flush_charge<Pol>(sm, acc, nr);
     }
-    __syncthreads();
+    sum_charge();
   }
   hk.finish(sm);
+  if constexpr (kCl) cl_barrier();  // no CTA leaves while another may still read its arrays
 }
 
-// Plain march: beam density from the simulation's grid, fields to its output grids.
-template <class Pol, int NT>
+// Plain march: beam density from the simulation's grid, fields to its output grids (in a
+// cluster, every CTA writes its share of the nodes).
+template <class Pol, int NT, bool kCl = false>
 struct PlainHooks {
   using R = typename Pol::R;
   using G = typename Pol::G;
   static constexpr bool kTraj = false;
   static constexpr bool kTrap = false;
+  static constexpr bool kCluster = kCl;
   const G *nb;
   G *opsi, *oez, *oer, *obth;
   int n1;
@@ -1564,7 +1732,8 @@ struct PlainHooks {
   __device__ __forceinline__ void slice_done(int k, MarchSmem<Pol> &sm) {
     if (!opsi) return;  // a timing probe of the tile autotuner keeps no output
     G *o1 = opsi + (size_t)k * n1, *o2 = oez + (size_t)k * n1, *o3 = oer + (size_t)k * n1, *o4 = obth + (size_t)k * n1;
-    for (int m = threadIdx.x; m < n1; m += NT) {
+    const int m0 = kCl ? cl_rank() * NT + threadIdx.x : threadIdx.x, dm = kCl ? cl_size() * NT : NT;
+    for (int m = m0; m < n1; m += dm) {
       const R ps = sm.psi[m], e = sm.ez[m], b = sm.bth[m];
       if (!(isfinite(ps) && isfinite(e) && isfinite(b))) flag(status, ST_NUMERIC);
       o1[m] = (G)ps;
@@ -1574,7 +1743,20 @@ struct PlainHooks {
     }
   }
   __device__ __forceinline__ void finish(MarchSmem<Pol> &) {}
+  __device__ __forceinline__ void between_pushes() {}
+  __device__ __forceinline__ bool given_up(int) { return false; }
 };
+
+// One cluster per simulation.
+template <class Pol, int NT, int PPT>
+__global__ void __launch_bounds__(NT, 1) march_cluster_kernel(const SimDesc *descs, const int *order) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i = blockIdx.x / cl_size();
+  const SimDesc &d = descs[order ? order[i] : i];
+  PlainHooks<Pol, NT, true> hk{(const typename Pol::G *)d.nb, (typename Pol::G *)d.psi, (typename Pol::G *)d.ez,
+                               (typename Pol::G *)d.er, (typename Pol::G *)d.bth, d.nr + 1, d.status};
+  march_body<Pol, NT, PPT>(d, smem_raw, hk);
+}
 
 // One CTA per simulation.  Tiles of fewer threads ask for more CTAs per SM, within the
 // same 128 registers per thread.

@@ -159,24 +159,29 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
   __syncthreads();
 
   int base = 0;  // slot offset of the chunk the position functors below read
-  auto state_pos = [&](int sl, int &c, R &f, R &u_r, R &u_t) {
+  auto state_pos = [&](int sl, int &c, R &f, R &u_r, R &) {
     sl += base;
     c = rs.c[sl];
     f = rs.f[sl];
-    u_r = rs.ur[sl];
-    const R r = ((R)c + f) * dR;
-    u_t = r > (R)0 ? rs.lz[sl] / r : (R)0;
+    u_r = rs.ur[sl];  // u_theta: current_values<true>
+  };
+  // 1/Gamma of stage 1 and u_theta of the slice's state
+  auto frame_of = [&](int sl, R r, R &iG, R &ut) {
+    const bool off = r > tiny_r<R>();
+    R ir;
+    rcp_pair(rs.G1[sl], off ? r : (R)1, iG, ir);
+    ut = off ? rs.lz[sl] * ir : (R)0;
   };
   auto midpoint_abs = [&](int sl, int &c, R &f, R &u_r, R &u_t) -> R {
     const int c0 = rs.c[sl];
     const R f0 = rs.f[sl], ur0 = rs.ur[sl];
     const R r = ((R)c0 + f0) * dR;
-    const R ut = r > (R)0 ? rs.lz[sl] / r : (R)0;
-    const R iG = (R)1 / rs.G1[sl];
+    R iG, ut, ex, ey;
+    frame_of(sl, r, iG, ut);
     const R dx = (R)0.5 * h * ur0 * iG, dy = (R)0.5 * h * ut * iG;
     const R uxh = ur0 + (R)0.5 * h * rs.F1[sl];
     R rr;
-    move_ring<R>(c0, f0, r, dx, dy, uxh, ut, inv_dr, dR, nr, c, f, rr, u_r, u_t);
+    move_ring<R>(c0, f0, r, dx, dy, uxh, ut, inv_dr, dR, nr, c, f, rr, u_r, u_t, ex, ey);
     return rr;
   };
   auto chunk_np = [&](int ch) { return np - ch * SLOTS < SLOTS ? np - ch * SLOTS : SLOTS; };
@@ -184,7 +189,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
   // charge of the initial slice = the ion background
   for (int ch = 0; ch < nch; ++ch) {
     const int b0 = ch * SLOTS, npc = chunk_np(ch);
-    ChargeWin<Pol> acc;
+    ChargeWin<Pol, win_cells(PPT)> acc;
     acc.init(-8);
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
@@ -213,8 +218,8 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
       const int npc = chunk_np(ch);
       R Gs[PPT], gqs[PPT];
       const RingSoA<R> rsc = shifted(rs, base);
-      pass_currents<Pol, NT, PPT>(sm, rsc, npc, nr, dR, d.status, state_pos, [&](unsigned miss) {
-        warp_misses<NT, PPT>(miss, [&](int sl) { current_miss<Pol>(sm, rsc, sl, dR, d.status, state_pos); });
+      pass_currents<true, Pol, NT, PPT>(sm, rsc, npc, nr, dR, d.status, state_pos, [&](unsigned miss) {
+        warp_misses<NT, PPT>(miss, [&](int sl) { current_miss<true, Pol>(sm, rsc, sl, dR, d.status, state_pos); });
       }, Gs, gqs);
 #pragma unroll
       for (int p = 0; p < PPT; ++p)
@@ -230,7 +235,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     for (int ch = 0; ch < nch; ++ch) {
       const int b0 = ch * SLOTS, npc = chunk_np(ch);
-      ChargeWin<Pol> acc;
+      ChargeWin<Pol, win_cells(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -249,7 +254,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
         int c;
         R f, u_r, u_t;
         midpoint_abs(b0 + sl, c, f, u_r, u_t);
-        ChargeWin<Pol>::direct(sm.rho, c, f, rs.w[b0 + sl]);
+        charge_direct(sm.rho, c, f, rs.w[b0 + sl]);
       });
       flush_charge<Pol>(sm, acc, nr);
     }
@@ -276,8 +281,8 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
       R Gs[PPT], gqs[PPT];
       auto mid_chunk = [&](int sl, int &c, R &f, R &u_r, R &u_t) { midpoint_abs(sl + base, c, f, u_r, u_t); };
       const RingSoA<R> rsc = shifted(rs, base);
-      pass_currents<Pol, NT, PPT>(sm, rsc, npc, nr, dR, d.status, mid_chunk, [&](unsigned miss) {
-        warp_misses<NT, PPT>(miss, [&](int sl) { current_miss<Pol>(sm, rsc, sl, dR, d.status, mid_chunk); });
+      pass_currents<false, Pol, NT, PPT>(sm, rsc, npc, nr, dR, d.status, mid_chunk, [&](unsigned miss) {
+        warp_misses<NT, PPT>(miss, [&](int sl) { current_miss<false, Pol>(sm, rsc, sl, dR, d.status, mid_chunk); });
       }, Gs, gqs);
 #pragma unroll
       for (int p = 0; p < PPT; ++p)
@@ -292,7 +297,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     for (int ch = 0; ch < nch; ++ch) {
       const int b0 = ch * SLOTS, npc = chunk_np(ch);
-      ChargeWin<Pol> acc;
+      ChargeWin<Pol, win_cells(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -304,26 +309,24 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
           midpoint_abs(sl, mc, mf, mu_r, mu_t);
           const R F2b = wr.F2[sl] - interp(sm.bth, mc, mf);
           const int c0 = rs.c[sl];
-          const R f0 = rs.f[sl], ur0 = rs.ur[sl], G1v = rs.G1[sl], F1v = rs.F1[sl];
+          const R f0 = rs.f[sl], ur0 = rs.ur[sl], F1v = rs.F1[sl];
           const R r = ((R)c0 + f0) * dR;
-          const R ut = r > (R)0 ? rs.lz[sl] / r : (R)0;
-          const R iG1 = (R)1 / G1v;
-          const R xh = r + (R)0.5 * h * ur0 * iG1;
-          const R yh = (R)0.5 * h * ut * iG1;
+          R iG1, ut, ex = (R)1, ey = (R)0;
+          frame_of(sl, r, iG1, ut);
+          const R xh = r + (R)0.5 * h * ur0 * iG1, yh = (R)0.5 * h * ut * iG1, h2 = xh * xh + yh * yh;
           const R uxh = ur0 + (R)0.5 * h * F1v;
-          const R rh = sqrt(xh * xh + yh * yh);
-          R ex = (R)1, ey = (R)0;
-          if (rh > (R)0) {
-            const R irh = (R)1 / rh;
+          if (h2 > tiny_r2<R>()) {
+            R rh, irh;
+            root_of(h2, rh, irh);
             ex = xh * irh;
             ey = yh * irh;
           }
-          const R iG2 = (R)1 / wr.G2[sl];
+          const R iG2 = rcp_of(wr.G2[sl]);
           const R dx = h * uxh * iG2, dy = h * ut * iG2;
           const R uxn = ur0 + h * F2b * ex, uyn = ut + h * F2b * ey;
           int cn;
-          R fn, rn, urn, utn;
-          move_ring<R>(c0, f0, r, dx, dy, uxn, uyn, inv_dr, dR, nr, cn, fn, rn, urn, utn);
+          R fn, rn, urn, utn, nx, ny;
+          move_ring<R>(c0, f0, r, dx, dy, uxn, uyn, inv_dr, dR, nr, cn, fn, rn, urn, utn, nx, ny);
           if (!(rn >= (R)0 && rn <= R_wall) || !isfinite(urn)) flag(d.status, ST_ESCAPE);
           rs.c[sl] = cn;
           rs.f[sl] = fn;
@@ -332,7 +335,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
         }
       }
       warp_misses<NT, PPT>(miss, [&](int sl) {  // the new positions are in the slots
-        ChargeWin<Pol>::direct(sm.rho, rs.c[b0 + sl], rs.f[b0 + sl], rs.w[b0 + sl]);
+        charge_direct(sm.rho, rs.c[b0 + sl], rs.f[b0 + sl], rs.w[b0 + sl]);
       });
       flush_charge<Pol>(sm, acc, nr);
     }

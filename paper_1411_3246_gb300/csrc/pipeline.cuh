@@ -74,7 +74,17 @@ __device__ __forceinline__ void st_release(int *p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <class Pol, int NT>
+// A counter's next value, released: everything this CTA wrote before (and saw) is visible to who
+// acquires it.
+__device__ __forceinline__ void red_release(int *p) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
+}
+
+// kCl: one step is marched by the CTAs of a cluster (march.cuh); every CTA holds the step's field
+// window and pushes its share of each cell.  progress[t] then counts the CTAs' finished cells: no
+// CTA finishes cell b + 1 before all have finished cell b (cluster barriers lie between), so a count
+// of cn (b + 1) means that all have finished cell b.
+template <class Pol, int NT, bool kCl = false>
 struct PipeHooks {
   using R = typename Pol::R;
   using G = typename Pol::G;
@@ -83,10 +93,13 @@ struct PipeHooks {
   using Box = typename W::Box;
   static constexpr bool kTraj = false;
   static constexpr bool kTrap = false;
+  static constexpr bool kCluster = kCl;
   const PipeArgs &a;
   int t;          // step within the launch
   R *win;         // 4 slices x (E_r, E_z, B_theta) x n1
-  int *ctl;       // [0] abort flag, [1] progress seen of step t-1
+  int *ctl;       // [0] abort flag, [1] progress seen of step t-1, [2] [3] the next-cell entries of
+                  // the cell pushed last; clusters also [4] second-list entries, [6] [7] this
+                  // CTA's abort flag as its peers read it, by the row's parity
   int n1, nr, nxi;
   double dr, dxi, rmax, ximax;
 
@@ -97,8 +110,8 @@ struct PipeHooks {
   // then meets at one barrier, so the decision is uniform.
   __device__ __forceinline__ bool wait_row(int row) {
     if (t == 0) return true;
-    const int need = min(nxi, row + 1);
-    if (threadIdx.x == 0 && ctl[1] < need) {
+    const int need = (kCl ? cl_size() : 1) * min(nxi, row + 1);
+    if (threadIdx.x == 0 && ctl[1] < need && !(kCl && ctl[0])) {
       long long it = 0;
       int v = ld_acquire(&a.progress[t - 1]);
       while (v < need) {
@@ -112,14 +125,36 @@ struct PipeHooks {
       }
       ctl[1] = v;
     }
+    if (kCl) {  // one CTA's answer is not the cluster's: march on, and ask the others (given_up)
+      if (threadIdx.x == 0) ctl[6 + (row & 1)] = ctl[0];
+      __syncthreads();
+      return true;
+    }
     __syncthreads();
     return ctl[0] == 0;
+  }
+  // whether any CTA of the cluster gave up waiting for this row or an earlier one.  A flag is read
+  // here and written again two rows on, with cluster barriers in between.
+  __device__ __forceinline__ bool given_up(int row) {
+    const int cn = cl_size();
+    int any = 0;
+    for (int r = 0; r < cn; ++r) any |= *cl_peer(ctl + 6 + (row & 1), r);
+    if (any && threadIdx.x == 0) ctl[0] = 1;
+    return any != 0;
+  }
+  // the list entries made while the last cell was pushed, by all CTAs of the cluster
+  __device__ __forceinline__ void between_pushes() {
+    if (threadIdx.x == 0) {
+      ctl[2] = ctl[3];
+      ctl[3] = __ldcg(a.defer_cnt + 2 * t);
+      ctl[4] = __ldcg(a.defer_cnt + 2 * t + 1);
+    }
   }
   __device__ __forceinline__ R nb_row(int row, int m) const { return (R)__ldcg(grid(t) + (size_t)row * n1 + m); }
 
   __device__ __forceinline__ void slice_done(int k, MarchSmem<Pol> &sm) {
     R *w = win + (size_t)(k & 3) * 3 * n1;
-    const bool out = a.write_last && t == a.nsteps - 1;
+    const bool out = a.write_last && t == a.nsteps - 1 && (!kCl || cl_rank() == 0);
     G *o1 = (G *)a.d.psi + (size_t)k * n1, *o2 = (G *)a.d.ez + (size_t)k * n1, *o3 = (G *)a.d.er + (size_t)k * n1,
       *o4 = (G *)a.d.bth + (size_t)k * n1;
     for (int m = threadIdx.x; m < n1; m += NT) {
@@ -269,7 +304,8 @@ struct PipeHooks {
   __device__ void push_cell(int b) {
     const Box bx = W::box(dxi, ximax, a.ffi, a.ffx);
     const int beg = a.bin_start[b], end = a.bin_start[b + 1];
-    for (int j = beg + threadIdx.x; j < end; j += NT) {
+    const int i0 = kCl ? cl_rank() * NT + threadIdx.x : threadIdx.x, di = kCl ? cl_size() * NT : NT;
+    for (int j = beg + i0; j < end; j += di) {
       Part p;
       load_part(j, p);  // every load of the particle at once, before any branch on them
       if (p.fl & 1) continue;
@@ -287,23 +323,27 @@ struct PipeHooks {
       }
       push_one(j, p, kk, g, bx);
     }
-    __syncthreads();  // every entry counted so far is written
+    if (!kCl) __syncthreads();  // every entry counted so far is written
     // this step's listed particles for cell b: the next-cell entries made while cell b - 1 was
     // pushed (ctl[2] .. ctl[3]), and the others whose target is b
     const int2 *near = a.near_list + (size_t)t * a.near_cap;
     const int2 *far = a.defer_list + (size_t)t * a.defer_cap;
-    for (int q = ctl[2] + threadIdx.x; q < ctl[3]; q += NT) push_listed(b, __ldcg(near + q % a.near_cap).x, bx);
-    const int nf = min(__ldcg(a.defer_cnt + 2 * t + 1), a.defer_cap);
-    for (int q = threadIdx.x; q < nf; q += NT) {
+    for (int q = ctl[2] + i0; q < ctl[3]; q += di) push_listed(b, __ldcg(near + q % a.near_cap).x, bx);
+    const int nf = min(kCl ? ctl[4] : __ldcg(a.defer_cnt + 2 * t + 1), a.defer_cap);
+    for (int q = i0; q < nf; q += di) {
       const int2 e = __ldcg(far + q);
       if (e.y == b) push_listed(b, e.x, bx);
     }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-      st_release(&a.progress[t], b + 1);
-      ctl[2] = ctl[3];  // the entries made while cell b was pushed are cell b + 1's
-      ctl[3] = __ldcg(a.defer_cnt + 2 * t);
+      if (kCl) {
+        red_release(&a.progress[t]);
+      } else {
+        st_release(&a.progress[t], b + 1);
+        ctl[2] = ctl[3];  // the entries made while cell b was pushed are cell b + 1's
+        ctl[3] = __ldcg(a.defer_cnt + 2 * t);
+      }
     }
   }
 };
@@ -337,6 +377,27 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(PipeArgs a) {
     march_body<Pol, NT, PPT>(d, smem_raw, hk);
     __syncthreads();
     if (ctl[0]) break;
+  }
+}
+
+// The same, one cluster per step.
+template <class Pol, int NT, int PPT>
+__global__ void __launch_bounds__(NT, 2) step_cluster_kernel(PipeArgs a) {
+  using R = typename Pol::R;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n1 = a.d.nr + 1, cn = cl_size();
+  const size_t base = (MarchSmem<Pol>::bytes(n1, NT * PPT) + 63) & ~(size_t)63;
+  R *win = (R *)(smem_raw + base);
+  int *ctl = (int *)(win + (size_t)12 * n1);
+  for (int t = blockIdx.x / cn; t < a.nsteps; t += gridDim.x / cn) {
+    if (threadIdx.x < 8) ctl[threadIdx.x] = 0;
+    __syncthreads();
+    PipeHooks<Pol, NT, true> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
+    SimDesc d = a.d;
+    if (!Pol::kSmemRings) d.ring_buf = (unsigned char *)a.ring_bufs + (size_t)(blockIdx.x / cn) * a.ring_stride;
+    march_body<Pol, NT, PPT>(d, smem_raw, hk);
+    __syncthreads();
+    if (ctl[0]) break;  // the same in every CTA of the cluster
   }
 }
 

@@ -113,7 +113,9 @@ struct wake_sim {
   // march tiles: simulations grouped by the tile the autotuner chose (planned at the first march)
   struct TileClass {
     TileFns fns;
-    int n1max = 0, off = 0, count = 0;
+    int n1max = 0, npmax = 0, off = 0, count = 0;
+    int cluster = 1;  // CTAs per simulation
+    bool slab = false;
     cudaStream_t side = nullptr;  // class 0 runs on the handle's stream
     cudaEvent_t done = nullptr;
   };
@@ -362,6 +364,28 @@ int probe_tile(wake_sim *h, const Sim &s, const SimDesc &d, const TileFns &f, do
   return WAKE_OK;
 }
 
+// CTAs per simulation (or beam step) when `count` of them run at once: 1, or a cluster that shares
+// each one's rings.  The field solves are repeated by every CTA and the sums over the cluster cost
+// about 13k cycles a slice (8 CTAs), so a cluster pays where a CTA's ring passes cost more.  FP64 (its
+// pipe bounds the ring passes; linear march alone 20.1 ms with one CTA, 13.2 with 4, 13.1 with 8; 256
+// rings 15.6, 11.8 and 12.0 ms; 24 steps 103 ms, 48 with 4): as many CTAs as leave 64 rings to each and
+// fit the GPU at once.  Mixed (one march alone, 1 / 4 / 8 CTAs: 512 rings 2.8 / 3.5 / 3.6 ms, 1024 6.4 /
+// 5.8 / 6.0, 1536 8.7 / 7.7 / 6.4, 4096 69.5 / 58.8 / 41.8): 4 from 1024 rings and 8 from 1536, and only
+// while half of the SMs stay free for other streams' work, since a cluster does more work in all.
+int pick_cluster(wake_sim *h, const wake_sim::TileClass &k, int count, bool step) {
+  if (h->tile_nt_forced || h->precision == WAKE_MIXED64) return 1;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  const bool fp64 = h->precision == WAKE_FP64;
+  int cn = 1;
+  if (fp64)
+    for (int c = 8; c > 1 && cn == 1; c /= 2) cn = count * c <= sms && k.npmax >= 64 * c ? c : 1;
+  else
+    cn = k.npmax >= 1536 && count * 16 <= sms ? 8 : (k.npmax >= 1024 && count * 8 <= sms ? 4 : 1);
+  return cn > 1 && cluster_max(h->precision, k.slab, step, k.n1max, k.npmax, cn) >= count ? cn : 1;
+}
+
 // Choose a tile per simulation (the best probe score per distinct (Nr, Np); the only
 // candidate when there is one) and group the simulations by tile, each group largest work
 // first.  Synchronous (the probes are timed).
@@ -433,6 +457,11 @@ int plan_tiles(wake_sim *h) {
     if (ep != cudaSuccess) return fail(WAKE_ECUDA, std::string("march tile set-up: ") + cudaGetErrorString(ep));
     h->classes[c].off = (int)order.size();
     h->classes[c].count = (int)mine.size();
+    for (int i : mine) h->classes[c].npmax = std::max(h->classes[c].npmax, h->sims[i].np);
+    h->classes[c].slab = h->sims[mine[0]].p.geometry == WAKE_SLAB;
+    bool one_geometry = true;
+    for (int i : mine) one_geometry = one_geometry && (h->sims[i].p.geometry == WAKE_SLAB) == h->classes[c].slab;
+    if (one_geometry && !pick[mine[0]].wide) h->classes[c].cluster = pick_cluster(h, h->classes[c], h->n, false);
     order.insert(order.end(), mine.begin(), mine.end());
     if (c > 0) {
       CUDA_TRY(cudaStreamCreateWithFlags(&h->classes[c].side, cudaStreamNonBlocking));
@@ -457,7 +486,10 @@ int launch_march(wake_sim *h) {
     auto &k = h->classes[c];
     cudaStream_t st = c == 0 ? h->stream : k.side;
     if (c > 0) CUDA_TRY(cudaStreamWaitEvent(st, h->fork, 0));
-    const cudaError_t e = k.fns.launch(h->d_desc, h->d_order + k.off, k.count, k.n1max, st);
+    const cudaError_t e =
+        k.cluster > 1 ? launch_march_cluster(h->precision, k.slab, h->d_desc, h->d_order + k.off, k.count, k.n1max, k.npmax,
+                                             k.cluster, st)
+                      : k.fns.launch(h->d_desc, h->d_order + k.off, k.count, k.n1max, st);
     if (e != cudaSuccess) return fail(WAKE_ECUDA, std::string("march launch: ") + cudaGetErrorString(e));
     if (c > 0) CUDA_TRY(cudaEventRecord(k.done, st));
   }
@@ -1228,6 +1260,15 @@ int step_batched(wake_sim *h, int nsteps) {
 // the grids of the later steps and the progress counters, launch.
 int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
   Sim &s = h->sims[0];
+  int cn = 1;
+  if (!wide_nt && h->precision != WAKE_MIXED64) {
+    wake_sim::TileClass k;
+    k.n1max = s.p.nr + 1;
+    k.npmax = s.np;
+    k.slab = s.p.geometry == WAKE_SLAB;
+    cn = pick_cluster(h, k, nsteps, true);
+    if (cn > 1) ctas_max = cluster_max(h->precision, k.slab, true, k.n1max, k.npmax, cn);
+  }
   const int fp64 = h->precision == WAKE_FP64;
   const size_t gs = gsize(h->precision), gbytes = gs * s.ng;
   // every step of a launch owns a density grid: up to a quarter of the free memory
@@ -1383,7 +1424,8 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
       h->ev.push_back(q);
     }
     CUDA_TRY(cudaEventRecord(h->ev[h->ev_used].first, h->stream));
-    const cudaError_t e = wide64 ? launch_step_wide_fp64(a, ctas, h->stream)
+    const cudaError_t e = cn > 1   ? launch_step_cluster(h->precision, a, cn, ctas, h->stream)
+                          : wide64 ? launch_step_wide_fp64(a, ctas, h->stream)
                                  : (wnt ? launch_step_wide(a, wnt, ctas, h->stream) : launch_step(h->precision, a, s.np, ctas, h->stream));
     if (e != cudaSuccess) return fail(WAKE_ECUDA, std::string("pipelined step launch: ") + cudaGetErrorString(e));
     CUDA_TRY(cudaEventRecord(h->ev[h->ev_used].second, h->stream));
