@@ -267,44 +267,80 @@ __device__ __forceinline__ void boris_step(BT &x, BT &y, BT &ux, BT &uy, typenam
   W::add(xi, dt * ((BT)1 + up2) / (gam * (gam + uzn)));
 }
 
-// One beam step through the grid fields of the last march, bilinear gather in (r, xi):
-// particles j0, j0 + stride, ...
+// The fields at the four nodes around a particle, weighted: from the three grids, or from nodes
+// packed as (E_r, E_z, B_theta, 0), one 16-byte load each instead of three.
 template <class BT, class G>
-__device__ __forceinline__ void push_range(const BeamDesc &b, int64_t j0, int64_t stride) {
-  const G *er = (const G *)b.er, *ez = (const G *)b.ez, *bt = (const G *)b.bth;
+struct GridFields {
+  const G *er, *ez, *bt;
+  __device__ __forceinline__ void at(size_t i00, int n1, BT w00, BT w01, BT w10, BT w11, BT &Er, BT &Ez, BT &Bt) const {
+    Er = w00 * (BT)er[i00] + w01 * (BT)er[i00 + 1] + w10 * (BT)er[i00 + n1] + w11 * (BT)er[i00 + n1 + 1];
+    Ez = w00 * (BT)ez[i00] + w01 * (BT)ez[i00 + 1] + w10 * (BT)ez[i00 + n1] + w11 * (BT)ez[i00 + n1 + 1];
+    Bt = w00 * (BT)bt[i00] + w01 * (BT)bt[i00 + 1] + w10 * (BT)bt[i00 + n1] + w11 * (BT)bt[i00 + n1 + 1];
+  }
+};
+struct PackedFields {
+  const float4 *f;
+  __device__ __forceinline__ void at(size_t i00, int n1, float w00, float w01, float w10, float w11, float &Er, float &Ez,
+                                     float &Bt) const {
+    const float4 a = __ldg(f + i00), b = __ldg(f + i00 + 1), c = __ldg(f + i00 + n1), d = __ldg(f + i00 + n1 + 1);
+    Er = w00 * a.x + w01 * b.x + w10 * c.x + w11 * d.x;
+    Ez = w00 * a.y + w01 * b.y + w10 * c.y + w11 * d.y;
+    Bt = w00 * a.z + w01 * b.z + w10 * c.z + w11 * d.z;
+  }
+};
+static __global__ void pack_fields_kernel(const float *__restrict__ er, const float *__restrict__ ez,
+                                          const float *__restrict__ bt, float4 *__restrict__ out, int64_t n) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+    out[t] = make_float4(er[t], ez[t], bt[t], 0.f);
+}
+
+// nsteps beam steps through the grid fields of the last march (the same in every step), bilinear
+// gather in (r, xi): particles j0, j0 + stride, ...  A particle's steps are taken one after the
+// other in registers: its state crosses memory once, whatever nsteps is (4.2e6 particles, 8 steps
+// on 200 x 500 cells: 1,269 us per pass with a launch per step).
+template <class BT, class Fields>
+__device__ __forceinline__ void push_range(const BeamDesc &b, const Fields &fld, int nsteps, int64_t j0, int64_t stride) {
   BT *X = (BT *)b.x, *Y = (BT *)b.y, *UX = (BT *)b.ux, *UY = (BT *)b.uy;
   const int n1 = b.nr + 1;
   using W = BeamWide<BT>;
   const BT inv_dr = (BT)(1.0 / b.dr), dt = (BT)b.ds, Rw = (BT)b.rmax;
   const typename W::Box bx = W::box(b.dxi, b.ximax, b.ffi, b.ffx);
   for (int64_t j = j0; j < b.n_cap; j += stride) {
-    if (b.lost[j] & 1) continue;
-    BT x = X[j], y = Y[j], ux = UX[j], uy = UY[j];
+    const uint8_t fl = b.lost[j];
+    BT x = X[j], y = Y[j], ux = UX[j], uy = UY[j];  // loaded beside the flag, not behind it
     typename W::T xi = W::ld(b.xi, j), uzd = W::ld(b.uz, j);
-    const BT r = sqrt(x * x + y * y);
-    int c, k;
-    BT f, g;
-    locate(r, inv_dr, b.nr, c, f);
-    W::cell(xi, bx, b.nxi, k, g);
-    const size_t i00 = (size_t)k * n1 + c;
-    const BT w00 = ((BT)1 - f) * ((BT)1 - g), w01 = f * ((BT)1 - g), w10 = ((BT)1 - f) * g, w11 = f * g;
-    const BT Er = w00 * (BT)er[i00] + w01 * (BT)er[i00 + 1] + w10 * (BT)er[i00 + n1] + w11 * (BT)er[i00 + n1 + 1];
-    const BT Ez = w00 * (BT)ez[i00] + w01 * (BT)ez[i00 + 1] + w10 * (BT)ez[i00 + n1] + w11 * (BT)ez[i00 + n1 + 1];
-    const BT Bt = w00 * (BT)bt[i00] + w01 * (BT)bt[i00 + 1] + w10 * (BT)bt[i00 + n1] + w11 * (BT)bt[i00 + n1 + 1];
-    boris_step<BT>(x, y, ux, uy, xi, uzd, r, Er, Ez, Bt, dt);
+    if (fl & 1) continue;
+    bool in = true;
+    for (int s = 0; s < nsteps && in; ++s) {
+      const BT r = sqrt(x * x + y * y);  // formed anew, as a launch per step forms it: the same bits
+      int c, k;
+      BT f, g;
+      locate(r, inv_dr, b.nr, c, f);
+      W::cell(xi, bx, b.nxi, k, g);
+      const BT w00 = ((BT)1 - f) * ((BT)1 - g), w01 = f * ((BT)1 - g), w10 = ((BT)1 - f) * g, w11 = f * g;
+      BT Er, Ez, Bt;
+      fld.at((size_t)k * n1 + c, n1, w00, w01, w10, w11, Er, Ez, Bt);
+      boris_step<BT>(x, y, ux, uy, xi, uzd, r, Er, Ez, Bt, dt);
+      const BT rn = sqrt(x * x + y * y);
+      in = W::inside(xi, bx) && rn < Rw;
+    }
     X[j] = x;
     Y[j] = y;
     UX[j] = ux;
     UY[j] = uy;
     W::st(b.xi, j, xi);
     W::st(b.uz, j, uzd);
-    const BT rn = sqrt(x * x + y * y);
-    if (!(W::inside(xi, bx) && rn < Rw)) b.lost[j] |= 1;
+    if (!in) b.lost[j] = fl | 1;
   }
 }
 template <class BT, class G>
-__global__ void beam_push_kernel(BeamDesc b) {
-  push_range<BT, G>(b, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+__global__ void beam_push_kernel(BeamDesc b, int nsteps) {
+  const GridFields<BT, G> fld{(const G *)b.er, (const G *)b.ez, (const G *)b.bth};
+  push_range<BT>(b, fld, nsteps, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+}
+static __global__ void beam_push_packed_kernel(BeamDesc b, const float4 *fields, int nsteps) {
+  push_range<float>(b, PackedFields{fields}, nsteps, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+                    (int64_t)gridDim.x * blockDim.x);
 }
 
 // Batched forms over the simulations of a handle: blockIdx.y is the simulation; simulations
@@ -330,9 +366,10 @@ __global__ void nb_normalize_batch_kernel(const BeamDesc *bs) {
                      (int64_t)gridDim.x * blockDim.x);
 }
 template <class BT, class G>
-__global__ void beam_push_batch_kernel(const BeamDesc *bs) {
+__global__ void beam_push_batch_kernel(const BeamDesc *bs, int nsteps) {
   const BeamDesc b = bs[blockIdx.y];
-  push_range<BT, G>(b, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+  const GridFields<BT, G> fld{(const G *)b.er, (const G *)b.ez, (const G *)b.bth};
+  push_range<BT>(b, fld, nsteps, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // Witness / drive sums in FP64: counts, sum(gamma - gamma_b), sum(gamma - gamma_b)^2.

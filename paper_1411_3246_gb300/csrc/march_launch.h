@@ -48,6 +48,10 @@ size_t wide_fp64_ring_bytes(int np, int n1);
 size_t step_wide_fp64_window_bytes(int n1);
 int step_wide_fp64_max_ctas(int n1);
 cudaError_t launch_step_wide_fp64(const PipeArgs &a, int ctas, cudaStream_t stream);
+// Pipelined steps in the wide form, one cluster of cn CTAs of 512 threads per step.
+size_t step_wide_cluster_ring_bytes(int np, int cn);
+int step_wide_cluster_max(int n1, int cn);
+cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cudaStream_t stream);
 // Pipelined steps of many simulations (pipeline.cuh batch_step_kernel), wide form.
 struct BatchArgs;
 int batch_step_max_ctas(int max_n1, int bnt);

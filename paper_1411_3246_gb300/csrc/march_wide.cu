@@ -92,6 +92,51 @@ cudaError_t launch_step_wide(const PipeArgs &a, int nt, int ctas, cudaStream_t s
   return nt == 256 ? step_wide_launch<256>(a, ctas, stream) : step_wide_launch<512>(a, ctas, stream);
 }
 
+// The steps of clusters of cn CTAs of 512 threads: ring bytes of one cluster, clusters the GPU holds
+// at once (0: does not fit), launch.
+static void wide_cluster_config(cudaLaunchConfig_t *c, cudaLaunchAttribute *at, int clusters, int cn, size_t bytes, bool coop,
+                                cudaStream_t stream) {
+  *c = cudaLaunchConfig_t{};
+  c->gridDim = dim3(clusters * cn);
+  c->blockDim = dim3(kWideNT);
+  c->dynamicSmemBytes = bytes;
+  c->stream = stream;
+  at[0] = at[1] = cudaLaunchAttribute{};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cn;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;
+  at[1].val.cooperative = 1;
+  c->attrs = at;
+  c->numAttrs = coop ? 2 : 1;
+}
+size_t step_wide_cluster_ring_bytes(int np, int cn) {
+  return (size_t)cn * wide_share_bytes<float, kWideNT, kWidePPT>((np + cn - 1) / cn);
+}
+int step_wide_cluster_max(int n1, int cn) {
+  auto kern = step_wide_cluster_kernel<PolWide, kWideNT, kWidePPT>;
+  const size_t smem = step_wide_smem(n1);
+  if (smem > kMaxSmemPerCta || n1 > PolWide::kScanE * kWideNT) return 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  cudaLaunchConfig_t c;
+  cudaLaunchAttribute at[2];
+  wide_cluster_config(&c, at, 1, cn, smem, false, nullptr);
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, kern, &c) == cudaSuccess ? n : 0;
+}
+cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cudaStream_t stream) {
+  auto kern = step_wide_cluster_kernel<PolWide, kWideNT, kWidePPT>;
+  const size_t smem = step_wide_smem(a.d.nr + 1);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t c;
+  cudaLaunchAttribute at[2];
+  wide_cluster_config(&c, at, clusters, cn, smem, true, stream);
+  PipeArgs arg = a;
+  void *args[] = {&arg};
+  return cudaLaunchKernelExC(&c, (const void *)kern, args);
+}
+
 // The batched pipelined kernel in CTAs of bnt = 512 or 256 threads (the latter two per SM).
 template <int NT>
 static int batch_ctas(int max_n1) {

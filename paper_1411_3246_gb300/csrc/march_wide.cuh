@@ -116,17 +116,39 @@ __host__ __device__ inline int wide_slots(int np) {
   return (np + NT * PPT - 1) / (NT * PPT) * (NT * PPT);
 }
 
+// Bytes of the ring slots of one CTA that marches `share` rings.
+template <class R, int NT, int PPT>
+__host__ __device__ inline size_t wide_share_bytes(int share) {
+  return (WideRings<R>::bytes(wide_slots<NT, PPT>(share)) + 255) & ~(size_t)255;
+}
+
 template <class Pol, int NT, int PPT, class Hooks>
 __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char *smem_raw, Hooks &hk) {
   using R = typename Pol::R;
   using Acc = typename Pol::Acc;
   constexpr int SLOTS = NT * PPT, PRE = Pol::kScanE;
-  const int tid = threadIdx.x, nr = d.nr, n1 = nr + 1, np = d.np, nxi = d.nxi;
-  const int nch = (np + SLOTS - 1) / SLOTS;
+  constexpr bool kCl = Hooks::kCluster;
+  // the CTA's rings j0 .. j0 + np - 1, as in march_body
+  const int cn = kCl ? cl_size() : 1, cr = kCl ? cl_rank() : 0;
+  const int share = kCl ? (d.np + cn - 1) / cn : d.np, j0 = cr * share;
+  const int tid = threadIdx.x, nr = d.nr, n1 = nr + 1, np = kCl ? max(0, min(share, d.np - j0)) : d.np, nxi = d.nxi;
+  const int nch = (share + SLOTS - 1) / SLOTS;
   MarchSmem<Pol> sm;
   sm.carve(smem_raw, n1, SLOTS);
   WideRings<R> wr;
-  wr.carve(d.ring_buf, nch * SLOTS);
+  wr.carve((unsigned char *)d.ring_buf + (kCl ? (size_t)cr * wide_share_bytes<R, NT, PPT>(share) : 0), nch * SLOTS);
+  auto sum_charge = [&]() {
+    if constexpr (kCl)
+      cluster_sum<NT>(sm.rho, n1, cn, cr);
+    else
+      __syncthreads();
+  };
+  auto sum_currents = [&]() {
+    if constexpr (kCl) {
+      using V = std::conditional_t<sizeof(Acc) == 4, float2, double>;
+      cluster_sum<NT>((V *)sm.jz, (int)(6 * n1 * sizeof(Acc) / sizeof(V)), cn, cr);
+    }
+  };
   const RingSoA<R> &rs = wr.s;  // follows the swaps of the re-sort
   const double drd = d.dr;
   const R h = (R)d.dxi, R_wall = (R)d.rmax, dR = (R)drd, inv_dr = (R)(1.0 / drd);
@@ -142,8 +164,8 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     const int base = ch * SLOTS;
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-      const int j = base + tid * PPT + p, sl = base + p * NT + tid;
-      if (j < np) {
+      const int jl = base + tid * PPT + p, sl = base + p * NT + tid, j = j0 + jl;
+      if (jl < np) {
         const double s = d.r0[j] / drd;
         int c = (int)floor(s);
         c = c < 0 ? 0 : (c > nr - 1 ? nr - 1 : c);
@@ -199,7 +221,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
       }
     flush_charge<Pol>(sm, acc, nr);
   }
-  __syncthreads();
+  sum_charge();
   for (int m = tid; m < n1; m += NT) sm.rho0[m] = sm.rho[m];
   __syncthreads();
 
@@ -229,6 +251,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
         }
     }
     __syncthreads();
+    sum_currents();
     solve_fields<Pol, NT>(sm, geo, nbk, nbk, sm.wtot);
     hk.slice_done(k, sm);
     if (k == nxi) break;
@@ -258,7 +281,8 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
       });
       flush_charge<Pol>(sm, acc, nr);
     }
-    __syncthreads();
+    sum_charge();
+    if constexpr (kCl) hk.between_pushes();
     // ======== stage 2 at xi_k + dxi/2 ========
     if (!hk.wait_row(k + 1)) break;  // row k+1 is first read by this stage
     R pre[PRE];
@@ -292,6 +316,9 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
         }
     }
     __syncthreads();
+    sum_currents();
+    if constexpr (kCl)
+      if (hk.given_up(k + 1)) break;  // the same answer in every CTA of the cluster
     solve_fields<Pol, NT>(sm, geo, nbk, nbk1, sm.wtot);
     // full step from the slice-k state with the midpoint derivative; charge of the new slice
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
@@ -339,9 +366,10 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
       });
       flush_charge<Pol>(sm, acc, nr);
     }
-    __syncthreads();
+    sum_charge();
   }
   hk.finish(sm);
+  if constexpr (kCl) cl_barrier();  // no CTA leaves while another may still read its arrays
 }
 
 template <class Pol, int NT, int PPT>

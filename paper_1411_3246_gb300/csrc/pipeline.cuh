@@ -427,6 +427,27 @@ __global__ void __launch_bounds__(NT, (NT < 512 ? 512 / NT : 1)) step_wide_kerne
   }
 }
 
+// The wide form, one cluster per step.
+template <class Pol, int NT, int PPT>
+__global__ void __launch_bounds__(NT, 1) step_wide_cluster_kernel(PipeArgs a) {
+  using R = typename Pol::R;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n1 = a.d.nr + 1, cn = cl_size();
+  const size_t base = (MarchSmem<Pol>::bytes(n1, NT * PPT) + 63) & ~(size_t)63;
+  int *ctl = (int *)(smem_raw + base);
+  R *win = (R *)((unsigned char *)a.win_bufs + (size_t)blockIdx.x * a.win_stride);
+  for (int t = blockIdx.x / cn; t < a.nsteps; t += gridDim.x / cn) {
+    if (threadIdx.x < 8) ctl[threadIdx.x] = 0;
+    __syncthreads();
+    PipeHooks<Pol, NT, true> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
+    SimDesc d = a.d;
+    d.ring_buf = (unsigned char *)a.ring_bufs + (size_t)(blockIdx.x / cn) * a.ring_stride;
+    march_body_wide<Pol, NT, PPT>(d, smem_raw, hk);
+    __syncthreads();
+    if (ctl[0]) break;  // the same in every CTA of the cluster
+  }
+}
+
 // Pipelined steps of many simulations in one persistent launch.  Work items are (simulation,
 // step) pairs in the order the host gives (all steps of a simulation consecutive, largest
 // simulations first); CTA c takes items c, c + gridDim.x, ...  An item's predecessor (the

@@ -62,6 +62,7 @@ struct Sim {
   size_t defer_bytes = 0;
   int2 *near_list = nullptr;  // pipelined steps: the next-cell rings
   size_t near_bytes = 0;
+  void *fpack = nullptr;  // mixed form, one simulation: packed nodes (E_r, E_z, B_theta, 0) of a push
   int *status = nullptr;
   // trapping (wake_set_trapping): beam slots for promoted particles, the march's promotions
   int64_t n_cap = 0;            // beam slots: n_beam, plus room for promoted particles
@@ -147,7 +148,7 @@ void free_sim(Sim &s) {
   void *ptrs[] = {s.r0, s.ur0, s.lz, s.G0, s.w, s.ring_buf, s.nb, s.psi, s.ez, s.er, s.bth, s.bx, s.by, s.bux, s.buy,
                   s.bxi, s.buz, s.blost, s.status, s.orig, s.bx2, s.by2, s.bux2, s.buy2, s.bxi2, s.buz2, s.blost2,
                   s.orig2, s.bin_count, s.bin_start, s.bin_cursor, s.slip, s.pgrids, s.progress, s.pring,
-                  s.defer_cnt, s.target, s.defer_list, s.near_list, s.bwt, s.bwt2, s.trap_list, s.trap_count,
+                  s.fpack, s.defer_cnt, s.target, s.defer_list, s.near_list, s.bwt, s.bwt2, s.trap_list, s.trap_count,
                   s.trap_used};
   for (void *q : ptrs)
     if (q) cudaFree(q);
@@ -558,6 +559,14 @@ int wake_init(const wake_params *p, int n_sims, void *stream, wake_sim **out) {
     if (p[i].n_beam > 0) {
       s.n_cap = p[i].n_beam;
       if ((rc = alloc_beam(h, s))) break;
+      // packed nodes for the separate pushes of a beam of more particles than nodes (a sixteenth
+      // of the grids' own and the beam's memory in the workloads that use it); without them the
+      // push gathers from the three grids
+      if (n_sims == 1 && h->precision != WAKE_FP64 && p[i].n_beam >= (int64_t)s.ng &&
+          cudaMalloc(&s.fpack, sizeof(float4) * s.ng) != cudaSuccess) {
+        s.fpack = nullptr;
+        cudaGetLastError();
+      }
     } else {
       // frozen analytic driver (Eq. 12) on the nodes
       const double dr = p[i].rmax / p[i].nr, dxi = p[i].ximax / p[i].nxi;
@@ -868,27 +877,24 @@ int wake_bind_fields(wake_sim *h, int sim, void *psi, void *ez, void *er, void *
   return WAKE_OK;
 }
 
-int wake_beam_push_steps(wake_sim *h, int nsteps) {
-  if (!h || nsteps < 0) return fail(WAKE_EINVAL, "wake_beam_push_steps: null handle or nsteps < 0");
-  for (int t = 0; t < nsteps; ++t) {
-    const int rc = wake_beam_push(h);
-    if (rc) return rc;
-  }
-  return WAKE_OK;
-}
+namespace {
 
-int wake_beam_push(wake_sim *h) {
-  if (!h) return fail(WAKE_EINVAL, "null handle");
+// nsteps beam steps through the fields of the last march.  A launch takes up to 64 of them, so that
+// no single kernel keeps other streams waiting long.
+int push_steps(wake_sim *h, int nsteps) {
   if (h->n > 1) {
     for (auto &s : h->sims)
       if (s.p.n_beam > 0 && (!s.beam || !s.marched))
         return fail(WAKE_ESTATE, "wake_beam_push needs a loaded beam and a march");
     if (h->max_beam == 0) return WAKE_OK;
     const dim3 gb(batch_blocks(h->max_beam), h->n);
-    if (h->precision == WAKE_FP64)
-      beam_push_batch_kernel<double, double><<<gb, 256, 0, h->stream>>>(h->d_bdesc);
-    else
-      beam_push_batch_kernel<float, float><<<gb, 256, 0, h->stream>>>(h->d_bdesc);
+    for (int t = 0; t < nsteps; t += 64) {
+      const int m = std::min(64, nsteps - t);
+      if (h->precision == WAKE_FP64)
+        beam_push_batch_kernel<double, double><<<gb, 256, 0, h->stream>>>(h->d_bdesc, m);
+      else
+        beam_push_batch_kernel<float, float><<<gb, 256, 0, h->stream>>>(h->d_bdesc, m);
+    }
     CUDA_TRY(cudaGetLastError());
     return WAKE_OK;
   }
@@ -908,13 +914,36 @@ int wake_beam_push(wake_sim *h) {
       s.trap_pending = false;
     }
     const int nb = grid_blocks(b.n_cap, 256);
-    if (h->precision == WAKE_FP64)
-      beam_push_kernel<double, double><<<nb, 256, 0, h->stream>>>(b);
-    else
-      beam_push_kernel<float, float><<<nb, 256, 0, h->stream>>>(b);
+    // packing moves 28 bytes a node once and saves eight of a push's twelve gathers
+    const bool packed = s.fpack && (double)nsteps * b.n_cap >= 2.0 * (double)s.ng;
+    if (packed)
+      pack_fields_kernel<<<grid_blocks((int64_t)s.ng, 256), 256, 0, h->stream>>>((const float *)s.er, (const float *)s.ez,
+                                                                                 (const float *)s.bth, (float4 *)s.fpack,
+                                                                                 (int64_t)s.ng);
+    for (int t = 0; t < nsteps; t += 64) {
+      const int m = std::min(64, nsteps - t);
+      if (h->precision == WAKE_FP64)
+        beam_push_kernel<double, double><<<nb, 256, 0, h->stream>>>(b, m);
+      else if (packed)
+        beam_push_packed_kernel<<<nb, 256, 0, h->stream>>>(b, (const float4 *)s.fpack, m);
+      else
+        beam_push_kernel<float, float><<<nb, 256, 0, h->stream>>>(b, m);
+    }
     CUDA_TRY(cudaGetLastError());
   }
   return WAKE_OK;
+}
+
+}  // namespace
+
+int wake_beam_push_steps(wake_sim *h, int nsteps) {
+  if (!h || nsteps < 0) return fail(WAKE_EINVAL, "wake_beam_push_steps: null handle or nsteps < 0");
+  return nsteps == 0 ? WAKE_OK : push_steps(h, nsteps);
+}
+
+int wake_beam_push(wake_sim *h) {
+  if (!h) return fail(WAKE_EINVAL, "null handle");
+  return push_steps(h, 1);
 }
 
 namespace {
@@ -1269,6 +1298,16 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
     cn = pick_cluster(h, k, nsteps, true);
     if (cn > 1) ctas_max = cluster_max(h->precision, k.slab, true, k.n1max, k.npmax, cn);
   }
+  if (wide_nt == 512 && h->precision == WAKE_MIXED && !h->tile_nt_forced && !h->step_form) {
+    // wide form, a cluster per step while all steps run at once: the ring passes are nearly all of
+    // its time (8 steps of 2,048 cells and 65,536 rings: 126 ms with one CTA each)
+    int dev = 0, sms = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    for (int c = 8; c > 1 && cn == 1; c /= 2)
+      if (nsteps * c <= sms && step_wide_cluster_max(s.p.nr + 1, c) >= nsteps) cn = c;
+    if (cn > 1) ctas_max = nsteps;
+  }
   const int fp64 = h->precision == WAKE_FP64;
   const size_t gs = gsize(h->precision), gbytes = gs * s.ng;
   // every step of a launch owns a density grid: up to a quarter of the free memory
@@ -1277,7 +1316,8 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
   const int chmax = (int)std::min<size_t>(1024, std::max<size_t>(1, free_b / 4 / gbytes - 1));
   const int wnt = wide_nt;  // 0: the tiled step kernel
   const bool wide64 = wnt && fp64;  // the FP64 wide form: node arrays in the ring buffer
-  const size_t rb = wide64 ? wide_fp64_ring_bytes(s.np, s.p.nr + 1)
+  const size_t rb = wnt && cn > 1 ? step_wide_cluster_ring_bytes(s.np, cn)  // per cluster
+                    : wide64      ? wide_fp64_ring_bytes(s.np, s.p.nr + 1)
                            : (wnt ? step_wide_ring_bytes(s.np, wnt) : ring_buf_bytes(h->precision));
   const size_t wb = wide64 ? step_wide_fp64_window_bytes(s.p.nr + 1)
                            : (wnt ? step_wide_window_bytes(s.p.nr + 1) : step_global_window_bytes(h->precision, s.p.nr + 1));
@@ -1332,12 +1372,13 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
     }
     if ((rc = alloc_target(s))) return rc;
     const int ctas = std::min(ch, ctas_max);
-    if (rb + wb > 0 && s.pring_bytes < (rb + wb) * ctas) {
+    const size_t pring_need = rb * ctas + wb * ctas * cn;  // rings per step, windows per CTA
+    if (pring_need > s.pring_bytes) {
       if (s.pring) cudaFree(s.pring);
       s.pring = nullptr;
       s.pring_bytes = 0;
-      if ((rc = dalloc(&s.pring, (rb + wb) * ctas))) return rc;
-      s.pring_bytes = (rb + wb) * ctas;
+      if ((rc = dalloc(&s.pring, pring_need))) return rc;
+      s.pring_bytes = pring_need;
     }
     int occ = 0;
     if ((rc = sort_beam(h, s, &occ))) return rc;
@@ -1424,7 +1465,8 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
       h->ev.push_back(q);
     }
     CUDA_TRY(cudaEventRecord(h->ev[h->ev_used].first, h->stream));
-    const cudaError_t e = cn > 1   ? launch_step_cluster(h->precision, a, cn, ctas, h->stream)
+    const cudaError_t e = cn > 1 && wnt ? launch_step_wide_cluster(a, cn, ctas, h->stream)
+                          : cn > 1 ? launch_step_cluster(h->precision, a, cn, ctas, h->stream)
                           : wide64 ? launch_step_wide_fp64(a, ctas, h->stream)
                                  : (wnt ? launch_step_wide(a, wnt, ctas, h->stream) : launch_step(h->precision, a, s.np, ctas, h->stream));
     if (e != cudaSuccess) return fail(WAKE_ECUDA, std::string("pipelined step launch: ") + cudaGetErrorString(e));
