@@ -44,3 +44,41 @@ def test_fused_pushes_equal_single_ones(form, slab, n_beam):
     assert 0.02 * n_beam < out[0][1].sum() < n_beam  # some are lost, not all
     assert np.array_equal(out[0][1], out[1][1])
     assert np.array_equal(out[0][0], out[1][0])
+
+
+def test_beam_conversions_round_to_nearest_even():
+    """A beam taken in FP64 and given back by the mixed form: x, y, u_x and u_y rounded to FP32, xi and
+    u_z to the float-float pair, as IEEE conversions give them, on ties, neighbours of powers of
+    two, subnormal and overflowing FP32 values and signed zeros; and the particles at the wall."""
+    import torch
+    from paper_1411_3246_gb300 import build, wake
+    build.build()
+    rng = np.random.default_rng(3)
+    base = np.concatenate([rng.standard_normal(4000) * 10.0 ** rng.integers(-44, 38, 4000), [0.0, -0.0, 1.0, -1.0, 2.0 ** -126,
+                           2.0 ** -149, 2.0 ** -150, 1.5 * 2.0 ** -149, 3.4028235e38, 3.4028236e38, 2.0 ** 100]])
+    f = base.astype(np.float32).astype(np.float64)
+    ties = (f + np.nextafter(base.astype(np.float32), np.float32(np.inf)).astype(np.float64)) / 2
+    with np.errstate(over="ignore"):
+        v = np.concatenate([base, ties, np.nextafter(ties, np.inf), np.nextafter(ties, -np.inf)])
+        v = v[np.isfinite(v)]
+        n = v.size
+        cfg = synth.config_blowout(n_beam=n, nr=33, nxi=71)
+        xyz = np.stack([v, np.roll(v, 1), np.roll(v, 2), np.roll(v, 3), np.roll(v, 5), np.roll(v, 7)])
+        edge = np.array([np.nextafter(cfg.rmax, 0), cfg.rmax, np.nextafter(cfg.rmax, 9), cfg.rmax * (1 - 1e-6), cfg.rmax * (1 + 1e-6)])
+        xyz[0, :5], xyz[1, :5], xyz[2, :5] = edge, 0.0, 1.0
+        ref = xyz.astype(np.float32).astype(np.float64)
+        for q in (2, 5):
+            hi = xyz[q].astype(np.float32).astype(np.float64)
+            ok = np.isfinite(hi)
+            ref[q, ok] = hi[ok] + (xyz[q, ok] - hi[ok]).astype(np.float32).astype(np.float64)
+        lost = ~((xyz[2] >= 0) & (xyz[2] < cfg.ximax) & (np.sqrt(xyz[0] ** 2 + xyz[1] ** 2) < cfg.rmax))
+    with wake.Simulations([cfg], wake.WAKE_MIXED) as s:
+        wake.wake_set_beam(s.h, 0, torch.from_numpy(xyz).cuda())
+        got, gl = s.beam(0)
+        got, gl = got.cpu().numpy(), gl.cpu().numpy()
+    assert np.array_equal(gl != 0, lost)
+    for q in range(6):
+        ok = np.isfinite(ref[q])
+        if q in (2, 5):
+            ok &= np.abs(ref[q]) < 1e38
+        assert np.array_equal(got[q][ok], ref[q][ok]) and np.array_equal(np.signbit(got[q][ok]), np.signbit(ref[q][ok])), q
