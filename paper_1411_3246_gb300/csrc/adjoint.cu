@@ -624,13 +624,13 @@ int wake_adjoint_init(const wake_params *p, int nsteps, int nbins, void *stream,
   a->nbins = nbins;
   a->stream = (cudaStream_t)stream;
   const int n1 = p->nr + 1, np = p->nr * p->ppc;
-  a->g = Dims{p->nr, p->nxi, np, p->rmax / p->nr, p->ximax / p->nxi, p->rmax};
+  a->g = Dims{p->nr, p->nxi, np, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->nr / p->rmax};
   a->B = std::max(1, (int)std::lround(std::sqrt((double)(p->nxi + 1))));
   a->nblk = (p->nxi + 1 + a->B - 1) / a->B;
   a->bc.n = p->n_beam;
   a->bc.n_drive = p->n_drive;
   a->bc.nbins = nbins;
-  a->bc.b = BoundsRZ{p->nr, p->nxi, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->ximax};
+  a->bc.b = BoundsRZ{p->nr, p->nxi, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->ximax, p->nr / p->rmax, p->nxi / p->ximax};
   a->bc.dt = p->ds;
   a->bc.gamma_b = p->gamma_b;
   a->ng = (size_t)(p->nxi + 1) * n1;

@@ -33,6 +33,36 @@ struct Par {
 // v is finite (not NaN or infinite): v - v is 0 exactly then.
 ADJ_HD inline bool finite(double v) { return v - v == 0.0; }
 
+// 1/x, and sqrt(x) with its reciprocal (x > 0).  GB300's FP64 pipe is the adjoint's bound: on the
+// device they are the hardware's approximation (about 20 bits) and one third-order Newton step,
+// with e = 1 - x r:  r (1 + e + e^2), and with e = 1 - x y^2:  y (1 + e/2 + 3 e^2 / 8), the root corrected
+// once; an ulp or so, at a third of the instructions of the IEEE operations.
+ADJ_HD inline double rcp(double x) {
+#ifdef __CUDA_ARCH__
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+#else
+  return 1.0 / x;
+#endif
+}
+ADJ_HD inline void root(double x, double &r, double &ir) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  y = fma(fma(0.375, e, 0.5), e * y, y);
+  const double g = x * y;
+  r = fma(fma(-g, g, x), 0.5 * y, g);
+  ir = y;
+#else
+  r = sqrt(x);
+  ir = 1.0 / r;
+#endif
+}
+constexpr double kTinyR = 1e-145, kTinyR2 = 1e-290;  // smaller radii count as the axis
+
 // A load of a value another CTA may have written in the same launch (the pipelined steps):
 // from L2 on the device (never a stale L1 line), a plain load on the host.
 ADJ_HD inline double rd(const double *p) {
@@ -94,12 +124,22 @@ ADJ_HD void par_scan(const Par &P, int n, bool reverse, In in, Out out) {
 struct Dims {
   int nr, nxi, np;
   double dr, dxi, R;
+  double inv_dr = 0.0;  // 1/dr where the caller has it (0: formed when needed)
+  ADJ_HD double idr() const { return inv_dr > 0.0 ? inv_dr : 1.0 / dr; }
 };
 
 ADJ_HD inline double vol(int i, int nr, double dr) {
   return i == 0 ? dr * dr / 6.0 : (i == nr ? dr * ((double)nr * dr / 2.0 - dr / 6.0) : (double)i * dr * dr);
 }
-ADJ_HD inline double alpha(int m, int nr) { return m == nr ? 1.0 : 0.5 - 1.0 / (6.0 * (double)m); }
+ADJ_HD inline double alpha(int m, int nr) { return m == nr ? 1.0 : 0.5 - rcp(6.0 * (double)m); }
+// The same with 1/dr: on the device the quotient r/dr costs five FP64 instructions.
+ADJ_HD inline void cell_at(double r, double idr, int nr, int &c, double &f) {
+  const double s = r * idr;
+  int i = (int)floor(s);
+  i = i < 0 ? 0 : (i > nr - 1 ? nr - 1 : i);
+  c = i;
+  f = s - (double)i;
+}
 ADJ_HD inline void cell_of(double r, double dr, int nr, int &c, double &f) {
   const double s = r / dr;
   int i = (int)floor(s);
@@ -109,43 +149,109 @@ ADJ_HD inline void cell_of(double r, double dr, int nr, int &c, double &f) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Tridiagonal systems a_q x_{q-1} + b_q x_q + c_q x_{q+1} = d_q (q = 0..n-1, a_0 = c_{n-1} = 0)
-// by parallel cyclic reduction.  Ping-pong between (a, b, c, d) and (a2, b2, c2, d2); x may
-// alias neither.  Ends with a barrier.
+// Tridiagonal systems a_q x_{q-1} + b_q x_q + c_q x_{q+1} = d_q (q = 0..n-1, a_0 = c_{n-1} = 0).
+// Device: one warp; lane l eliminates its E = ceil(n / 32) consecutive rows downwards (into a2: the
+// coupling to the separator before, b2: 1/b, d2) and upwards (its first row), the 32 last rows
+// (separators) are reduced over the lanes by parallel cyclic reduction, and the downward rows give
+// the rest: about a quarter of the operations of a cyclic reduction of all rows and no barriers.
+// Host: Gaussian elimination.  x may alias d but none of the others.  Ends with a barrier.
 // ---------------------------------------------------------------------------------------
-ADJ_HD inline void pcr(const Par &P, int n, double *a, double *b, double *c, double *d, double *a2, double *b2,
-                       double *c2, double *d2, double *x) {
-  double *A = a, *B = b, *C = c, *D = d, *A2 = a2, *B2 = b2, *C2 = c2, *D2 = d2;
-  for (int s = 1; s < n; s <<= 1) {
-    for (int q = P.tid; q < n; q += P.nt) {
-      const int lo = q - s, hi = q + s;
-      double na = 0.0, nb = B[q], nc = 0.0, nd = D[q];
-      if (lo >= 0) {
-        const double k1 = A[q] / B[lo];
-        nb -= k1 * C[lo];
-        nd -= k1 * D[lo];
-        na = -k1 * A[lo];
+ADJ_HD inline void tri_solve(const Par &P, int n, const double *a, const double *b, const double *c, const double *d,
+                             double *a2, double *b2, double *d2, double *x) {
+#ifdef __CUDA_ARCH__
+  if (P.tid < 32) {
+    const unsigned all = 0xffffffffu;
+    const int lane = P.tid, E = (n + 31) >> 5, q0 = lane * E, q1 = q0 + E < n ? q0 + E : n;  // rows q0 .. q1-1
+    // a lane past the rows: the identity
+    double L = 0.0, B = 1.0, C = 0.0, D = 0.0;        // its separator row
+    double ub = 1.0, ua = 0.0, ur = 0.0, ud = 0.0;    // its first row after the upward elimination
+    if (q0 < n) {
+      L = a[q0];
+      B = b[q0];
+      C = c[q0];
+      D = d[q0];
+      double rb = rcp(B);
+      a2[q0] = L;
+      b2[q0] = rb;
+      d2[q0] = D;
+      int u = q1 - 2;  // upwards from the row before the separator
+      double urb = 0.0;
+      if (u >= q0) {
+        ua = a[u];
+        ub = b[u];
+        ur = c[u];
+        ud = d[u];
+        urb = rcp(ub);
       }
-      if (hi < n) {
-        const double k2 = C[q] / B[hi];
-        nb -= k2 * A[hi];
-        nd -= k2 * D[hi];
-        nc = -k2 * C[hi];
+      for (int q = q0 + 1; q < q1; ++q) {
+        const double aq = a[q], k = aq * rb;
+        B = b[q] - k * C;
+        D = d[q] - k * D;
+        L = -k * L;
+        C = c[q];
+        rb = rcp(B);
+        a2[q] = L;
+        b2[q] = rb;
+        d2[q] = D;
+        if (u > q0) {
+          --u;
+          const double ku = c[u] * urb;
+          ub = b[u] - ku * ua;
+          ud = d[u] - ku * ud;
+          ur = -ku * ur;
+          ua = a[u];
+          urb = rcp(ub);
+        }
       }
-      A2[q] = na;
-      B2[q] = nb;
-      C2[q] = nc;
-      D2[q] = nd;
     }
-    P.sync();
-    double *t;
-    t = A; A = A2; A2 = t;
-    t = B; B = B2; B2 = t;
-    t = C; C = C2; C2 = t;
-    t = D; D = D2; D2 = t;
+    // the separator's right neighbour is the next lane's first row, whose unknown is eliminated when
+    // that lane has rows before its separator (else it is that separator itself)
+    const double na = __shfl_down_sync(all, ua, 1), nb = __shfl_down_sync(all, ub, 1), nr = __shfl_down_sync(all, ur, 1),
+                 nd = __shfl_down_sync(all, ud, 1);
+    const int nq0 = q0 + E, nrows = nq0 < n ? (nq0 + E < n ? E : n - nq0) : 0;  // the next lane's rows
+    if (nrows > 1) {
+      const double k = C * rcp(nb);
+      B -= k * na;
+      D -= k * nd;
+      C = -k * nr;
+    }
+    if (lane == 31 || nrows == 0) C = 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double rb = rcp(B);
+      const double am = __shfl_up_sync(all, L, o), cm = __shfl_up_sync(all, C, o), dm = __shfl_up_sync(all, D, o),
+                   rm = __shfl_up_sync(all, rb, o);
+      const double ap = __shfl_down_sync(all, L, o), cp = __shfl_down_sync(all, C, o), dp = __shfl_down_sync(all, D, o),
+                   rp = __shfl_down_sync(all, rb, o);
+      const double k1 = lane >= o ? L * rm : 0.0, k2 = lane + o < 32 ? C * rp : 0.0;
+      B = B - k1 * cm - k2 * ap;
+      D = D - k1 * dm - k2 * dp;
+      L = -k1 * am;
+      C = -k2 * cp;
+    }
+    double z = D * rcp(B);
+    const double up = __shfl_up_sync(all, z, 1), zl = lane == 0 ? 0.0 : up;
+    if (q0 < n) {
+      x[q1 - 1] = z;
+      for (int q = q1 - 2; q >= q0; --q) {
+        z = (d2[q] - a2[q] * zl - c[q] * z) * b2[q];
+        x[q] = z;
+      }
+    }
   }
-  for (int q = P.tid; q < n; q += P.nt) x[q] = D[q] / B[q];
   P.sync();
+#else
+  b2[0] = c[0] / b[0];
+  d2[0] = d[0] / b[0];
+  for (int q = 1; q < n; ++q) {
+    const double m = 1.0 / (b[q] - a[q] * b2[q - 1]);
+    b2[q] = c[q] * m;
+    d2[q] = (d[q] - a[q] * d2[q - 1]) * m;
+  }
+  x[n - 1] = d2[n - 1];
+  for (int q = n - 2; q >= 0; --q) x[q] = d2[q] - b2[q] * x[q + 1];
+  (void)a2;
+#endif
 }
 
 // ---------------------------------------------------------------------------------------
@@ -189,19 +295,19 @@ ADJ_HD inline double interp(const double *v, int c, double f) { return (1.0 - f)
 // differences, a half cell at the wall, B_0 = 0.  Writes ta, tb, tc (tb includes -chi).
 ADJ_HD inline void helmholtz_rows(const Par &P, const Dims &g, const Nodes &S, Work &W) {
   const int nr = g.nr;
-  const double idr2 = 1.0 / (g.dr * g.dr);
+  const double idr2 = g.idr() * g.idr();
   for (int i = 1 + P.tid; i <= nr; i += P.nt) {
     const int q = i - 1;
-    const double rm = i - 0.5;
+    const double im = rcp(i - 0.5);
     if (i < nr) {
-      const double rp = i + 0.5;
-      W.ta[q] = q == 0 ? 0.0 : (i - 1) / rm * idr2;
-      W.tc[q] = (i + 1) / rp * idr2;
-      W.tb[q] = -(double)i * (1.0 / rp + 1.0 / rm) * idr2 - S.chi[i];
+      const double ip = rcp(i + 0.5);
+      W.ta[q] = q == 0 ? 0.0 : (i - 1) * im * idr2;
+      W.tc[q] = (i + 1) * ip * idr2;
+      W.tb[q] = -(double)i * (ip + im) * idr2 - S.chi[i];
     } else {
-      W.ta[q] = q == 0 ? 0.0 : 2.0 * (i - 1) / rm * idr2;
+      W.ta[q] = q == 0 ? 0.0 : 2.0 * (i - 1) * im * idr2;
       W.tc[q] = 0.0;
-      W.tb[q] = -2.0 * (double)i / rm * idr2 - S.chi[i];
+      W.tb[q] = -2.0 * (double)i * im * idr2 - S.chi[i];
     }
   }
 }
@@ -213,13 +319,13 @@ ADJ_HD inline void helmholtz_rows(const Par &P, const Dims &g, const Nodes &S, W
 ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, const double *G0, const double *w,
                                  const double *rho0, const double *nb, Nodes &S, Work &W, double *Fc, int *bad) {
   const int nr = g.nr, n1 = nr + 1, np = g.np;
-  const double dr = g.dr;
+  const double dr = g.dr, idr = g.idr();
   for (int i = P.tid; i < n1; i += P.nt) S.rho[i] = S.jz[i] = S.chi[i] = S.T[i] = S.P[i] = S.U[i] = S.K[i] = 0.0;
   P.sync();
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_of(R.r[j], dr, nr, c, f);
+    cell_at(R.r[j], idr, nr, c, f);
     add_to(&S.rho[c], w[j] * (1.0 - f));
     add_to(&S.rho[c + 1], w[j] * f);
   }
@@ -232,7 +338,7 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
                return;
              }
              const double dl = S.rho[m] - rho0[m];
-             S.dpsi[m] = (incl - dl + alpha(m, nr) * dl) / (m * dr);
+             S.dpsi[m] = (incl - dl + alpha(m, nr) * dl) * rcp(m * dr);
            });
   // psi(R) = 0, inward trapezoid
   par_scan(P, n1, true, [&](int m) { return m < nr ? 0.5 * dr * (S.dpsi[m] + S.dpsi[m + 1]) : 0.0; },
@@ -241,20 +347,21 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
     const double r = R.r[j], ur = R.ur[j], ut = R.ut[j];
     int c;
     double f;
-    cell_of(r, dr, nr, c, f);
+    cell_at(r, idr, nr, c, f);
     const double Gam = G0[j] + interp(S.psi, c, f);
     if (!(Gam > 0.0)) *bad = 1;
     const double up2 = ur * ur + ut * ut;
-    const double gam = (1.0 + up2 + Gam * Gam) / (2.0 * Gam), uz = gam - Gam;
-    const double a = ur / Gam, dp = interp(S.dpsi, c, f);
-    const double cent = r > 0.0 ? ut * ut / (Gam * r) : 0.0;
-    const double F0 = (gam / Gam) * dp + cent;
+    const bool off = r > kTinyR;
+    const double rs = off ? r : 1.0, ig = rcp(Gam * rs), iG = ig * rs;  // 1/Gamma and 1/(Gamma r)
+    const double gam = (1.0 + up2 + Gam * Gam) * 0.5 * iG, uz = gam - Gam;
+    const double a = ur * iG, dp = interp(S.dpsi, c, f);
+    const double cent = off ? ut * ut * ig : 0.0;
+    const double F0 = gam * iG * dp + cent;
     R.Gam[j] = Gam;
     R.gam[j] = gam;
     R.dp[j] = dp;
     const double wj = w[j];
-    const double vjz = -wj * uz / Gam, vchi = wj / Gam, vT = wj * a * a, vP = wj * (a * a * dp - F0) / Gam,
-                 vU = wj * a / Gam;
+    const double vchi = wj * iG, vjz = -uz * vchi, vU = vchi * a, vT = wj * a * a, vP = vchi * (a * a * dp - F0);
     add_to(&S.jz[c], vjz * (1.0 - f));
     add_to(&S.jz[c + 1], vjz * f);
     add_to(&S.chi[c], vchi * (1.0 - f));
@@ -269,16 +376,16 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
   }
   P.sync();
   for (int i = P.tid; i < n1; i += P.nt) {
-    const double V = vol(i, nr, dr);
-    S.jz[i] = S.jz[i] / V - nb[i];
-    S.chi[i] /= V;
-    S.T[i] /= V;
-    S.P[i] /= V;
-    S.U[i] /= V;
+    const double iV = rcp(vol(i, nr, dr));
+    S.jz[i] = S.jz[i] * iV - nb[i];
+    S.chi[i] *= iV;
+    S.T[i] *= iV;
+    S.P[i] *= iV;
+    S.U[i] *= iV;
     double dz = 0.0;
     if (i > 0) {
       const double al = alpha(i, nr), Km = i < nr ? S.K[i] : 0.0;
-      dz = -((1.0 - al) * S.K[i - 1] + al * Km) / dr / (i * dr);
+      dz = -((1.0 - al) * S.K[i - 1] + al * Km) * idr * rcp(i * dr);
     }
     S.dez[i] = dz;
   }
@@ -291,22 +398,21 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
   for (int i = 1 + P.tid; i <= nr; i += P.nt) {
     const int q = i - 1;
     if (i < nr)
-      W.td[q] = (S.jz[i + 1] - S.jz[i - 1]) / (2.0 * dr) + S.Q[i] + (S.T[i + 1] - S.T[i - 1]) / (2.0 * dr) +
-                S.T[i] / (i * dr);
+      W.td[q] = ((S.jz[i + 1] - S.jz[i - 1]) + (S.T[i + 1] - S.T[i - 1])) * 0.5 * idr + S.Q[i] + S.T[i] * rcp(i * dr);
     else
-      W.td[q] = S.Q[i] + (S.T[i] - S.T[i - 1]) / dr + S.T[i] / (i * dr) - (S.jz[i - 1] + S.jz[i]) / dr;
+      W.td[q] = S.Q[i] + (S.T[i] - S.T[i - 1]) * idr + S.T[i] * rcp(i * dr) - (S.jz[i - 1] + S.jz[i]) * idr;
   }
   P.sync();
-  pcr(P, nr, W.ta, W.tb, W.tc, W.td, W.a2, W.b2, W.c2, W.d2, S.bth + 1);
+  tri_solve(P, nr, W.ta, W.tb, W.tc, W.td, W.a2, W.b2, W.d2, S.bth + 1);
   if (P.tid == 0) S.bth[0] = 0.0;
   P.sync();
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_of(R.r[j], dr, nr, c, f);
+    cell_at(R.r[j], idr, nr, c, f);
     const double bf = interp(S.bth, c, f);
     R.bf[j] = bf;
-    Fc[j] = (R.gam[j] / R.Gam[j]) * R.dp[j] - bf;
+    Fc[j] = R.gam[j] * rcp(R.Gam[j]) * R.dp[j] - bf;
   }
   P.sync();
 }
@@ -322,7 +428,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
                                  double *lG0, double *lw, double *lnb, double nb_scale, double *lrho0,
                                  double *lgam_s, double *lGam_s, double *ldp_s) {
   const int nr = g.nr, n1 = nr + 1, np = g.np;
-  const double dr = g.dr;
+  const double dr = g.dr, idr = g.idr();
   for (int i = P.tid; i < n1; i += P.nt) {
     W.l_rho[i] = W.l_dpsi[i] = W.l_psi[i] = W.l_jz[i] = W.l_chi[i] = W.l_T[i] = W.l_P[i] = W.l_U[i] = 0.0;
     W.l_K[i] = W.l_dez[i] = W.l_Q[i] = W.l_td[i] = 0.0;
@@ -340,15 +446,15 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_of(R.r[j], dr, nr, c, f);
-    const double iG = 1.0 / R.Gam[j], gam = R.gam[j], dp = R.dp[j], lFj = lF[j];
+    cell_at(R.r[j], idr, nr, c, f);
+    const double iG = rcp(R.Gam[j]), gam = R.gam[j], dp = R.dp[j], lFj = lF[j];
     lgam_s[j] = lFj * dp * iG;
     lGam_s[j] = lG[j] - lFj * gam * dp * iG * iG;
     ldp_s[j] = lFj * gam * iG;
     const double lbf = -lFj;
     add_to(&W.l_bth[c], lbf * (1.0 - f));
     add_to(&W.l_bth[c + 1], lbf * f);
-    lr[j] += lbf * (S.bth[c + 1] - S.bth[c]) / dr;
+    lr[j] += lbf * (S.bth[c + 1] - S.bth[c]) * idr;
   }
   P.sync();
   // B = A(chi)^-1 td: l_td = A^-T l_B (rows 1..nr), l_chi_i += l_td_q B_i.  A^T has
@@ -361,7 +467,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     W.d2[q] = W.l_bth[q + 1];
   }
   P.sync();
-  pcr(P, nr, W.a2, W.tb, W.c2, W.d2, W.ta, W.b2, W.tc, W.td, W.l_td);
+  tri_solve(P, nr, W.a2, W.tb, W.c2, W.d2, W.ta, W.b2, W.td, W.l_td);
   // td rows -> l_jz, l_Q, l_T; l_chi
   for (int i = 1 + P.tid; i <= nr; i += P.nt) {
     const int q = i - 1;
@@ -369,16 +475,16 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     add_to(&W.l_chi[i], lt * S.bth[i]);
     add_to(&W.l_Q[i], lt);
     if (i < nr) {
-      add_to(&W.l_jz[i + 1], lt / (2.0 * dr));
-      add_to(&W.l_jz[i - 1], -lt / (2.0 * dr));
-      add_to(&W.l_T[i + 1], lt / (2.0 * dr));
-      add_to(&W.l_T[i - 1], -lt / (2.0 * dr));
-      add_to(&W.l_T[i], lt / (i * dr));
+      add_to(&W.l_jz[i + 1], 0.5 * lt * idr);
+      add_to(&W.l_jz[i - 1], -0.5 * lt * idr);
+      add_to(&W.l_T[i + 1], 0.5 * lt * idr);
+      add_to(&W.l_T[i - 1], -0.5 * lt * idr);
+      add_to(&W.l_T[i], lt * rcp(i * dr));
     } else {
-      add_to(&W.l_T[i], lt * (1.0 / dr + 1.0 / (i * dr)));
-      add_to(&W.l_T[i - 1], -lt / dr);
-      add_to(&W.l_jz[i - 1], -lt / dr);
-      add_to(&W.l_jz[i], -lt / dr);
+      add_to(&W.l_T[i], lt * (idr + rcp(i * dr)));
+      add_to(&W.l_T[i - 1], -lt * idr);
+      add_to(&W.l_jz[i - 1], -lt * idr);
+      add_to(&W.l_jz[i], -lt * idr);
     }
   }
   P.sync();
@@ -400,17 +506,17 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   for (int i = P.tid; i < n1; i += P.nt) {
     double lk = 0.0;
     if (i < nr) {
-      lk -= W.l_dez[i + 1] * (1.0 - alpha(i + 1, nr)) / ((i + 1) * dr * dr);
-      if (i > 0) lk -= W.l_dez[i] * alpha(i, nr) / (i * dr * dr);
+      lk -= W.l_dez[i + 1] * (1.0 - alpha(i + 1, nr)) * rcp((i + 1) * dr * dr);
+      if (i > 0) lk -= W.l_dez[i] * alpha(i, nr) * rcp(i * dr * dr);
     }
     W.l_K[i] = lk;
-    const double V = vol(i, nr, dr);
+    const double iV = rcp(vol(i, nr, dr));
     lnb[i] -= nb_scale * W.l_jz[i];
-    W.l_jz[i] /= V;
-    W.l_chi[i] /= V;
-    W.l_T[i] /= V;
-    W.l_P[i] /= V;
-    W.l_U[i] /= V;
+    W.l_jz[i] *= iV;
+    W.l_chi[i] *= iV;
+    W.l_T[i] *= iV;
+    W.l_P[i] *= iV;
+    W.l_U[i] *= iV;
   }
   P.sync();
   // per ring: deposits, F0, gamma/u_z, Gamma = G0 + psi(r)
@@ -418,9 +524,11 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     const double r = R.r[j], ur = R.ur[j], ut = R.ut[j];
     int c;
     double f;
-    cell_of(r, dr, nr, c, f);
+    cell_at(r, idr, nr, c, f);
     const double Gam = R.Gam[j], gam = R.gam[j], dp = R.dp[j], uz = gam - Gam, wj = w[j];
-    const double iG = 1.0 / Gam, iG2 = iG * iG, ir = r > 0.0 ? 1.0 / r : 0.0;
+    const bool off = r > kTinyR;
+    const double rs = off ? r : 1.0, t0 = rcp(Gam * rs);
+    const double iG = t0 * rs, iG2 = iG * iG, ir = off ? t0 * Gam : 0.0;
     const double up2 = ur * ur + ut * ut, a = ur * iG;
     const double cent = ut * ut * iG * ir;
     const double F0 = gam * iG * dp + cent;
@@ -432,7 +540,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
                  lU = W.l_U[c] * g0 + W.l_U[c + 1] * g1, lK = W.l_K[c];
     double lf = vjz * (W.l_jz[c + 1] - W.l_jz[c]) + vchi * (W.l_chi[c + 1] - W.l_chi[c]) +
                 vT * (W.l_T[c + 1] - W.l_T[c]) + vP * (W.l_P[c + 1] - W.l_P[c]) + vU * (W.l_U[c + 1] - W.l_U[c]);
-    double lrj = lf / dr;
+    double lrj = lf * idr;
     lw[j] += (-ljz * uz + lchi + lP * (a * a * dp - F0) + lU * a) * iG + lT * a * a + lK * a;
     double luz = -ljz * wj * iG;
     double lGam = lGam_s[j] + (ljz * wj * uz - lchi * wj - lP * wj * (a * a * dp - F0) - lU * wj * a) * iG2;
@@ -444,7 +552,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     ldp += lF0 * gam * iG;
     const double lcent = lF0;
     double lutj = 0.0;
-    if (r > 0.0) {
+    if (off) {
       lutj += lcent * 2.0 * ut * iG * ir;
       lGam -= lcent * cent * iG;
       lrj -= lcent * cent * ir;
@@ -461,11 +569,11 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     // psi'(r) and psi(r) gathers
     add_to(&W.l_dpsi[c], ldp * g0);
     add_to(&W.l_dpsi[c + 1], ldp * g1);
-    lrj += ldp * (S.dpsi[c + 1] - S.dpsi[c]) / dr;
+    lrj += ldp * (S.dpsi[c + 1] - S.dpsi[c]) * idr;
     lG0[j] += lGam;
     add_to(&W.l_psi[c], lGam * g0);
     add_to(&W.l_psi[c + 1], lGam * g1);
-    lrj += lGam * (S.psi[c + 1] - S.psi[c]) / dr;
+    lrj += lGam * (S.psi[c + 1] - S.psi[c]) * idr;
     lr[j] += lrj;
     lur[j] += lurj;
     lut[j] += lutj;
@@ -478,10 +586,10 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   P.sync();
   // psi'_m = (sum_{i<m} delta_i + alpha_m delta_m) / (m dr):
   // l_delta_i = sum_{m>i} l_psi'_m / (m dr) + [i>0] alpha_i l_psi'_i / (i dr)
-  par_scan(P, n1, true, [&](int m) { return m > 0 ? W.l_dpsi[m] / (m * dr) : 0.0; },
+  par_scan(P, n1, true, [&](int m) { return m > 0 ? W.l_dpsi[m] * rcp(m * dr) : 0.0; },
            [&](int m, double incl) { W.l_td[m] = incl; });
   for (int i = P.tid; i < n1; i += P.nt) {
-    const double own = i > 0 ? W.l_dpsi[i] / (i * dr) : 0.0;
+    const double own = i > 0 ? W.l_dpsi[i] * rcp(i * dr) : 0.0;
     const double ld = (W.l_td[i] - own) + (i > 0 ? alpha(i, nr) * own : 0.0);
     W.l_rho[i] = ld;
     lrho0[i] -= ld;
@@ -490,9 +598,9 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_of(R.r[j], dr, nr, c, f);
+    cell_at(R.r[j], idr, nr, c, f);
     lw[j] += W.l_rho[c] * (1.0 - f) + W.l_rho[c + 1] * f;
-    lr[j] += w[j] * (W.l_rho[c + 1] - W.l_rho[c]) / dr;
+    lr[j] += w[j] * (W.l_rho[c + 1] - W.l_rho[c]) * idr;
   }
   P.sync();
 }
@@ -518,16 +626,20 @@ struct Mid {
 ADJ_HD inline void midpoint(const Par &P, const Dims &g, const Rings &R1, Mid &M, Rings &R2, int *bad) {
   const double h = 0.5 * g.dxi;
   for (int j = P.tid; j < g.np; j += P.nt) {
-    const double xh = R1.r[j] + h * R1.ur[j] / M.G1[j], yh = h * R1.ut[j] / M.G1[j];
+    const double hG = h * rcp(M.G1[j]);
+    const double xh = R1.r[j] + hG * R1.ur[j], yh = hG * R1.ut[j];
     const double uxh = R1.ur[j] + h * M.F1[j], uyh = R1.ut[j];
     M.xh[j] = xh;
     M.yh[j] = yh;
     M.uxh[j] = uxh;
     M.uyh[j] = uyh;
-    double rr = sqrt(xh * xh + yh * yh), urr, utt;
-    if (rr > 0.0) {
-      urr = (xh * uxh + yh * uyh) / rr;
-      utt = (xh * uyh - yh * uxh) / rr;
+    const double h2 = xh * xh + yh * yh;
+    double rr = 0.0, urr, utt;
+    if (h2 > kTinyR2) {
+      double irr;
+      root(h2, rr, irr);
+      urr = (xh * uxh + yh * uyh) * irr;
+      utt = (xh * uyh - yh * uxh) * irr;
     } else {
       urr = sqrt(uxh * uxh + uyh * uyh);
       utt = 0.0;
@@ -553,16 +665,26 @@ ADJ_HD inline void full_step(const Par &P, const Dims &g, const Rings &R1, const
   const double dxi = g.dxi;
   for (int j = P.tid; j < g.np; j += P.nt) {
     const double xh = M.xh[j], yh = M.yh[j];
-    const double rr = sqrt(xh * xh + yh * yh);
-    double ex = 1.0, ey = 0.0;
-    if (rr > 0.0) {
-      ex = xh / rr;
-      ey = yh / rr;
+    const double h2 = xh * xh + yh * yh;
+    double ex = 1.0, ey = 0.0, irr = 0.0;
+    if (h2 > kTinyR2) {
+      double rr;
+      root(h2, rr, irr);
+      ex = xh * irr;
+      ey = yh * irr;
     }
-    const double xn = R1.r[j] + dxi * M.uxh[j] / M.G2[j], yn = dxi * M.uyh[j] / M.G2[j];
+    const double hG = dxi * rcp(M.G2[j]);
+    const double xn = R1.r[j] + hG * M.uxh[j], yn = hG * M.uyh[j];
     const double uxn = R1.ur[j] + dxi * M.F2[j] * ex, uyn = R1.ut[j] + dxi * M.F2[j] * ey;
-    double r2 = sqrt(xn * xn + yn * yn);
-    double u2 = r2 > 0.0 ? (xn * uxn + yn * uyn) / r2 : sqrt(uxn * uxn + uyn * uyn);
+    const double n2 = xn * xn + yn * yn;
+    double r2 = 0.0, u2;
+    if (n2 > kTinyR2) {
+      double ir2;
+      root(n2, r2, ir2);
+      u2 = (xn * uxn + yn * uyn) * ir2;
+    } else {
+      u2 = sqrt(uxn * uxn + uyn * uyn);
+    }
     if (r2 > g.R) {
       r2 = 2.0 * g.R - r2;
       u2 = -u2;
@@ -582,16 +704,19 @@ ADJ_HD inline void full_step_reverse(const Par &P, const Dims &g, const Rings &R
   const double dxi = g.dxi;
   for (int j = P.tid; j < g.np; j += P.nt) {
     const double xh = M.xh[j], yh = M.yh[j], G2 = M.G2[j], F2 = M.F2[j], uxh = M.uxh[j], uyh = M.uyh[j];
-    const double rr = sqrt(xh * xh + yh * yh);
-    double ex = 1.0, ey = 0.0;
-    if (rr > 0.0) {
-      ex = xh / rr;
-      ey = yh / rr;
+    const double h2 = xh * xh + yh * yh;
+    double ex = 1.0, ey = 0.0, irr = 0.0;
+    if (h2 > kTinyR2) {
+      double rr;
+      root(h2, rr, irr);
+      ex = xh * irr;
+      ey = yh * irr;
     }
-    const double iG2 = 1.0 / G2;
+    const double iG2 = rcp(G2);
     const double xn = R1.r[j] + dxi * uxh * iG2, yn = dxi * uyh * iG2;
     const double uxn = R1.ur[j] + dxi * F2 * ex, uyn = R1.ut[j] + dxi * F2 * ey;
-    const double r2 = sqrt(xn * xn + yn * yn), ir2 = 1.0 / r2;
+    double r2, ir2;
+    root(xn * xn + yn * yn, r2, ir2);
     const double u2 = (xn * uxn + yn * uyn) * ir2;
     double lr2 = lrn[j], lu2 = lurn[j];
     if (r2 > g.R) {
@@ -609,8 +734,8 @@ ADJ_HD inline void full_step_reverse(const Par &P, const Dims &g, const Rings &R
     double lux = lxn * dxi * iG2, luy = lyn * dxi * iG2;
     double lG = -(lxn * uxh + lyn * uyh) * dxi * iG2 * iG2;
     double lx = 0.0, ly = 0.0;
-    if (rr > 0.0) {
-      const double irr = 1.0 / rr, ir3 = irr * irr * irr;
+    if (irr > 0.0) {
+      const double ir3 = irr * irr * irr;
       lx = lex * (irr - xh * xh * ir3) - ley * yh * xh * ir3;
       ly = -lex * xh * yh * ir3 + ley * (irr - yh * yh * ir3);
     }
@@ -633,7 +758,7 @@ ADJ_HD inline void midpoint_reverse(const Par &P, const Dims &g, const Rings &R1
   const double h = 0.5 * g.dxi;
   for (int j = P.tid; j < g.np; j += P.nt) {
     const double xh = M.xh[j], yh = M.yh[j], uxh = M.uxh[j], uyh = M.uyh[j];
-    const double rr = sqrt(xh * xh + yh * yh);
+    const double h2 = xh * xh + yh * yh;
     double lrr = lr2[j], lurr = lur2[j];
     const double lutt = lut2[j];
     if (M.reflh[j] != 0.0) {
@@ -641,15 +766,16 @@ ADJ_HD inline void midpoint_reverse(const Par &P, const Dims &g, const Rings &R1
       lurr = -lurr;
     }
     double lxh = lxh0[j], lyh = lyh0[j], luxh = luxh0[j], luyh = luyh0[j];
-    if (rr > 0.0) {
-      const double irr = 1.0 / rr;
+    if (h2 > kTinyR2) {
+      double rr, irr;
+      root(h2, rr, irr);
       const double urr = (xh * uxh + yh * uyh) * irr, utt = (xh * uyh - yh * uxh) * irr;
       lxh += (lrr * xh + lurr * (uxh - urr * xh * irr) + lutt * (uyh - utt * xh * irr)) * irr;
       lyh += (lrr * yh + lurr * (uyh - urr * yh * irr) + lutt * (-uxh - utt * yh * irr)) * irr;
       luxh += (lurr * xh - lutt * yh) * irr;
       luyh += (lurr * yh + lutt * xh) * irr;
     }
-    const double iG1 = 1.0 / M.G1[j], ur = R1.ur[j], ut = R1.ut[j];
+    const double iG1 = rcp(M.G1[j]), ur = R1.ur[j], ut = R1.ut[j];
     lr[j] += lxh;
     lur[j] += lxh * h * iG1 + luxh;
     lut[j] += lyh * h * iG1 + luyh;
@@ -666,34 +792,41 @@ ADJ_HD inline void midpoint_reverse(const Par &P, const Dims &g, const Rings &R1
 struct BoundsRZ {
   int nr, nxi;
   double dr, dxi, rmax, ximax;
+  double inv_dr = 0.0, inv_dxi = 0.0;  // as Dims::inv_dr
+  ADJ_HD double idr() const { return inv_dr > 0.0 ? inv_dr : 1.0 / dr; }
+  ADJ_HD double idxi() const { return inv_dxi > 0.0 ? inv_dxi : 1.0 / dxi; }
 };
 
 // Bilinear node weights of a point: cell (c, k), offsets (f, g).
 ADJ_HD inline void cell_rz(const BoundsRZ &b, double r, double xi, int &c, double &f, int &k, double &gg) {
-  cell_of(r, b.dr, b.nr, c, f);
-  cell_of(xi, b.dxi, b.nxi, k, gg);
+  cell_at(r, b.idr(), b.nr, c, f);
+  cell_at(xi, b.idxi(), b.nxi, k, gg);
 }
 
 // Boris step with the fields (Er, Ez, Bt) at the particle.  In/out: x, y, ux, uy, uz, xi.
 ADJ_HD inline void boris(double &x, double &y, double &ux, double &uy, double &uz, double &xi, double Er, double Ez,
                          double Bt, double dt) {
   const double h = -0.5 * dt;
-  const double r = sqrt(x * x + y * y);
-  const double cs = r > 0.0 ? x / r : 0.0, sn = r > 0.0 ? y / r : 0.0;
+  const double r2 = x * x + y * y;
+  double r = 0.0, ir = 0.0;
+  if (r2 > kTinyR2) root(r2, r, ir);
+  const double cs = x * ir, sn = y * ir;
   const double Ex = Er * cs, Ey = Er * sn, Bx = -Bt * sn, By = Bt * cs;
   const double mx = ux + h * Ex, my = uy + h * Ey, mz = uz + h * Ez;
-  const double gm = sqrt(1.0 + mx * mx + my * my + mz * mz);
-  const double tx = h * Bx / gm, ty = h * By / gm;
+  double gm, igm;
+  root(1.0 + mx * mx + my * my + mz * mz, gm, igm);
+  const double tx = h * Bx * igm, ty = h * By * igm;
   const double px = mx - mz * ty, py = my + mz * tx, pz = mz + (mx * ty - my * tx);
-  const double s = 2.0 / (1.0 + tx * tx + ty * ty);
+  const double s = 2.0 * rcp(1.0 + tx * tx + ty * ty);
   const double sx = s * tx, sy = s * ty;
   const double uxn = mx - pz * sy + h * Ex, uyn = my + pz * sx + h * Ey;
   const double uzn = uz + (2.0 * h * Ez + (px * sy - py * sx));
   const double up2 = uxn * uxn + uyn * uyn;
-  const double gam = sqrt(1.0 + up2 + uzn * uzn);
-  x += dt * uxn / gam;
-  y += dt * uyn / gam;
-  xi += dt * (1.0 + up2) / (gam * (gam + uzn));
+  double gam, igam;
+  root(1.0 + up2 + uzn * uzn, gam, igam);
+  x += dt * uxn * igam;
+  y += dt * uyn * igam;
+  xi += dt * (1.0 + up2) * igam * rcp(gam + uzn);
   ux = uxn;
   uy = uyn;
   uz = uzn;
@@ -706,35 +839,40 @@ ADJ_HD inline void boris_reverse(double x, double y, double ux, double uy, doubl
                                  double Bt, double dt, double &lx, double &ly, double &lux, double &luy,
                                  double &luz, double &lxi, double &lEr, double &lEz, double &lBt) {
   const double h = -0.5 * dt;
-  const double r = sqrt(x * x + y * y);
-  const double cs = r > 0.0 ? x / r : 0.0, sn = r > 0.0 ? y / r : 0.0;
+  const double r2 = x * x + y * y;
+  double r = 0.0, ir = 0.0;
+  if (r2 > kTinyR2) root(r2, r, ir);
+  const double cs = x * ir, sn = y * ir;
   const double Ex = Er * cs, Ey = Er * sn, Bx = -Bt * sn, By = Bt * cs;
   const double mx = ux + h * Ex, my = uy + h * Ey, mz = uz + h * Ez;
-  const double gm2 = 1.0 + mx * mx + my * my + mz * mz, gm = sqrt(gm2);
-  const double tx = h * Bx / gm, ty = h * By / gm;
+  double gm, igm;
+  root(1.0 + mx * mx + my * my + mz * mz, gm, igm);
+  const double tx = h * Bx * igm, ty = h * By * igm;
   const double px = mx - mz * ty, py = my + mz * tx, pz = mz + (mx * ty - my * tx);
-  const double den = 1.0 + tx * tx + ty * ty, s = 2.0 / den;
+  const double s = 2.0 * rcp(1.0 + tx * tx + ty * ty);
   const double sx = s * tx, sy = s * ty;
   const double uxn = mx - pz * sy + h * Ex, uyn = my + pz * sx + h * Ey;
   const double uzn = uz + (2.0 * h * Ez + (px * sy - py * sx));
   const double up2 = uxn * uxn + uyn * uyn;
-  const double gam2 = 1.0 + up2 + uzn * uzn, gam = sqrt(gam2);
+  double gam, igam;
+  root(1.0 + up2 + uzn * uzn, gam, igam);
   // xi' = xi + dt (1 + up2) / (gam (gam + uzn)), x' = x + dt uxn / gam, y' = y + dt uyn / gam
-  const double D = gam * (gam + uzn), Nn = 1.0 + up2;
+  const double iD = igam * rcp(gam + uzn), Nn = 1.0 + up2;
   double luxn = lux, luyn = luy, luzn = luz;  // adjoints of the new momenta
   double lgam = 0.0, lup2 = 0.0;
   // xi
-  lup2 += lxi * dt / D;
-  const double lD = -lxi * dt * Nn / (D * D);
+  lup2 += lxi * dt * iD;
+  const double lD = -lxi * dt * Nn * iD * iD;
   lgam += lD * (2.0 * gam + uzn);
   luzn += lD * gam;
   // x, y
-  luxn += lx * dt / gam;
-  luyn += ly * dt / gam;
-  lgam += -lx * dt * uxn / (gam * gam) - ly * dt * uyn / (gam * gam);
+  const double dg = dt * igam;
+  luxn += lx * dg;
+  luyn += ly * dg;
+  lgam += -(lx * uxn + ly * uyn) * dg * igam;
   // gam = sqrt(1 + up2 + uzn^2)
-  lup2 += lgam / (2.0 * gam);
-  luzn += lgam * uzn / gam;
+  lup2 += 0.5 * lgam * igam;
+  luzn += lgam * uzn * igam;
   luxn += lup2 * 2.0 * uxn;
   luyn += lup2 * 2.0 * uyn;
   // uzn = uz + 2 h Ez + px sy - py sx
@@ -747,7 +885,7 @@ ADJ_HD inline void boris_reverse(double x, double y, double ux, double uy, doubl
   // sx = s tx, sy = s ty, s = 2 / den
   double ltx = lsx * s, lty = lsy * s;
   const double ls = lsx * tx + lsy * ty;
-  const double lden = -ls * 2.0 / (den * den);
+  const double lden = -0.5 * ls * s * s;  // ds/dden = -2/den^2 = -s^2/2
   ltx += lden * 2.0 * tx;
   lty += lden * 2.0 * ty;
   // pz = mz + mx ty - my tx; py = my + mz tx; px = mx - mz ty
@@ -757,12 +895,13 @@ ADJ_HD inline void boris_reverse(double x, double y, double ux, double uy, doubl
   lty += lpz * mx - lpx * mz;
   ltx += -lpz * my + lpy * mz;
   // tx = h Bx / gm, ty = h By / gm
-  double lBx = ltx * h / gm, lBy = lty * h / gm;
-  const double lgm = -ltx * h * Bx / gm2 - lty * h * By / gm2;
+  double lBx = ltx * h * igm, lBy = lty * h * igm;
+  const double lgm = -(ltx * tx + lty * ty) * igm;
   // gm = sqrt(1 + mx^2 + my^2 + mz^2)
-  lmx += lgm * mx / gm;
-  lmy += lgm * my / gm;
-  lmz += lgm * mz / gm;
+  const double lgi = lgm * igm;
+  lmx += lgi * mx;
+  lmy += lgi * my;
+  lmz += lgi * mz;
   // mx = ux + h Ex, my = uy + h Ey, mz = uz + h Ez
   lux = lmx;
   luy = lmy;
@@ -775,10 +914,9 @@ ADJ_HD inline void boris_reverse(double x, double y, double ux, double uy, doubl
   lBt = -lBx * sn + lBy * cs;
   lEz = lEz_;
   const double lcs = lEx * Er + lBy * Bt, lsn = lEy * Er - lBx * Bt;
-  if (r > 0.0) {
-    const double r3 = r * r * r;
-    lx += lcs * (1.0 / r - x * x / r3) - lsn * x * y / r3;
-    ly += -lcs * x * y / r3 + lsn * (1.0 / r - y * y / r3);
+  if (ir > 0.0) {
+    lx += (lcs * (1.0 - cs * cs) - lsn * cs * sn) * ir;
+    ly += (-lcs * cs * sn + lsn * (1.0 - sn * sn)) * ir;
   }
   // lxi unchanged: the step adds to xi
 }
@@ -860,7 +998,7 @@ ADJ_HD inline bool march_slices(const Par &P, const MarchArgs &a, Work &W, int k
         ck[np + j] = T.R1.ur[j];
       }
     }
-    for (int j = P.tid; j < np; j += P.nt) T.R1.ut[j] = T.R1.r[j] > 0.0 ? a.l[j] / T.R1.r[j] : 0.0;
+    for (int j = P.tid; j < np; j += P.nt) T.R1.ut[j] = T.R1.r[j] > kTinyR ? a.l[j] * rcp(T.R1.r[j]) : 0.0;
     P.sync();
     stage_forward(P, g, T.R1, a.G0, a.w, a.rho0, a.nb + (size_t)k * n1, T.S1, W, T.M.F1, bad);
     for (int j = P.tid; j < np; j += P.nt) T.M.G1[j] = T.R1.Gam[j];
@@ -1001,9 +1139,10 @@ ADJ_HD inline bool march_reverse_body(const Par &P, const MarchArgs &a, Work &W,
       for (int j = P.tid; j < np; j += P.nt) {
         const double r = T.R1.r[j], lut = L[LR_LUT][j];
         double lr = L[LR_LR][j];
-        if (r > 0.0) {
-          a.ll[j] += lut / r;
-          lr -= lut * a.l[j] / (r * r);
+        if (r > kTinyR) {
+          const double ir = rcp(r), q = lut * ir;
+          a.ll[j] += q;
+          lr -= q * a.l[j] * ir;
         }
         L[LR_LRN][j] = lr;
         L[LR_LURN][j] = L[LR_LUR][j];
@@ -1091,7 +1230,7 @@ ADJ_HD inline void deposit_one(const BeamConst &c, const Beam &s, const double *
 // 1 / (hat volume) of node (k, i): V_i in r, dxi in xi (dxi/2 at both ends).
 ADJ_HD inline double node_scale(const BoundsRZ &b, int k, int i) {
   const double vx = (k == 0 || k == b.nxi) ? 0.5 * b.dxi : b.dxi;
-  return 1.0 / (vol(i, b.nr, b.dr) * vx);
+  return rcp(vol(i, b.nr, b.dr) * vx);
 }
 
 ADJ_HD inline void gather3(const BoundsRZ &b, const double *er, const double *ez, const double *bt, int c, double f,
@@ -1197,11 +1336,12 @@ ADJ_HD inline void push_reverse_one(const BeamConst &c, const Beam &s0, const do
     lf += ls[q] * ((1.0 - gx) * (v[i0 + 1] - v[i0]) + gx * (v[i0 + n1 + 1] - v[i0 + n1]));
     lg += ls[q] * ((1.0 - f) * (v[i0 + n1] - v[i0]) + f * (v[i0 + n1 + 1] - v[i0 + 1]));
   }
-  if (r > 0.0) {
-    lx += lf / c.b.dr * x / r;
-    ly += lf / c.b.dr * y / r;
+  if (r > kTinyR) {
+    const double q = lf * c.b.idr() * rcp(r);
+    lx += q * x;
+    ly += q * y;
   }
-  lxi += lg / c.b.dxi;
+  lxi += lg * c.b.idxi();
   lam.x[j] = lx;
   lam.y[j] = ly;
   lam.ux[j] = lux;
@@ -1227,11 +1367,12 @@ ADJ_HD inline void deposit_reverse_one(const BeamConst &c, const Beam &s, const 
   lw[j] = rd(lw + j) + (L00 * (1.0 - f) * (1.0 - gx) + L01 * f * (1.0 - gx) + L10 * (1.0 - f) * gx + L11 * f * gx);
   const double lf = w * ((1.0 - gx) * (L01 - L00) + gx * (L11 - L10));
   const double lg = w * ((1.0 - f) * (L10 - L00) + f * (L11 - L01));
-  if (r > 0.0) {
-    lam.x[j] = rd(lam.x + j) + lf / c.b.dr * x / r;
-    lam.y[j] = rd(lam.y + j) + lf / c.b.dr * y / r;
+  if (r > kTinyR) {
+    const double q = lf * c.b.idr() * rcp(r);
+    lam.x[j] = rd(lam.x + j) + q * x;
+    lam.y[j] = rd(lam.y + j) + q * y;
   }
-  lam.xi[j] = rd(lam.xi + j) + lg / c.b.dxi;
+  lam.xi[j] = rd(lam.xi + j) + lg * c.b.idxi();
 }
 
 // deposit_one with the division by the hats' volumes folded in (node_scale per node): the
