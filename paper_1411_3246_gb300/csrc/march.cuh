@@ -138,31 +138,6 @@ __device__ __forceinline__ void rcp_pair(double a, double b, double &ia, double 
   ib = t * a;
 }
 
-// exclusive prefix over the lanes of one warp of per-lane totals (lane 0 gets 0)
-template <class W>
-__device__ __forceinline__ W warp_excl_prefix(W v, int lane) {
-  W incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const W t = wide_shfl_up(incl, o);
-    if (lane >= o) incl = wide_add(incl, t);
-  }
-  const W ex = wide_shfl_up(incl, 1);
-  return lane == 0 ? wide_zero<W>() : ex;
-}
-// exclusive suffix over the lanes of one warp (lane 31 gets 0)
-template <class W>
-__device__ __forceinline__ W warp_excl_suffix(W v, int lane) {
-  W incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const W t = wide_shfl_down(incl, o);
-    if (lane + o < 32) incl = wide_add(incl, t);
-  }
-  const W ex = wide_shfl_down(incl, 1);
-  return lane == 31 ? wide_zero<W>() : ex;
-}
-
 // ---------------------------------------------------------------------------------------
 // thread-block clusters: one simulation marched by several CTAs (Hooks::kCluster).  Each CTA
 // holds a share of the rings and deposits them into its own node arrays; the arrays are summed
@@ -762,7 +737,7 @@ __device__ __forceinline__ void solve_psi(MarchSmem<Pol> &sm, const NodeGeo<Pol>
       [&](int m, W incl) { sm.psi[m] = -(R)wide_value(incl); });
 }
 
-// E_z, the Helmholtz system for B_theta and its PCR solve, from the current-type deposits
+// E_z, the Helmholtz system for B_theta and its solve, from the current-type deposits
 // and the beam-density rows nbA, nbB (averaged).  Ends with a barrier.
 template <class Pol, int NT>
 __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<Pol> &geo, const typename Pol::R *nbA,

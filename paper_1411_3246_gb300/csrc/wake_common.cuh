@@ -77,79 +77,4 @@ __host__ __device__ __forceinline__ double nb_eq12(double r, double xi, double n
 
 __device__ __forceinline__ void flag(int *status, int bit) { atomicOr(status, bit); }
 
-// Block-wide in-place inclusive scan of a[0..n-1] (suffix scan if reverse), n arbitrary:
-// each thread sums a contiguous chunk, warps scan the chunk sums with shuffles, warp 0
-// scans the warp totals.  Ends with a barrier; wtot needs NT/32 doubles.
-template <int NT>
-__device__ __forceinline__ void block_scan(double *a, int n, double *wtot, bool reverse) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int E = (n + NT - 1) / NT;
-  const int beg = tid * E, end = min(n, beg + E);
-  double s = 0.0;
-  for (int q = beg; q < end; ++q) s += a[reverse ? n - 1 - q : q];
-  double incl = s;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const double t = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += t;
-  }
-  if (lane == 31) wtot[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    double t = lane < NT / 32 ? wtot[lane] : 0.0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double u = __shfl_up_sync(kFull, t, o);
-      if (lane >= o) t += u;
-    }
-    if (lane < NT / 32) wtot[lane] = t;
-  }
-  __syncthreads();
-  double run = incl - s + (warp > 0 ? wtot[warp - 1] : 0.0);
-  for (int q = beg; q < end; ++q) {
-    const int i = reverse ? n - 1 - q : q;
-    run += a[i];
-    a[i] = run;
-  }
-  __syncthreads();
-}
-
-// Parallel cyclic reduction (Hockney) for a tridiagonal system of n rows:
-//   a_q x_{q-1} + b_q x_q + c_q x_{q+1} = d_q,  a_0 = c_{n-1} = 0.
-// Each step eliminates the couplings at distance s and doubles s; after ceil(log2 n) steps
-// every row is decoupled and x_q = d_q / b_q.  Arrays are double-buffered (A -> B -> A ...);
-// returns which buffer holds the result (0 = first).  Ends with a barrier.
-template <int NT, class S>
-__device__ __forceinline__ int pcr_solve(S *a0, S *b0, S *c0, S *d0, S *a1, S *b1, S *c1, S *d1,
-                                         int n) {
-  int cur = 0;
-  for (int s = 1; s < n; s <<= 1) {
-    S *a = cur ? a1 : a0, *b = cur ? b1 : b0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
-    S *an = cur ? a0 : a1, *bn = cur ? b0 : b1, *cn = cur ? c0 : c1, *dn = cur ? d0 : d1;
-    for (int q = threadIdx.x; q < n; q += NT) {
-      S aq = a[q], bq = b[q], cq = c[q], dq = d[q];
-      S na = (S)0, nc = (S)0;
-      if (q - s >= 0) {
-        const S k1 = aq / b[q - s];
-        bq -= c[q - s] * k1;
-        dq -= d[q - s] * k1;
-        na = -a[q - s] * k1;
-      }
-      if (q + s < n) {
-        const S k2 = cq / b[q + s];
-        bq -= a[q + s] * k2;
-        dq -= d[q + s] * k2;
-        nc = -c[q + s] * k2;
-      }
-      an[q] = na;
-      bn[q] = bq;
-      cn[q] = nc;
-      dn[q] = dq;
-    }
-    __syncthreads();
-    cur ^= 1;
-  }
-  return cur;
-}
-
 }  // namespace wake
