@@ -250,6 +250,51 @@ __global__ void beam_deposit_kernel(BeamDesc b) {
   deposit_range<BT, G>(b, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
+// Beam density by cells (pipeline.cuh, PipeArgs::corners): node (row, m) is the sum of the shares that
+// the up to four cells around it hold for it.
+__device__ __forceinline__ float corner_node(const float4 *g, int row, int m, int nr, int nxi) {
+  const float *p = (const float *)(g + (size_t)row * nr + m);
+  float v = 0.f;
+  if (row < nxi) {
+    if (m < nr) v += __ldcg(p);
+    if (m > 0) v += __ldcg(p - 4 + 1);
+  }
+  if (row > 0) {
+    const float *q = p - 4 * (size_t)nr;
+    if (m < nr) v += __ldcg(q + 2);
+    if (m > 0) v += __ldcg(q - 4 + 3);
+  }
+  return v;
+}
+static __global__ void nb_from_corners_kernel(const float4 *__restrict__ g, float *__restrict__ nb, int nr, int nxi) {
+  const int n1 = nr + 1;
+  const int64_t tot = (int64_t)(nxi + 1) * n1;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x)
+    nb[t] = corner_node(g, (int)(t / n1), (int)(t % n1), nr, nxi);
+}
+// The deposit of a launch's first step in that layout, divided by the hats' volumes.
+static __global__ void beam_deposit_corners_kernel(BeamDesc b, float4 *g) {
+  using W = BeamWide<float>;
+  const float inv_dr = (float)(1.0 / b.dr), wf = (float)(b.slab ? 1.0 / (b.dr * b.dxi) : 1.0 / (b.dr * b.dr * b.dxi));
+  const W::Box bx = W::box(b.dxi, b.ximax, b.ffi, b.ffx);
+  const int nr = b.nr;
+  auto iv = [&](int i) -> float {  // 1 / V_i in units of 1 / dr^2 (slab 1 / dx)
+    if (b.slab) return (i == 0 || i == nr) ? 2.f : 1.f;
+    return i == 0 ? 6.f : (i == nr ? 1.f / (0.5f * nr - (float)(1.0 / 6.0)) : 1.f / (float)i);
+  };
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < b.n_cap; j += (int64_t)gridDim.x * blockDim.x) {
+    if (b.lost[j] & 1) continue;
+    const float x = ((const float *)b.x)[j], y = ((const float *)b.y)[j], w = wf * ((const float *)b.w)[j];
+    int c, k;
+    float f, q;
+    locate(sqrtf(x * x + y * y), inv_dr, nr, c, f);
+    W::cell(W::ld(b.xi, j), bx, b.nxi, k, q);
+    const float a0 = w * iv(c) * (1.f - f), a1 = w * iv(c + 1) * f;
+    const float q0 = (1.f - q) * (k == 0 ? 2.f : 1.f), q1 = q * (k + 1 == b.nxi ? 2.f : 1.f);
+    atomicAdd(g + (size_t)k * nr + c, make_float4(a0 * q0, a1 * q0, a0 * q1, a1 * q1));
+  }
+}
+
 // Divide the raw deposit by the hats' volumes: V_i in r, dxi in xi (dxi/2 at both ends).
 template <class G>
 __device__ __forceinline__ void normalize_range(G *nb, int nr, int nxi, double dr, double dxi, int slab, int64_t t0,

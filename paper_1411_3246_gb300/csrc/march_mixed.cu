@@ -25,9 +25,9 @@ bool march_tile_mixed512(int nt, int ppt, TileFns *out, bool slab) {
   }
 }
 
-template <class P, int PPT>
+template <class P, int PPT, bool kCorn = false>
 static cudaError_t go_step(const PipeArgs &a, int ctas, cudaStream_t stream) {
-  auto kern = step_kernel<P, PolMixed::NT, PPT>;
+  auto kern = step_kernel<P, PolMixed::NT, PPT, kCorn>;
   const size_t smem = step_smem_bytes<PolMixed, PolMixed::NT, PPT>(a.d.nr + 1);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -68,6 +68,15 @@ cudaError_t launch_step_mixed(const PipeArgs &a, int np, int ctas, cudaStream_t 
       case 2: return go_step<SlabOf<PolMixed>, 2>(a, ctas, stream);
       case 4: return go_step<SlabOf<PolMixed>, 4>(a, ctas, stream);
       case 8: return go_step<SlabOf<PolMixed>, 8>(a, ctas, stream);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  if (a.corners) {
+    switch (ppt_for(np)) {
+      case 1: return go_step<PolMixed, 1, true>(a, ctas, stream);
+      case 2: return go_step<PolMixed, 2, true>(a, ctas, stream);
+      case 4: return go_step<PolMixed, 4, true>(a, ctas, stream);
+      case 8: return go_step<PolMixed, 8, true>(a, ctas, stream);
       default: return cudaErrorInvalidValue;
     }
   }

@@ -29,7 +29,10 @@ constexpr int ST_LISTFULL = 16;  // more slipped particles than a step's lists h
 struct PipeArgs {
   SimDesc d;              // the simulation (plasma, output grids, status)
   void *grids;            // nsteps + 1 beam-density grids (G), grid t at t * ng
-  size_t ng;              // nodes per grid
+  size_t ng;              // nodes per grid (corners: cells per grid)
+  int corners;            // mixed form, one CTA per step, cylinder: the grids hold, per cell (k, c), the four corner shares of the
+                          // particles in it (float4: nodes (k,c), (k,c+1), (k+1,c), (k+1,c+1)), so a
+                          // particle is deposited by one 16-byte atomic instead of four
   int *progress;          // nsteps counters: sorted cells pushed by step t
   int nsteps;
   int write_last;         // write the last step's fields to the output grids
@@ -84,7 +87,9 @@ __device__ __forceinline__ void red_release(int *p) {
 // window and pushes its share of each cell.  progress[t] then counts the CTAs' finished cells: no
 // CTA finishes cell b + 1 before all have finished cell b (cluster barriers lie between), so a count
 // of cn (b + 1) means that all have finished cell b.
-template <class Pol, int NT, bool kCl = false>
+// kCorn: the density grids are kept by cells (PipeArgs::corners); a kernel of its own, since the test
+// alone, never taken, cost the 200-step blowout run 1.5%.
+template <class Pol, int NT, bool kCl = false, bool kCorn = false>
 struct PipeHooks {
   using R = typename Pol::R;
   using G = typename Pol::G;
@@ -150,7 +155,10 @@ struct PipeHooks {
       ctl[4] = __ldcg(a.defer_cnt + 2 * t + 1);
     }
   }
-  __device__ __forceinline__ R nb_row(int row, int m) const { return (R)__ldcg(grid(t) + (size_t)row * n1 + m); }
+  __device__ __forceinline__ R nb_row(int row, int m) const {
+    if constexpr (kCorn) return corner_node((const float4 *)a.grids + (size_t)t * a.ng, row, m, nr, nxi);
+    return (R)__ldcg(grid(t) + (size_t)row * n1 + m);
+  }
 
   __device__ __forceinline__ void slice_done(int k, MarchSmem<Pol> &sm) {
     R *w = win + (size_t)(k & 3) * 3 * n1;
@@ -246,11 +254,16 @@ struct PipeHooks {
     const BT ix0 = k2 == 0 ? (BT)2 : (BT)1, ix1 = k2 + 1 == nxi ? (BT)2 : (BT)1;
     const BT v0 = iv(c2), v1 = iv(c2 + 1);
     const BT s00 = wq * v0 * ix0, s01 = wq * v1 * ix0, s10 = wq * v0 * ix1, s11 = wq * v1 * ix1;
-    G *row = nbn + (size_t)k2 * n1 + c2;
-    atomicAdd(row, (G)(s00 * ((BT)1 - f2) * ((BT)1 - g2)));
-    atomicAdd(row + 1, (G)(s01 * f2 * ((BT)1 - g2)));
-    atomicAdd(row + n1, (G)(s10 * ((BT)1 - f2) * g2));
-    atomicAdd(row + n1 + 1, (G)(s11 * f2 * g2));
+    if constexpr (kCorn) {
+      atomicAdd((float4 *)a.grids + (size_t)(t + 1) * a.ng + (size_t)k2 * nr + c2,
+                make_float4(s00 * (1.f - f2) * (1.f - g2), s01 * f2 * (1.f - g2), s10 * (1.f - f2) * g2, s11 * f2 * g2));
+    } else {
+      G *row = nbn + (size_t)k2 * n1 + c2;
+      atomicAdd(row, (G)(s00 * ((BT)1 - f2) * ((BT)1 - g2)));
+      atomicAdd(row + 1, (G)(s01 * f2 * ((BT)1 - g2)));
+      atomicAdd(row + n1, (G)(s10 * ((BT)1 - f2) * g2));
+      atomicAdd(row + n1 + 1, (G)(s11 * f2 * g2));
+    }
   }
 
   // List particle j (state p), met while cell b is pushed, for the push of cell tgt > b.  A
@@ -348,7 +361,7 @@ struct PipeHooks {
   }
 };
 
-template <class Pol, int NT, int PPT>
+template <class Pol, int NT, int PPT, bool kCorn = false>
 __global__ void __launch_bounds__(NT, 1) step_kernel(PipeArgs a) {
   using R = typename Pol::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -371,7 +384,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(PipeArgs a) {
       ctl[3] = 0;
     }
     __syncthreads();
-    PipeHooks<Pol, NT> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
+    PipeHooks<Pol, NT, false, kCorn> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
     if (!Pol::kSmemRings) d.ring_buf = (unsigned char *)a.ring_bufs + (size_t)blockIdx.x * a.ring_stride;
     march_body<Pol, NT, PPT>(d, smem_raw, hk);
