@@ -202,7 +202,9 @@ int wake_bind_fields(wake_sim *s, int sim, void *psi, void *ez, void *er, void *
  * particle, measured at the start of each launch, slips more than 1/8 of a cell per step
  * takes the separate calls (the check synchronises the stream once per launch).  A particle
  * found behind the cell it was sorted into, or more slipped particles than the launch's
- * lists hold, raise WAKE_ESTATE through wake_status.
+ * lists hold, raise WAKE_ESTATE through wake_status.  Where the steps of a call are few against the
+ * GPU's SMs, a cluster of 2 to 8 CTAs shares each step (FP64, WAKE_MIXED), with the same results but
+ * for the order of the deposit sums.
  */
 int wake_step(wake_sim *s, int nsteps);
 
@@ -215,7 +217,9 @@ int wake_step(wake_sim *s, int nsteps);
  * 768 radial cells with more than 4096 rings, up to nr = 2048 and 65,536 rings) runs in the
  * wide form, which keeps its rings in a global buffer and processes them in chunks of
  * 512 x 8 (nt = 512, ppt = 8 here); WAKE_TILE_NT=-1 forces the wide form.  Before the first
- * march both are 0.  Instrumentation and tuning: the paper has no counterpart.
+ * march both are 0.  While few simulations march at once, a cluster of 2 to 8 CTAs of 256 threads
+ * shares each one's rings in place of the tile (not where WAKE_TILE_NT is set).  Instrumentation
+ * and tuning: the paper has no counterpart.
  */
 int wake_tile(wake_sim *s, int sim, int *nt, int *ppt);
 
