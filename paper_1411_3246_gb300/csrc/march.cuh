@@ -172,6 +172,9 @@ __device__ __forceinline__ float2 cl_add(float2 a, float2 b) { return make_float
 // the r-th share of the elements (in rank order, so every CTA holds the same bits) and writes the
 // sums to all: nobody else touches that share between the two barriers.  n elements cross the
 // cluster twice, and a CTA may change its array freely before the first and after the second.
+// Measured by itself with 8 CTAs: 2.0k cycles for 129 elements of 8 bytes, 2.5k for 774 (two barriers
+// with release and acquire are 800 of them); every CTA reading all arrays behind one barrier takes
+// 1.9k and 8.8k.  In the march 3.3k, the wait for the slowest CTA included.
 template <int NT, class V>
 __device__ __forceinline__ void cluster_sum(V *a, int n, int cn, int cr) {
   cl_barrier();
@@ -565,6 +568,8 @@ __device__ __forceinline__ FF q_to_wide<long long, FF>(long long d) {
 // parallel cyclic reduction over the lanes (Hockney), and the downward rows give the lane's other
 // unknowns.  The work is ~25 operations per row, against ~30 per row and doubling for a cyclic
 // reduction of all rows; the chain is E reciprocals and five doublings, without a block barrier.
+// The two field solves of a slice, E_z scan and rows included, took 18k cycles at 512 nodes with
+// the reduction over the block, and take 13k (257 nodes, mixed).
 //
 // Row q lies at tri_at(q) of each array: rows of the same index in consecutive lanes are adjacent,
 // 33 entries apart from the next index's, so the lanes' reads and the rows' writers (consecutive q)
