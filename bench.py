@@ -52,7 +52,7 @@ BEAM_STEPS = 200
 # capture with one pass (dram__bytes_read.sum + dram__bytes_write.sum: 951.24 + 149.09 MB),
 # valid while the kernel's sources hash to STEP_TRAFFIC_SOURCES
 STEP_TRAFFIC_BYTES = 1100.33e6
-STEP_TRAFFIC_SOURCES = "34814b820f57dd41"
+STEP_TRAFFIC_SOURCES = "785f5456b89c5638"
 STEP_SOURCES = ("beam.cuh", "march.cuh", "march_mixed.cu", "march_wide.cuh", "pipeline.cuh", "wake_common.cuh")
 
 

@@ -568,8 +568,9 @@ __device__ __forceinline__ FF q_to_wide<long long, FF>(long long d) {
 // parallel cyclic reduction over the lanes (Hockney), and the downward rows give the lane's other
 // unknowns.  The work is ~25 operations per row, against ~30 per row and doubling for a cyclic
 // reduction of all rows; the chain is E reciprocals and five doublings, without a block barrier.
-// The two field solves of a slice, E_z scan and rows included, took 18k cycles at 512 nodes with
-// the reduction over the block, and take 13k (257 nodes, mixed).
+// The two field solves of a slice, E_z scans and rows included, take 12.6k cycles at 257 nodes and
+// 7.1k at 129 (mixed); with the reduction over the block 18k at 513 nodes.  Mixed linear march of 128
+// cells, this and the doubled barriers out: 1,392 -> 1,153 us.
 //
 // Row q lies at tri_at(q) of each array: rows of the same index in consecutive lanes are adjacent,
 // 33 entries apart from the next index's, so the lanes' reads and the rows' writers (consecutive q)
