@@ -50,16 +50,8 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
   const float h = s + e;
   return FF{h, e - (h - s)};
 }
-// The scans' sum: the rounding error of the high parts (two-sum) joins the low parts, without a
-// renormalisation at each level, so a level's chain is a shuffle and two adds instead of nine (the
-// error is formed beside the next level's shuffle).  The low part stays below n ulp of the high one.
-__device__ __forceinline__ FF ff_sum(FF a, FF b) {
-  const float s = a.h + b.h;
-  const float bb = s - a.h;
-  return FF{s, (a.l + b.l) + ((a.h - (s - bb)) + (b.h - bb))};
-}
 __device__ __forceinline__ double wide_add(double a, double b) { return a + b; }
-__device__ __forceinline__ FF wide_add(FF a, FF b) { return ff_sum(a, b); }
+__device__ __forceinline__ FF wide_add(FF a, FF b) { return ff_add(a, b); }
 __device__ __forceinline__ double wide_shfl_up(double a, int o) { return __shfl_up_sync(kFull, a, o); }
 __device__ __forceinline__ FF wide_shfl_up(FF a, int o) {
   return FF{__shfl_up_sync(kFull, a.h, o), __shfl_up_sync(kFull, a.l, o)};
