@@ -217,7 +217,7 @@ int wake_step(wake_sim *s, int nsteps);
  * 768 radial cells with more than 4096 rings, up to nr = 2048 and 65,536 rings) runs in the
  * wide form, which keeps its rings in a global buffer and processes them in chunks of
  * 512 x 8 (nt = 512, ppt = 8 here); WAKE_TILE_NT=-1 forces the wide form.  Before the first
- * march both are 0.  While few simulations march at once, a cluster of 2 to 8 CTAs of 256 threads
+ * march both are 0.  While few FP64 simulations march at once, a cluster of 2 to 8 CTAs of 256 threads
  * shares each one's rings in place of the tile (not where WAKE_TILE_NT is set).  Instrumentation
  * and tuning: the paper has no counterpart.
  */

@@ -12,7 +12,7 @@
 //       nodes and the radial current K_c of each cell (pass_currents);
 //   P2  E_z = d_xi psi (Eq. 7) by a block-wide inward scan of the cell currents; Q = P + E_z U;
 //       B_theta from Eq. 6 differentiated in r (Helmholtz form, shift chi), a tridiagonal
-//       system solved on row sums by one warp (solve_fields);
+//       system solved on row sums by one warp, in the mixed plain marches by the block (solve_fields);
 //   P3  per ring: the Cartesian radial force (gamma/Gamma) psi' - B_theta (Eqs. 4-5 with the
 //       centrifugal term carried by the local frame), the move to the next stage's position,
 //       and that position's charge deposit (linear hats).
@@ -197,6 +197,15 @@ __device__ __forceinline__ void cluster_sum(V *a, int n, int cn, int cr) {
 // FP64: rings in global memory in their initial order, node coefficients from tables (FP64
 // division is slow on this chip).  kWinGlobal: the pipelined step keeps its field window in
 // global memory (its shared memory is full).
+//
+// kPlain: the arithmetic of the mixed forms' plain marches, whose fields the caller gets: rings
+// deposited through windows of three cells, u_theta and the centrifugal term by divisions, B_theta by
+// cyclic reduction over the block.  A ring's radial current counts in one cell (K), so E_z jumps at a
+// node when a ring crosses into the next cell a slice earlier; which slice that is hangs on the last bit
+// of the fields before it, and another order of operations anywhere (solver, windows, sums over a
+// cluster) moves E_z at single nodes by 1e-3 of its rms, without being nearer to 64 bits or farther.  So
+// these marches keep the order they always had.  The carried beam (StepOf) reads the fields at its own
+// particles, where the jumps average out, and takes the faster forms.
 // ---------------------------------------------------------------------------------------
 struct PolFP64 {
   using R = double;
@@ -212,6 +221,7 @@ struct PolFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
+  static constexpr bool kPlain = false;
   static constexpr int kScanE = 3;  // nodes per thread in the block scans: n1 <= kScanE * NT
 };
 struct PolMixed {
@@ -228,6 +238,7 @@ struct PolMixed {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
+  static constexpr bool kPlain = true;
   static constexpr int kScanE = 3;
 };
 // The precision split in which only the particle arithmetic is FP32: each ring's push and its
@@ -248,6 +259,7 @@ struct PolMixed64 {
   static constexpr bool kWinGlobal = true;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
+  static constexpr bool kPlain = true;
   static constexpr int kScanE = 3;
 };
 // The mixed arithmetic for boxes too large for one CTA's shared memory to hold the rings
@@ -267,6 +279,7 @@ struct PolWide {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
+  static constexpr bool kPlain = true;
   static constexpr int kScanE = 5;
 };
 
@@ -287,7 +300,13 @@ struct PolWideFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
+  static constexpr bool kPlain = false;
   static constexpr int kScanE = 5;
+};
+// A policy in the pipelined beam steps.
+template <class P>
+struct StepOf : P {
+  static constexpr bool kPlain = false;
 };
 // A policy marched by clusters of narrower CTAs (march_cluster_*.cu).
 template <class P>
@@ -307,6 +326,9 @@ struct SlabOf : P {
 // Rows per lane of the tridiagonal solve (tri_solve_warp) of n rows, and the length of its arrays.
 __host__ __device__ constexpr int tri_per_lane(int n) { return (n + 31) >> 5; }
 __host__ __device__ constexpr int tri_len(int n) { return 33 * ((n + 31) >> 5); }
+// Entries of a tridiagonal row array for n1 nodes.
+template <class Pol>
+__host__ __device__ constexpr int row_len(int n1) { return Pol::kPlain ? n1 + 32 : tri_len(n1); }
 
 // Ring slot arrays: cell index, offset in the cell, u_r, the constants l_z, Gamma_0, w, and
 // the stage-1 Gamma and radial force kept for the full step; with ids, each slot also carries
@@ -353,7 +375,7 @@ struct MarchSmem {
 
   __host__ __device__ static size_t bytes(int n1, int slots, bool ids = false) {
     size_t b = sizeof(typename Pol::W) * 64 + sizeof(typename Pol::Q) * 2 * (size_t)n1 + sizeof(Acc) * 6 * (size_t)n1 +
-               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + sizeof(N) * 4 * (size_t)tri_len(n1) + 256;
+               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + sizeof(N) * 4 * (size_t)row_len<Pol>(n1) + 256;
     b += sizeof(N) * (Pol::kTables ? 6 : 2) * (size_t)n1;
     if (Pol::kSortEvery > 0) b += sizeof(int) * ((size_t)n1 + 32);
     if (Pol::kSmemRings) b += RingSoA<R>::bytes(slots, ids) + 32;
@@ -376,10 +398,10 @@ struct MarchSmem {
     dpsi = rp; rp += n1;
     ez = rp; rp += n1;
     bth = rp; rp += n1;
-    ta = rp; rp += tri_len(n1);
-    tb = rp; rp += tri_len(n1);
-    tc = rp; rp += tri_len(n1);
-    td = rp; rp += tri_len(n1);
+    ta = rp; rp += row_len<Pol>(n1);
+    tb = rp; rp += row_len<Pol>(n1);
+    tc = rp; rp += row_len<Pol>(n1);
+    td = rp; rp += row_len<Pol>(n1);
     invR = invV = alpha = ga = gb = gc = nullptr;
     invR = rp; rp += n1;
     ga = rp; rp += n1;
@@ -405,7 +427,7 @@ struct MarchSmem {
   // The out-of-window ring queue: slot ids in the tridiagonal rows, which are free from the end
   // of one solve to the start of the next (a ring pass and the deposits that follow it)
   __device__ __forceinline__ int *queue() const { return (int *)ta; }
-  __device__ __forceinline__ int queue_cap(int n1) const { return (int)(4 * (size_t)tri_len(n1) * sizeof(N) / sizeof(int)); }
+  __device__ __forceinline__ int queue_cap(int n1) const { return (int)(4 * (size_t)row_len<Pol>(n1) * sizeof(N) / sizeof(int)); }
 };
 
 // ---------------------------------------------------------------------------------------
@@ -561,8 +583,7 @@ __device__ __forceinline__ FF q_to_wide<long long, FF>(long long d) {
 // unknowns.  The work is ~25 operations per row, against ~30 per row and doubling for a cyclic
 // reduction of all rows; the chain is E reciprocals and five doublings, without a block barrier.
 // The two field solves of a slice, E_z scans and rows included, take 12.6k cycles at 257 nodes and
-// 7.1k at 129 (mixed); with the reduction over the block 18k at 513 nodes.  Mixed linear march of 128
-// cells, this and the doubled barriers out: 1,392 -> 1,153 us.
+// 7.1k at 129 (mixed); with the reduction over the block 18k at 513 nodes.
 //
 // Row q lies at tri_at(q) of each array: rows of the same index in consecutive lanes are adjacent,
 // 33 entries apart from the next index's, so the lanes' reads and the rows' writers (consecutive q)
@@ -645,6 +666,119 @@ __device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S
     const int v = e * 33 + lane;
     x = (wd[v] - wl[v] * zl - tc[v] * x) * wr[v];
     if (q0 + e < n) out(q0 + e, x);
+  }
+}
+
+// The same system by parallel cyclic reduction over the block (kPlain), rows in natural order, every
+// doubling over the block with a barrier.  Double-buffered; returns the buffer holding the result
+// (x_q = d_q / s_q there).  Ends with a barrier.
+template <int NT, class S>
+__device__ __forceinline__ int pcr_rowsum(S *a0, S *s0, S *c0, S *d0, S *a1, S *s1, S *c1, S *d1, int n) {
+  int cur = 0;
+  for (int k = 1; k < n; k <<= 1) {
+    const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
+    S *an = cur ? a0 : a1, *sn = cur ? s0 : s1, *cn = cur ? c0 : c1, *dn = cur ? d0 : d1;
+    for (int q = threadIdx.x; q < n; q += NT) {
+      const S aq = a[q], cq = c[q];
+      S sq = sm_[q], dq = d[q], na = (S)0, nc = (S)0;
+      if (q - k >= 0) {
+        const S bm = sm_[q - k] - a[q - k] - c[q - k];
+        const S k1 = aq / bm;
+        sq -= k1 * sm_[q - k];
+        dq -= k1 * d[q - k];
+        na = -a[q - k] * k1;
+      }
+      if (q + k < n) {
+        const S bp = sm_[q + k] - a[q + k] - c[q + k];
+        const S k2 = cq / bp;
+        sq -= k2 * sm_[q + k];
+        dq -= k2 * d[q + k];
+        nc = -c[q + k] * k2;
+      }
+      an[q] = na;
+      sn[q] = sq;
+      cn[q] = nc;
+      dn[q] = dq;
+    }
+    __syncthreads();
+    cur ^= 1;
+  }
+  return cur;
+}
+
+// The same with the last doublings in warps (the tiles; in the wide form, whose time is in the rings, it
+// is not faster, and its compiled roundings are others).  The first doublings (strides 1 .. ns/2) run over
+// the block, double-buffered, one barrier each.  They leave ns independent systems, rows r, r + ns, r + 2 ns, ... (ns the smallest power of two >= NT/32
+// with n <= 32 ns); each is finished by one warp, lane l holding row r + ns l, with the remaining
+// doublings (lane strides 1 .. 16) done by shuffles.  out(q, x_q) receives the solution.
+template <int NT, class S, class Out>
+__device__ __forceinline__ void pcr_rowsum_solve(S *a0, S *s0, S *c0, S *d0, S *a1, S *s1, S *c1, S *d1, int n,
+                                                 Out &&out) {
+  constexpr int W = NT / 32;
+  int ns = W;
+  while (32 * ns < n) ns <<= 1;
+  int cur = 0;
+  for (int k = 1; k < ns && k < n; k <<= 1) {
+    const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
+    S *an = cur ? a0 : a1, *sn = cur ? s0 : s1, *cn = cur ? c0 : c1, *dn = cur ? d0 : d1;
+    for (int q = threadIdx.x; q < n; q += NT) {
+      const S aq = a[q], cq = c[q];
+      S sq = sm_[q], dq = d[q], na = (S)0, nc = (S)0;
+      if (q - k >= 0) {
+        const S bm = sm_[q - k] - a[q - k] - c[q - k];
+        const S k1 = aq / bm;
+        sq -= k1 * sm_[q - k];
+        dq -= k1 * d[q - k];
+        na = -a[q - k] * k1;
+      }
+      if (q + k < n) {
+        const S bp = sm_[q + k] - a[q + k] - c[q + k];
+        const S k2 = cq / bp;
+        sq -= k2 * sm_[q + k];
+        dq -= k2 * d[q + k];
+        nc = -c[q + k] * k2;
+      }
+      an[q] = na;
+      sn[q] = sq;
+      cn[q] = nc;
+      dn[q] = dq;
+    }
+    __syncthreads();
+    cur ^= 1;
+  }
+  const S *a = cur ? a1 : a0, *sm_ = cur ? s1 : s0, *c = cur ? c1 : c0, *d = cur ? d1 : d0;
+  const int lane = threadIdx.x & 31;
+  for (int r = threadIdx.x >> 5; r < ns; r += W) {
+    const int q = r + ns * lane;
+    const bool on = q < n;  // rows past n: the identity (their neighbours' couplings to them are zero)
+    S aq = on ? a[q] : (S)0, sq = on ? sm_[q] : (S)1, cq = on ? c[q] : (S)0, dq = on ? d[q] : (S)0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const S am = __shfl_up_sync(kFull, aq, o), smm = __shfl_up_sync(kFull, sq, o);
+      const S cm = __shfl_up_sync(kFull, cq, o), dm = __shfl_up_sync(kFull, dq, o);
+      const S ap = __shfl_down_sync(kFull, aq, o), spp = __shfl_down_sync(kFull, sq, o);
+      const S cp = __shfl_down_sync(kFull, cq, o), dp = __shfl_down_sync(kFull, dq, o);
+      S s2 = sq, d2 = dq, na = (S)0, nc = (S)0;
+      if (lane >= o) {
+        const S bm = smm - am - cm;
+        const S k1 = aq / bm;
+        s2 -= k1 * smm;
+        d2 -= k1 * dm;
+        na = -am * k1;
+      }
+      if (lane + o < 32) {
+        const S bp = spp - ap - cp;
+        const S k2 = cq / bp;
+        s2 -= k2 * spp;
+        d2 -= k2 * dp;
+        nc = -cp * k2;
+      }
+      aq = na;
+      sq = s2;
+      cq = nc;
+      dq = d2;
+    }
+    if (on) out(q, dq / sq);
   }
 }
 
@@ -760,11 +894,11 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
   // rows) read where the rows need them
   auto dens = [&](const Acc *v, int m) -> R { return (R)v[m] * geo.invV(m); };
   auto jz_node = [&](int m) -> R { return (R)sm.jz[m] * geo.invV(m) - (R)0.5 * ((R)nbA[m] + (R)nbB[m]); };
-  // rows q = 0..nr-1 (node i = q + 1): central differences, a half cell at the wall; the rows
-  // past them up to whole lanes are -x = 0
+  // rows q = 0..nr-1 (node i = q + 1): central differences, a half cell at the wall; the one-warp
+  // solve's rows past them up to whole lanes are -x = 0
   const R i2dr = (R)0.5 * inv_dr;
   const TriAt at(nr);
-  const int nrows = 32 * at.E;
+  const int nrows = Pol::kPlain ? nr : 32 * at.E;
   for (int q = tid; q < nrows; q += NT) {
     R a = (R)0, c = (R)0, s = (R)-1, rhs = (R)0;
     if (q < nr) {
@@ -779,20 +913,28 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
       else
         rhs = Qi + (Ti - dens(sm.T, i - 1)) * inv_dr + Ti * geo.curv(i) - (jz_node(i - 1) + jz_node(i)) * inv_dr;
     }
-    const int r = at(q);
+    const int r = Pol::kPlain ? q : at(q);
     sm.ta[r] = a;
     sm.tb[r] = s;
     sm.tc[r] = c;
     sm.td[r] = rhs;
   }
   __syncthreads();
-  // one warp solves; its scratch reuses the six deposit arrays (contiguous, dead once the rows are
-  // set up, zeroed before the next pass B): 3 tri_len(nr) <= 6 (nr + 1) whenever nr > 32
+  // the solver's scratch reuses the six deposit arrays (contiguous, dead once the rows are set up,
+  // zeroed before the next pass B): the one-warp solve's 3 tri_len(nr) <= 6 (nr + 1) whenever nr > 32,
+  // the reduction's second buffer in four of them
   static_assert(sizeof(Acc) == sizeof(R), "the solver's scratch reuses the deposit arrays");
-  if (tid < 32) {
-    tri_solve_warp<R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, nr, [&](int q, R x) { sm.bth[q + 1] = x; });
-    if (tid == 0) sm.bth[0] = (R)0;
+  auto out = [&](int q, R x) { sm.bth[q + 1] = x; };  // row q is node q + 1
+  if constexpr (!Pol::kPlain) {
+    if (tid < 32) tri_solve_warp<R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, nr, out);
+  } else if constexpr (Pol::kSmemRings) {
+    pcr_rowsum_solve<NT, R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, (R *)sm.chi, (R *)sm.T, (R *)sm.P, nr, out);
+  } else {
+    const int cur = pcr_rowsum<NT, R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, (R *)sm.chi, (R *)sm.T, (R *)sm.P, nr);
+    const R *bb = cur ? (const R *)sm.chi : sm.tb, *dd = cur ? (const R *)sm.P : sm.td;  // row sum = diagonal now
+    for (int q = tid; q < nr; q += NT) out(q, dd[q] / bb[q]);
   }
+  if (tid == 0) sm.bth[0] = (R)0;
   __syncthreads();
 }
 
@@ -866,8 +1008,9 @@ __device__ __forceinline__ void move_ring(int c, R f, R r, R dx, R dy, R ux, R u
 
 // Cells of a thread's deposit window: a thread of one ring needs that ring's cell only, a thread
 // of two rarely more than two.  Every cell less is a node less to sum over the warp and to add:
-// 11, 17 or 23 sums per thread of a current pass.
-__host__ __device__ constexpr int win_cells(int ppt) { return ppt == 1 ? 1 : ppt == 2 ? 2 : 3; }
+// 11, 17 or 23 sums per thread of a current pass.  (kPlain: always three.)
+template <class Pol>
+__host__ __device__ constexpr int win_cells(int ppt) { return Pol::kPlain ? 3 : ppt == 1 ? 1 : ppt == 2 ? 2 : 3; }
 
 // Window of three (or NC) cells c0..c0+2 (NC + 1 nodes) summed in registers; a ring outside the
 // window deposits directly.
@@ -1121,6 +1264,9 @@ __device__ __forceinline__ void current_values(const MarchSmem<Pol> &sm, const R
   if (slab) {
     iG = rcp_of(G);
     if (kFromL) u_t = rs.lz[sl];
+  } else if (Pol::kPlain) {
+    iG = rcp_of(G);
+    if (kFromL) u_t = rp > (R)0 ? rs.lz[sl] / rp : (R)0;
   } else {
     const bool off = rp > tiny_r<R>();
     rcp_pair(G, off ? rp : (R)1, iG, ir);
@@ -1132,7 +1278,8 @@ __device__ __forceinline__ void current_values(const MarchSmem<Pol> &sm, const R
   const R uz = gam - G;
   const R a = u_r * iG;
   const R dp = interp(sm.dpsi, c, f);
-  const R cent = slab ? (R)0 : u_t * u_t * iG * ir;  // Eq. 4's centrifugal term (cylinder)
+  // Eq. 4's centrifugal term (cylinder)
+  const R cent = slab ? (R)0 : Pol::kPlain ? (rp > (R)0 ? u_t * u_t * iG / rp : (R)0) : u_t * u_t * iG * ir;
   g = gam * iG * dp;
   const R w = rs.w[sl];
   v[0] = -w * uz * iG;
@@ -1183,7 +1330,7 @@ __device__ __forceinline__ void pass_currents(MarchSmem<Pol> &sm, const RingSoA<
   using R = typename Pol::R;
   using Acc = typename Pol::Acc;
   const int t = threadIdx.x;
-  constexpr int NC = win_cells(PPT);
+  constexpr int NC = win_cells<Pol>(PPT);
   WindowAcc<R, 5, NC> acc;
   acc.init(-8);
   R kw[NC];
@@ -1465,6 +1612,9 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     if (slab) {
       iG = rcp_of(rs.G1[sl]);
       ut = (R)0;
+    } else if (Pol::kPlain) {
+      iG = rcp_of(rs.G1[sl]);
+      ut = r > (R)0 ? rs.lz[sl] / r : (R)0;
     } else {
       const bool off = r > tiny_r<R>();
       R ir;
@@ -1509,7 +1659,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
   // charge of the initial slice; it is also the ion background (the deposit of the
   // unperturbed electrons), so psi starts exactly at zero
   {
-    ChargeWin<Pol, win_cells(PPT)> acc;
+    ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
     acc.init(-8);
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
@@ -1558,7 +1708,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     // the midpoint of each ring, kept in registers for stage 2 and the full step (its direction too
     // where a thread has few rings; more would spill)
-    constexpr bool kKeepDir = PPT <= 2;
+    constexpr bool kKeepDir = PPT <= 2 && !Pol::kPlain;
     int MC[PPT];
     R MF[PPT], MUR[PPT], MUT[PPT], MEX[kKeepDir ? PPT : 1], MEY[kKeepDir ? PPT : 1];
 #pragma unroll
@@ -1567,7 +1717,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
       MF[p] = MUR[p] = MUT[p] = (R)0;
     }
     {
-      ChargeWin<Pol, win_cells(PPT)> acc;
+      ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -1635,7 +1785,7 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
     // deposit of the new slice
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     {
-      ChargeWin<Pol, win_cells(PPT)> acc;
+      ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -1658,7 +1808,14 @@ __device__ __forceinline__ void march_body(const SimDesc &d, unsigned char *smem
             ey = MEY[p];
           } else {
             const R xh = r + (R)0.5 * h * ur0 * iG1, yh = (R)0.5 * h * ut * iG1, h2 = xh * xh + yh * yh;
-            if (h2 > tiny_r2<R>()) {
+            if constexpr (Pol::kPlain) {
+              const R rh = sqrt(h2);
+              if (rh > (R)0) {
+                const R irh = (R)1 / rh;
+                ex = xh * irh;
+                ey = yh * irh;
+              }
+            } else if (h2 > tiny_r2<R>()) {
               R rh, irh;
               root_of(h2, rh, irh);
               ex = xh * irh;

@@ -1,7 +1,8 @@
-// Cluster forms of the march and of the pipelined step (march.cuh, Hooks::kCluster): one
+// Cluster forms of the FP64 march and of the pipelined step (march.cuh, Hooks::kCluster): one
 // simulation, or one beam step, per cluster of 2, 4 or 8 CTAs of 256 threads, for launches with
 // fewer simulations (steps) than the GPU has SMs.  One template set, instantiated per precision
-// form (march_cluster_mixed.cu, march_cluster_fp64.cu).
+// form (march_cluster_mixed.cu, march_cluster_fp64.cu).  The mixed plain marches have none: sums
+// over a cluster are another order of their deposits (march.cuh, kPlain).
 #pragma once
 
 #include <mutex>
@@ -18,7 +19,8 @@ inline int cluster_ppt(int np, int cn) {
   return ppt <= 1 ? 1 : ppt <= 2 ? 2 : ppt <= 4 ? 4 : ppt <= 8 ? 8 : 0;
 }
 
-template <class P>
+// kMarch: the form has cluster marches, not steps only.
+template <class P, bool kMarch = true>
 struct ClusterForm {
   using C = ClusterOf<P>;
   using S = SlabOf<ClusterOf<P>>;
@@ -38,7 +40,9 @@ struct ClusterForm {
   }
   template <class Q, int PPT>
   static const void *kernel_of(bool step) {
-    return step ? (const void *)step_cluster_kernel<Q, kClNT, PPT> : (const void *)march_cluster_kernel<Q, kClNT, PPT>;
+    if constexpr (kMarch)
+      if (!step) return (const void *)march_cluster_kernel<Q, kClNT, PPT>;
+    return (const void *)step_cluster_kernel<Q, kClNT, PPT>;
   }
   template <class Q>
   static const void *kernel(bool step, int ppt) {
@@ -56,7 +60,7 @@ struct ClusterForm {
     *err = cudaSuccess;
     const int ppt = cluster_ppt(np, cn);
     *bytes = smem_of(step, n1, ppt);
-    if (ppt == 0 || n1 > C::kScanE * kClNT || *bytes > kMaxSmemPerCta) return nullptr;
+    if ((!step && !kMarch) || ppt == 0 || n1 > C::kScanE * kClNT || *bytes > kMaxSmemPerCta) return nullptr;
     const void *k = slab ? kernel<S>(step, ppt) : kernel<C>(step, ppt);
     static std::mutex mu;
     static size_t set[2][2][4] = {};

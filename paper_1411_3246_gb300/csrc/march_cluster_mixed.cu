@@ -1,23 +1,23 @@
-// Cluster forms of the mixed march (march_cluster.cuh), and the choice between the forms.
+// Cluster forms of the mixed pipelined steps (march_cluster.cuh), and the choice between the forms.
 #include "march_cluster.cuh"
 
 namespace wake {
 
+using StepClusters = ClusterForm<StepOf<PolMixed>, false>;
+
 int cluster_max(int form, bool slab, bool step, int n1, int np, int cn) {
-  if (form == kFormMixed) return ClusterForm<PolMixed>::max_clusters(slab, step, n1, np, cn);
+  if (form == kFormMixed) return StepClusters::max_clusters(slab, step, n1, np, cn);
   return form == kFormFP64 ? cluster_max_fp64(slab, step, n1, np, cn) : 0;
 }
 cudaError_t launch_march_cluster(int form, bool slab, const SimDesc *d, const int *order, int count, int n1, int np, int cn,
                                  cudaStream_t stream) {
-  if (form == kFormFP64) return launch_march_cluster_fp64(slab, d, order, count, n1, np, cn, stream);
-  void *args[] = {&d, &order};
-  return ClusterForm<PolMixed>::launch(slab, false, n1, np, cn, count, args, stream);
+  return form == kFormFP64 ? launch_march_cluster_fp64(slab, d, order, count, n1, np, cn, stream) : cudaErrorInvalidValue;
 }
 cudaError_t launch_step_cluster(int form, const PipeArgs &a, int cn, int clusters, cudaStream_t stream) {
   if (form == kFormFP64) return launch_step_cluster_fp64(a, cn, clusters, stream);
   PipeArgs arg = a;
   void *args[] = {&arg};
-  return ClusterForm<PolMixed>::launch(a.d.slab != 0, true, a.d.nr + 1, a.d.np, cn, clusters, args, stream);
+  return StepClusters::launch(a.d.slab != 0, true, a.d.nr + 1, a.d.np, cn, clusters, args, stream);
 }
 
 }  // namespace wake

@@ -58,9 +58,9 @@ int batch_step_max_ctas(int max_n1, int bnt);
 size_t batch_ring_bytes(int max_np, int bnt);
 cudaError_t launch_batch_steps(const BatchArgs &b, int max_n1, int bnt, int ctas, cudaStream_t stream);
 
-// Clusters of cn = 2, 4 or 8 CTAs per simulation or beam step (march_cluster.cuh): how many the GPU
-// holds at once (0: the form, grid or ring count has none), and the launches: `count` simulations
-// of at most n1 nodes and np rings, or the steps of `a` on `clusters` resident clusters.
+// Clusters of cn = 2, 4 or 8 CTAs per simulation (FP64) or beam step (FP64, mixed; march_cluster.cuh):
+// how many the GPU holds at once (0: the form, grid or ring count has none), and the launches: `count`
+// simulations of at most n1 nodes and np rings, or the steps of `a` on `clusters` resident clusters.
 int cluster_max(int form, bool slab, bool step, int n1, int np, int cn);
 cudaError_t launch_march_cluster(int form, bool slab, const SimDesc *d, const int *order, int count, int n1, int np, int cn,
                                  cudaStream_t stream);

@@ -25,67 +25,69 @@ bool march_tile_mixed512(int nt, int ppt, TileFns *out, bool slab) {
   }
 }
 
+using StepMixed = StepOf<PolMixed>;
+
 template <class P, int PPT, bool kCorn = false>
 static cudaError_t go_step(const PipeArgs &a, int ctas, cudaStream_t stream) {
-  auto kern = step_kernel<P, PolMixed::NT, PPT, kCorn>;
-  const size_t smem = step_smem_bytes<PolMixed, PolMixed::NT, PPT>(a.d.nr + 1);
+  auto kern = step_kernel<P, StepMixed::NT, PPT, kCorn>;
+  const size_t smem = step_smem_bytes<StepMixed, StepMixed::NT, PPT>(a.d.nr + 1);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   PipeArgs arg = a;
   void *args[] = {&arg};
-  return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(PolMixed::NT), args, smem, stream);
+  return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(StepMixed::NT), args, smem, stream);
 }
 template <int PPT>
 static int ctas_step(int n1) {
-  auto kern = step_kernel<PolMixed, PolMixed::NT, PPT>;
-  const size_t smem = step_smem_bytes<PolMixed, PolMixed::NT, PPT>(n1);
+  auto kern = step_kernel<StepMixed, StepMixed::NT, PPT>;
+  const size_t smem = step_smem_bytes<StepMixed, StepMixed::NT, PPT>(n1);
   if (smem > 227 * 1024) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int per_sm = 0, dev = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PolMixed::NT, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, StepMixed::NT, smem) != cudaSuccess) return 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return per_sm * sms;
 }
 static int ppt_for(int np) {
-  const int ppt = (np + PolMixed::NT - 1) / PolMixed::NT;
+  const int ppt = (np + StepMixed::NT - 1) / StepMixed::NT;
   return ppt <= 1 ? 1 : ppt <= 2 ? 2 : ppt <= 4 ? 4 : ppt <= 8 ? 8 : ppt <= 16 ? 16 : 0;
 }
 static size_t step_bytes_for(int n1, int np) {
   switch (ppt_for(np)) {
-    case 1: return step_smem_bytes<PolMixed, PolMixed::NT, 1>(n1);
-    case 2: return step_smem_bytes<PolMixed, PolMixed::NT, 2>(n1);
-    case 4: return step_smem_bytes<PolMixed, PolMixed::NT, 4>(n1);
-    case 8: return step_smem_bytes<PolMixed, PolMixed::NT, 8>(n1);
-    case 16: return step_smem_bytes<PolMixed, PolMixed::NT, 16>(n1);
+    case 1: return step_smem_bytes<StepMixed, StepMixed::NT, 1>(n1);
+    case 2: return step_smem_bytes<StepMixed, StepMixed::NT, 2>(n1);
+    case 4: return step_smem_bytes<StepMixed, StepMixed::NT, 4>(n1);
+    case 8: return step_smem_bytes<StepMixed, StepMixed::NT, 8>(n1);
+    case 16: return step_smem_bytes<StepMixed, StepMixed::NT, 16>(n1);
     default: return (size_t)1 << 40;
   }
 }
 cudaError_t launch_step_mixed(const PipeArgs &a, int np, int ctas, cudaStream_t stream) {
   if (a.d.slab) {  // the slab geometry's kernels (up to 8 rings per thread)
     switch (ppt_for(np)) {
-      case 1: return go_step<SlabOf<PolMixed>, 1>(a, ctas, stream);
-      case 2: return go_step<SlabOf<PolMixed>, 2>(a, ctas, stream);
-      case 4: return go_step<SlabOf<PolMixed>, 4>(a, ctas, stream);
-      case 8: return go_step<SlabOf<PolMixed>, 8>(a, ctas, stream);
+      case 1: return go_step<SlabOf<StepMixed>, 1>(a, ctas, stream);
+      case 2: return go_step<SlabOf<StepMixed>, 2>(a, ctas, stream);
+      case 4: return go_step<SlabOf<StepMixed>, 4>(a, ctas, stream);
+      case 8: return go_step<SlabOf<StepMixed>, 8>(a, ctas, stream);
       default: return cudaErrorInvalidValue;
     }
   }
   if (a.corners) {
     switch (ppt_for(np)) {
-      case 1: return go_step<PolMixed, 1, true>(a, ctas, stream);
-      case 2: return go_step<PolMixed, 2, true>(a, ctas, stream);
-      case 4: return go_step<PolMixed, 4, true>(a, ctas, stream);
-      case 8: return go_step<PolMixed, 8, true>(a, ctas, stream);
+      case 1: return go_step<StepMixed, 1, true>(a, ctas, stream);
+      case 2: return go_step<StepMixed, 2, true>(a, ctas, stream);
+      case 4: return go_step<StepMixed, 4, true>(a, ctas, stream);
+      case 8: return go_step<StepMixed, 8, true>(a, ctas, stream);
       default: return cudaErrorInvalidValue;
     }
   }
   switch (ppt_for(np)) {
-    case 1: return go_step<PolMixed, 1>(a, ctas, stream);
-    case 2: return go_step<PolMixed, 2>(a, ctas, stream);
-    case 4: return go_step<PolMixed, 4>(a, ctas, stream);
-    case 8: return go_step<PolMixed, 8>(a, ctas, stream);
-    case 16: return go_step<PolMixed, 16>(a, ctas, stream);
+    case 1: return go_step<StepMixed, 1>(a, ctas, stream);
+    case 2: return go_step<StepMixed, 2>(a, ctas, stream);
+    case 4: return go_step<StepMixed, 4>(a, ctas, stream);
+    case 8: return go_step<StepMixed, 8>(a, ctas, stream);
+    case 16: return go_step<StepMixed, 16>(a, ctas, stream);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -27,58 +27,60 @@ bool march_tile_mixed64(int nt, int ppt, TileFns *out, bool slab) {
   }
 }
 
+using StepMixed64 = StepOf<PolMixed64>;
+
 template <class P, int PPT>
 static cudaError_t go_step(const PipeArgs &a, int ctas, cudaStream_t stream) {
-  auto kern = step_kernel<P, PolMixed64::NT, PPT>;
-  const size_t smem = step_smem_bytes<PolMixed64, PolMixed64::NT, PPT>(a.d.nr + 1);
+  auto kern = step_kernel<P, StepMixed64::NT, PPT>;
+  const size_t smem = step_smem_bytes<StepMixed64, StepMixed64::NT, PPT>(a.d.nr + 1);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   PipeArgs arg = a;
   void *args[] = {&arg};
-  return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(PolMixed64::NT), args, smem, stream);
+  return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(StepMixed64::NT), args, smem, stream);
 }
 template <int PPT>
 static int ctas_step(int n1) {
-  auto kern = step_kernel<PolMixed64, PolMixed64::NT, PPT>;
-  const size_t smem = step_smem_bytes<PolMixed64, PolMixed64::NT, PPT>(n1);
+  auto kern = step_kernel<StepMixed64, StepMixed64::NT, PPT>;
+  const size_t smem = step_smem_bytes<StepMixed64, StepMixed64::NT, PPT>(n1);
   if (smem > 227 * 1024) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int per_sm = 0, dev = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PolMixed64::NT, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, StepMixed64::NT, smem) != cudaSuccess) return 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return per_sm * sms;
 }
 static int ppt_for(int np) {
-  const int ppt = (np + PolMixed64::NT - 1) / PolMixed64::NT;
+  const int ppt = (np + StepMixed64::NT - 1) / StepMixed64::NT;
   return ppt <= 1 ? 1 : ppt <= 2 ? 2 : ppt <= 4 ? 4 : ppt <= 8 ? 8 : ppt <= 16 ? 16 : 0;
 }
 static size_t step_bytes_for(int n1, int np) {
   switch (ppt_for(np)) {
-    case 1: return step_smem_bytes<PolMixed64, PolMixed64::NT, 1>(n1);
-    case 2: return step_smem_bytes<PolMixed64, PolMixed64::NT, 2>(n1);
-    case 4: return step_smem_bytes<PolMixed64, PolMixed64::NT, 4>(n1);
-    case 8: return step_smem_bytes<PolMixed64, PolMixed64::NT, 8>(n1);
-    case 16: return step_smem_bytes<PolMixed64, PolMixed64::NT, 16>(n1);
+    case 1: return step_smem_bytes<StepMixed64, StepMixed64::NT, 1>(n1);
+    case 2: return step_smem_bytes<StepMixed64, StepMixed64::NT, 2>(n1);
+    case 4: return step_smem_bytes<StepMixed64, StepMixed64::NT, 4>(n1);
+    case 8: return step_smem_bytes<StepMixed64, StepMixed64::NT, 8>(n1);
+    case 16: return step_smem_bytes<StepMixed64, StepMixed64::NT, 16>(n1);
     default: return (size_t)1 << 40;
   }
 }
 cudaError_t launch_step_mixed64(const PipeArgs &a, int np, int ctas, cudaStream_t stream) {
   if (a.d.slab) {
     switch (ppt_for(np)) {
-      case 1: return go_step<SlabOf<PolMixed64>, 1>(a, ctas, stream);
-      case 2: return go_step<SlabOf<PolMixed64>, 2>(a, ctas, stream);
-      case 4: return go_step<SlabOf<PolMixed64>, 4>(a, ctas, stream);
-      case 8: return go_step<SlabOf<PolMixed64>, 8>(a, ctas, stream);
+      case 1: return go_step<SlabOf<StepMixed64>, 1>(a, ctas, stream);
+      case 2: return go_step<SlabOf<StepMixed64>, 2>(a, ctas, stream);
+      case 4: return go_step<SlabOf<StepMixed64>, 4>(a, ctas, stream);
+      case 8: return go_step<SlabOf<StepMixed64>, 8>(a, ctas, stream);
       default: return cudaErrorInvalidValue;
     }
   }
   switch (ppt_for(np)) {
-    case 1: return go_step<PolMixed64, 1>(a, ctas, stream);
-    case 2: return go_step<PolMixed64, 2>(a, ctas, stream);
-    case 4: return go_step<PolMixed64, 4>(a, ctas, stream);
-    case 8: return go_step<PolMixed64, 8>(a, ctas, stream);
-    case 16: return go_step<PolMixed64, 16>(a, ctas, stream);
+    case 1: return go_step<StepMixed64, 1>(a, ctas, stream);
+    case 2: return go_step<StepMixed64, 2>(a, ctas, stream);
+    case 4: return go_step<StepMixed64, 4>(a, ctas, stream);
+    case 8: return go_step<StepMixed64, 8>(a, ctas, stream);
+    case 16: return go_step<StepMixed64, 16>(a, ctas, stream);
     default: return cudaErrorInvalidValue;
   }
 }

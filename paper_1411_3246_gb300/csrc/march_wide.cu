@@ -41,8 +41,10 @@ int wide_occupancy(int n1) {
   return per_sm;
 }
 
+using StepWide = StepOf<PolWide>;
+
 size_t step_wide_smem(int n1) {
-  return ((MarchSmem<PolWide>::bytes(n1, kWideNT * kWidePPT) + 63) & ~(size_t)63) + 64;
+  return ((MarchSmem<StepWide>::bytes(n1, kWideNT * kWidePPT) + 63) & ~(size_t)63) + 64;
 }
 
 }  // namespace
@@ -57,11 +59,11 @@ size_t step_wide_window_bytes(int n1) { return sizeof(float) * 12 * (size_t)n1; 
 
 template <int NT>
 static size_t step_wide_smem_nt(int n1) {
-  return ((MarchSmem<PolWide>::bytes(n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
+  return ((MarchSmem<StepWide>::bytes(n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
 }
 template <int NT>
 static int step_wide_ctas(int n1) {
-  auto kern = step_wide_kernel<PolWide, NT, kWidePPT>;
+  auto kern = step_wide_kernel<StepWide, NT, kWidePPT>;
   const size_t smem = step_wide_smem_nt<NT>(n1);
   if (smem > kMaxSmemPerCta || n1 > PolWide::kScanE * NT) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -73,7 +75,7 @@ static int step_wide_ctas(int n1) {
 }
 template <int NT>
 static cudaError_t step_wide_launch(const PipeArgs &a, int ctas, cudaStream_t stream) {
-  auto kern = step_wide_kernel<PolWide, NT, kWidePPT>;
+  auto kern = step_wide_kernel<StepWide, NT, kWidePPT>;
   const size_t smem = step_wide_smem_nt<NT>(a.d.nr + 1);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -114,7 +116,7 @@ size_t step_wide_cluster_ring_bytes(int np, int cn) {
   return (size_t)cn * wide_share_bytes<float, kWideNT, kWidePPT>((np + cn - 1) / cn);
 }
 int step_wide_cluster_max(int n1, int cn) {
-  auto kern = step_wide_cluster_kernel<PolWide, kWideNT, kWidePPT>;
+  auto kern = step_wide_cluster_kernel<StepWide, kWideNT, kWidePPT>;
   const size_t smem = step_wide_smem(n1);
   if (smem > kMaxSmemPerCta || n1 > PolWide::kScanE * kWideNT) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -125,7 +127,7 @@ int step_wide_cluster_max(int n1, int cn) {
   return cudaOccupancyMaxActiveClusters(&n, kern, &c) == cudaSuccess ? n : 0;
 }
 cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cudaStream_t stream) {
-  auto kern = step_wide_cluster_kernel<PolWide, kWideNT, kWidePPT>;
+  auto kern = step_wide_cluster_kernel<StepWide, kWideNT, kWidePPT>;
   const size_t smem = step_wide_smem(a.d.nr + 1);
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -140,8 +142,8 @@ cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cu
 // The batched pipelined kernel in CTAs of bnt = 512 or 256 threads (the latter two per SM).
 template <int NT>
 static int batch_ctas(int max_n1) {
-  auto kern = batch_step_kernel<PolWide, NT, kWidePPT>;
-  const size_t smem = ((MarchSmem<PolWide>::bytes(max_n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
+  auto kern = batch_step_kernel<StepWide, NT, kWidePPT>;
+  const size_t smem = ((MarchSmem<StepWide>::bytes(max_n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
   if (smem > kMaxSmemPerCta || max_n1 > PolWide::kScanE * NT) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int per_sm = 0, dev = 0, sms = 0;
@@ -152,8 +154,8 @@ static int batch_ctas(int max_n1) {
 }
 template <int NT>
 static cudaError_t batch_launch(const BatchArgs &b, int max_n1, int ctas, cudaStream_t stream) {
-  auto kern = batch_step_kernel<PolWide, NT, kWidePPT>;
-  const size_t smem = ((MarchSmem<PolWide>::bytes(max_n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
+  auto kern = batch_step_kernel<StepWide, NT, kWidePPT>;
+  const size_t smem = ((MarchSmem<StepWide>::bytes(max_n1, NT * kWidePPT) + 63) & ~(size_t)63) + 64;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   BatchArgs arg = b;

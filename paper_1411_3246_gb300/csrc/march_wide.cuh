@@ -189,10 +189,15 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
   };
   // 1/Gamma of stage 1 and u_theta of the slice's state
   auto frame_of = [&](int sl, R r, R &iG, R &ut) {
-    const bool off = r > tiny_r<R>();
-    R ir;
-    rcp_pair(rs.G1[sl], off ? r : (R)1, iG, ir);
-    ut = off ? rs.lz[sl] * ir : (R)0;
+    if (Pol::kPlain) {
+      iG = rcp_of(rs.G1[sl]);
+      ut = r > (R)0 ? rs.lz[sl] / r : (R)0;
+    } else {
+      const bool off = r > tiny_r<R>();
+      R ir;
+      rcp_pair(rs.G1[sl], off ? r : (R)1, iG, ir);
+      ut = off ? rs.lz[sl] * ir : (R)0;
+    }
   };
   auto midpoint_abs = [&](int sl, int &c, R &f, R &u_r, R &u_t) -> R {
     const int c0 = rs.c[sl];
@@ -211,7 +216,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
   // charge of the initial slice = the ion background
   for (int ch = 0; ch < nch; ++ch) {
     const int b0 = ch * SLOTS, npc = chunk_np(ch);
-    ChargeWin<Pol, win_cells(PPT)> acc;
+    ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
     acc.init(-8);
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
@@ -258,7 +263,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     for (int ch = 0; ch < nch; ++ch) {
       const int b0 = ch * SLOTS, npc = chunk_np(ch);
-      ChargeWin<Pol, win_cells(PPT)> acc;
+      ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -324,7 +329,7 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
     for (int i = tid; i < n1; i += NT) sm.jz[i] = sm.chi[i] = sm.T[i] = sm.P[i] = sm.U[i] = sm.K[i] = (Acc)0;
     for (int ch = 0; ch < nch; ++ch) {
       const int b0 = ch * SLOTS, npc = chunk_np(ch);
-      ChargeWin<Pol, win_cells(PPT)> acc;
+      ChargeWin<Pol, win_cells<Pol>(PPT)> acc;
       acc.init(-8);
       unsigned miss = 0u;
 #pragma unroll
@@ -342,7 +347,14 @@ __device__ __forceinline__ void march_body_wide(const SimDesc &d, unsigned char 
           frame_of(sl, r, iG1, ut);
           const R xh = r + (R)0.5 * h * ur0 * iG1, yh = (R)0.5 * h * ut * iG1, h2 = xh * xh + yh * yh;
           const R uxh = ur0 + (R)0.5 * h * F1v;
-          if (h2 > tiny_r2<R>()) {
+          if constexpr (Pol::kPlain) {
+            const R rh = sqrt(h2);
+            if (rh > (R)0) {
+              const R irh = (R)1 / rh;
+              ex = xh * irh;
+              ey = yh * irh;
+            }
+          } else if (h2 > tiny_r2<R>()) {
             R rh, irh;
             root_of(h2, rh, irh);
             ex = xh * irh;

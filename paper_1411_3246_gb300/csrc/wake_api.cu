@@ -375,7 +375,7 @@ int probe_tile(wake_sim *h, const Sim &s, const SimDesc &d, const TileFns &f, do
 // 5.8 / 6.0, 1536 8.7 / 7.7 / 6.4, 4096 69.5 / 58.8 / 41.8): 4 from 1024 rings and 8 from 1536, and only
 // while half of the SMs stay free for other streams' work, since a cluster does more work in all.
 int pick_cluster(wake_sim *h, const wake_sim::TileClass &k, int count, bool step) {
-  if (h->tile_nt_forced || h->precision == WAKE_MIXED64) return 1;
+  if (h->tile_nt_forced || h->precision == WAKE_MIXED64 || (h->precision == WAKE_MIXED && !step)) return 1;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
