@@ -27,15 +27,12 @@ __global__ void __launch_bounds__(kNT, 1) march_wide_g_kernel(const SimDesc *des
 }
 
 __global__ void __launch_bounds__(kNT, 1) step_wide_g_kernel(PipeArgs a) {
-  __shared__ int ctl[2];
+  __shared__ int ctl[kCtlWords];
   const int n1 = a.d.nr + 1;
   double *win = (double *)((unsigned char *)a.win_bufs + (size_t)blockIdx.x * a.win_stride);
   unsigned char *rb = (unsigned char *)a.ring_bufs + (size_t)blockIdx.x * a.ring_stride;
   for (int t = blockIdx.x; t < a.nsteps; t += gridDim.x) {
-    if (threadIdx.x == 0) {
-      ctl[0] = 0;
-      ctl[1] = 0;
-    }
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<PW, kNT> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;

@@ -83,6 +83,13 @@ __device__ __forceinline__ void red_release(int *p) {
   asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
 
+// A CTA's control words (PipeHooks::ctl), in shared memory of every step kernel: cleared before each
+// step; the caller's barrier follows.
+constexpr int kCtlWords = 8;
+__device__ __forceinline__ void ctl_clear(int *ctl) {
+  if (threadIdx.x < kCtlWords) ctl[threadIdx.x] = 0;
+}
+
 // kCl: one step is marched by the CTAs of a cluster (march.cuh); every CTA holds the step's field
 // window and pushes its share of each cell.  progress[t] then counts the CTAs' finished cells: no
 // CTA finishes cell b + 1 before all have finished cell b (cluster barriers lie between), so a count
@@ -102,7 +109,7 @@ struct PipeHooks {
   const PipeArgs &a;
   int t;          // step within the launch
   R *win;         // 4 slices x (E_r, E_z, B_theta) x n1
-  int *ctl;       // [0] abort flag, [1] progress seen of step t-1, [2] [3] the next-cell entries of
+  int *ctl;       // kCtlWords: [0] abort flag, [1] progress seen of step t-1, [2] [3] the next-cell entries of
                   // the cell pushed last; clusters also [4] second-list entries, [6] [7] this
                   // CTA's abort flag as its peers read it, by the row's parity
   int n1, nr, nxi;
@@ -377,12 +384,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(PipeArgs a) {
     ctl = (int *)(win + (size_t)12 * n1);
   }
   for (int t = blockIdx.x; t < a.nsteps; t += gridDim.x) {
-    if (threadIdx.x == 0) {
-      ctl[0] = 0;
-      ctl[1] = 0;
-      ctl[2] = 0;  // the next-cell list entries of the cell pushed last
-      ctl[3] = 0;
-    }
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<Pol, NT, false, kCorn> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(NT, 2) step_cluster_kernel(PipeArgs a) {
   R *win = (R *)(smem_raw + base);
   int *ctl = (int *)(win + (size_t)12 * n1);
   for (int t = blockIdx.x / cn; t < a.nsteps; t += gridDim.x / cn) {
-    if (threadIdx.x < 8) ctl[threadIdx.x] = 0;
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<Pol, NT, true> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
@@ -424,12 +426,7 @@ __global__ void __launch_bounds__(NT, (NT < 512 ? 512 / NT : 1)) step_wide_kerne
   int *ctl = (int *)(smem_raw + base);
   R *win = (R *)((unsigned char *)a.win_bufs + (size_t)blockIdx.x * a.win_stride);
   for (int t = blockIdx.x; t < a.nsteps; t += gridDim.x) {
-    if (threadIdx.x == 0) {
-      ctl[0] = 0;
-      ctl[1] = 0;
-      ctl[2] = 0;  // the next-cell list entries of the cell pushed last
-      ctl[3] = 0;
-    }
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<Pol, NT> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
@@ -450,7 +447,7 @@ __global__ void __launch_bounds__(NT, 1) step_wide_cluster_kernel(PipeArgs a) {
   int *ctl = (int *)(smem_raw + base);
   R *win = (R *)((unsigned char *)a.win_bufs + (size_t)blockIdx.x * a.win_stride);
   for (int t = blockIdx.x / cn; t < a.nsteps; t += gridDim.x / cn) {
-    if (threadIdx.x < 8) ctl[threadIdx.x] = 0;
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<Pol, NT, true> hk{a, t, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
@@ -488,12 +485,7 @@ __global__ void __launch_bounds__(NT, (NT < 512 ? 512 / NT : 1)) batch_step_kern
     const size_t base = (MarchSmem<Pol>::bytes(n1, NT * PPT) + 63) & ~(size_t)63;
     int *ctl = (int *)(smem_raw + base);
     R *win = (R *)((unsigned char *)b.win_bufs + (size_t)blockIdx.x * b.win_stride);
-    if (threadIdx.x == 0) {
-      ctl[0] = 0;
-      ctl[1] = 0;
-      ctl[2] = 0;  // the next-cell list entries of the cell pushed last
-      ctl[3] = 0;
-    }
+    ctl_clear(ctl);
     __syncthreads();
     PipeHooks<Pol, NT> hk{a, it.y, win, ctl, n1, a.d.nr, a.d.nxi, a.d.dr, a.d.dxi, a.d.rmax, a.d.ximax};
     SimDesc d = a.d;
