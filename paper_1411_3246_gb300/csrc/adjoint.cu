@@ -251,7 +251,6 @@ __global__ void __launch_bounds__(kNT, 1) adj_fwd_pipe_kernel(AdjPipe a) {
   W.carve(sm, a.m.g.nr + 1);
   __shared__ int bad, ctl[1];
   const int nxi = a.m.g.nxi, n1 = a.m.g.nr + 1;
-  const double dxi = a.bc.b.dxi;
   for (int t = blockIdx.x; t < a.nsteps; t += gridDim.x) {
     if (P.tid == 0) {
       bad = 0;
@@ -276,9 +275,7 @@ __global__ void __launch_bounds__(kNT, 1) adj_fwd_pipe_kernel(AdjPipe a) {
       for (int i = a.cstart[b] + P.tid; i < a.cstart[b + 1]; i += P.nt) {
         const int64_t j = a.order[i];
         if (b < nxi && !rd(s0.lost + j)) {
-          int kk;
-          double gg;
-          cell_of(rd(s0.xi + j), dxi, nxi, kk, gg);
+          const int kk = cell_xi(a.bc.b, rd(s0.xi + j));
           if (kk != b && kk != b + 1) {  // its fields are not solved yet: flag, keep the state
             atomicOr(a.m.status, kAdjDrift);
             s1.x[j] = rd(s0.x + j); s1.y[j] = rd(s0.y + j); s1.ux[j] = rd(s0.ux + j);
@@ -315,7 +312,6 @@ __global__ void __launch_bounds__(kNT, 1) adj_rev_pipe_kernel(AdjPipe a) {
   W.carve(sm, a.m.g.nr + 1);
   __shared__ int bad, ctl[2];
   const int nxi = a.m.g.nxi;
-  const double dxi = a.bc.b.dxi;
   const int64_t n = a.bc.n;
   const Beam lam{a.lam, a.lam + n, a.lam + 2 * n, a.lam + 3 * n, a.lam + 4 * n, a.lam + 5 * n, nullptr};
   for (int it = blockIdx.x; it < a.nsteps; it += gridDim.x) {
@@ -345,9 +341,7 @@ __global__ void __launch_bounds__(kNT, 1) adj_rev_pipe_kernel(AdjPipe a) {
       for (int i = a.cstart[b] + P.tid; i < a.cstart[b + 1]; i += P.nt) {
         const int64_t j = a.order[i];
         if (s0.lost[j]) continue;
-        int kk;
-        double gg;
-        cell_of(s0.xi[j], dxi, nxi, kk, gg);
+        const int kk = cell_xi(a.bc.b, s0.xi[j]);
         if (kk != b && kk != b + 1) {
           atomicOr(a.m.status, kAdjDrift);
           continue;
@@ -408,11 +402,7 @@ __global__ void adj_slip_kernel(BeamConst c, Beam s, unsigned long long *out) {
 }
 // Counting sort of the particles by the xi cell of a state (lost: cell nxi).
 __device__ __forceinline__ int adj_cell(const BeamConst &c, const Beam &s, int64_t j) {
-  if (s.lost[j]) return c.b.nxi;
-  int k;
-  double g;
-  cell_of(s.xi[j], c.b.dxi, c.b.nxi, k, g);
-  return k;
+  return s.lost[j] ? c.b.nxi : cell_xi(c.b, s.xi[j]);
 }
 __global__ void adj_cell_count_kernel(BeamConst c, Beam s, int *count) {
   GRID_LOOP(j, c.n) atomicAdd(&count[adj_cell(c, s, j)], 1);
@@ -624,13 +614,14 @@ int wake_adjoint_init(const wake_params *p, int nsteps, int nbins, void *stream,
   a->nbins = nbins;
   a->stream = (cudaStream_t)stream;
   const int n1 = p->nr + 1, np = p->nr * p->ppc;
-  a->g = Dims{p->nr, p->nxi, np, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->nr / p->rmax};
+  a->g = Dims{p->nr, p->nxi, np, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, 1.0 / (p->rmax / p->nr)};
   a->B = std::max(1, (int)std::lround(std::sqrt((double)(p->nxi + 1))));
   a->nblk = (p->nxi + 1 + a->B - 1) / a->B;
   a->bc.n = p->n_beam;
   a->bc.n_drive = p->n_drive;
   a->bc.nbins = nbins;
-  a->bc.b = BoundsRZ{p->nr, p->nxi, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->ximax, p->nr / p->rmax, p->nxi / p->ximax};
+  a->bc.b = BoundsRZ{p->nr, p->nxi, p->rmax / p->nr, p->ximax / p->nxi, p->rmax, p->ximax,
+                     1.0 / (p->rmax / p->nr), 1.0 / (p->ximax / p->nxi)};
   a->bc.dt = p->ds;
   a->bc.gamma_b = p->gamma_b;
   a->ng = (size_t)(p->nxi + 1) * n1;

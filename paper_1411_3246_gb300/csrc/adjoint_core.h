@@ -12,6 +12,8 @@
 #include <cmath>
 #include <cstdint>
 
+#include "fp64_arith.h"
+
 #if defined(__CUDACC__)
 #define ADJ_HD __host__ __device__
 #else
@@ -124,7 +126,7 @@ ADJ_HD void par_scan(const Par &P, int n, bool reverse, In in, Out out) {
 struct Dims {
   int nr, nxi, np;
   double dr, dxi, R;
-  double inv_dr = 0.0;  // 1/dr where the caller has it (0: formed when needed)
+  double inv_dr = 0.0;  // 1.0 / dr where the caller has it (0: formed when needed)
   ADJ_HD double idr() const { return inv_dr > 0.0 ? inv_dr : 1.0 / dr; }
 };
 
@@ -132,16 +134,11 @@ ADJ_HD inline double vol(int i, int nr, double dr) {
   return i == 0 ? dr * dr / 6.0 : (i == nr ? dr * ((double)nr * dr / 2.0 - dr / 6.0) : (double)i * dr * dr);
 }
 ADJ_HD inline double alpha(int m, int nr) { return m == nr ? 1.0 : 0.5 - rcp(6.0 * (double)m); }
-// The same with 1/dr: on the device the quotient r/dr costs five FP64 instructions.
-ADJ_HD inline void cell_at(double r, double idr, int nr, int &c, double &f) {
-  const double s = r * idr;
-  int i = (int)floor(s);
-  i = i < 0 ? 0 : (i > nr - 1 ? nr - 1 : i);
-  c = i;
-  f = s - (double)i;
-}
-ADJ_HD inline void cell_of(double r, double dr, int nr, int &c, double &f) {
-  const double s = r / dr;
+// The cell of a coordinate r, its offset in it: the one place that finds cells, in r and in xi, for the
+// beam's order, its deposit, its push and the plasma alike (a particle on a node must lie in the same
+// cell for all of them: the pipelined steps read and add to the rows of that cell only).
+ADJ_HD inline void cell_at(double r, double dr, double idr, int nr, int &c, double &f) {
+  const double s = quot64(r, dr, idr);
   int i = (int)floor(s);
   i = i < 0 ? 0 : (i > nr - 1 ? nr - 1 : i);
   c = i;
@@ -325,7 +322,7 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_at(R.r[j], idr, nr, c, f);
+    cell_at(R.r[j], dr, idr, nr, c, f);
     add_to(&S.rho[c], w[j] * (1.0 - f));
     add_to(&S.rho[c + 1], w[j] * f);
   }
@@ -347,7 +344,7 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
     const double r = R.r[j], ur = R.ur[j], ut = R.ut[j];
     int c;
     double f;
-    cell_at(r, idr, nr, c, f);
+    cell_at(r, dr, idr, nr, c, f);
     const double Gam = G0[j] + interp(S.psi, c, f);
     if (!(Gam > 0.0)) *bad = 1;
     const double up2 = ur * ur + ut * ut;
@@ -409,7 +406,7 @@ ADJ_HD inline void stage_forward(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_at(R.r[j], idr, nr, c, f);
+    cell_at(R.r[j], dr, idr, nr, c, f);
     const double bf = interp(S.bth, c, f);
     R.bf[j] = bf;
     Fc[j] = R.gam[j] * rcp(R.Gam[j]) * R.dp[j] - bf;
@@ -446,7 +443,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_at(R.r[j], idr, nr, c, f);
+    cell_at(R.r[j], dr, idr, nr, c, f);
     const double iG = rcp(R.Gam[j]), gam = R.gam[j], dp = R.dp[j], lFj = lF[j];
     lgam_s[j] = lFj * dp * iG;
     lGam_s[j] = lG[j] - lFj * gam * dp * iG * iG;
@@ -524,7 +521,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
     const double r = R.r[j], ur = R.ur[j], ut = R.ut[j];
     int c;
     double f;
-    cell_at(r, idr, nr, c, f);
+    cell_at(r, dr, idr, nr, c, f);
     const double Gam = R.Gam[j], gam = R.gam[j], dp = R.dp[j], uz = gam - Gam, wj = w[j];
     const bool off = r > kTinyR;
     const double rs = off ? r : 1.0, t0 = rcp(Gam * rs);
@@ -598,7 +595,7 @@ ADJ_HD inline void stage_reverse(const Par &P, const Dims &g, const Rings &R, co
   for (int j = P.tid; j < np; j += P.nt) {
     int c;
     double f;
-    cell_at(R.r[j], idr, nr, c, f);
+    cell_at(R.r[j], dr, idr, nr, c, f);
     lw[j] += W.l_rho[c] * (1.0 - f) + W.l_rho[c + 1] * f;
     lr[j] += w[j] * (W.l_rho[c + 1] - W.l_rho[c]) * idr;
   }
@@ -799,8 +796,15 @@ struct BoundsRZ {
 
 // Bilinear node weights of a point: cell (c, k), offsets (f, g).
 ADJ_HD inline void cell_rz(const BoundsRZ &b, double r, double xi, int &c, double &f, int &k, double &gg) {
-  cell_at(r, b.idr(), b.nr, c, f);
-  cell_at(xi, b.idxi(), b.nxi, k, gg);
+  cell_at(r, b.dr, b.idr(), b.nr, c, f);
+  cell_at(xi, b.dxi, b.idxi(), b.nxi, k, gg);
+}
+// The xi cell alone.
+ADJ_HD inline int cell_xi(const BoundsRZ &b, double xi) {
+  int k;
+  double gg;
+  cell_at(xi, b.dxi, b.idxi(), b.nxi, k, gg);
+  return k;
 }
 
 // Boris step with the fields (Er, Ez, Bt) at the particle.  In/out: x, y, ux, uy, uz, xi.
@@ -1414,7 +1418,7 @@ ADJ_HD inline double rho0_node(const Dims &g, const double *r0, const double *w,
   for (int j = 0; j < g.np; ++j) {
     int c;
     double f;
-    cell_of(r0[j], g.dr, g.nr, c, f);
+    cell_at(r0[j], g.dr, g.idr(), g.nr, c, f);
     if (c == i) s += w[j] * (1.0 - f);
     if (c + 1 == i) s += w[j] * f;
   }
@@ -1452,7 +1456,7 @@ ADJ_HD inline double theta_ring_one(const Dims &g, const double *nm_p, const dou
   const double dw = base * (dG0 * g0 - G0 * dg0) / (g0 * g0);
   int cc;
   double f;
-  cell_of(r0[j], g.dr, g.nr, cc, f);
+  cell_at(r0[j], g.dr, g.idr(), g.nr, cc, f);
   const double lwj = lw_p[j] + lrho0[cc] * (1.0 - f) + lrho0[cc + 1] * f;
   return lur0[j] * nr_ + ll[j] * r0[j] * nt + lG0[j] * dG0 + lwj * dw;
 }
