@@ -6,7 +6,9 @@
 //
 // The code is plain C++ with __host__ __device__ qualifiers.  Block-parallel loops go through
 // Par (thread index, thread count, barrier): a CUDA block runs them with its threads, the
-// host with one "thread", so the same arithmetic can be checked on a CPU.
+// host with one "thread", so the formulas can be checked on a CPU.  Two parts are the device's own:
+// fp64_arith.h (the host takes plain operations) and the tridiagonal solve (tri_solve: the host
+// eliminates row by row).
 #pragma once
 
 #include <cmath>
@@ -14,11 +16,7 @@
 
 #include "fp64_arith.h"
 
-#if defined(__CUDACC__)
-#define ADJ_HD __host__ __device__
-#else
-#define ADJ_HD
-#endif
+#define ADJ_HD WAKE_HD
 
 namespace wake {
 namespace adj {
@@ -35,34 +33,9 @@ struct Par {
 // v is finite (not NaN or infinite): v - v is 0 exactly then.
 ADJ_HD inline bool finite(double v) { return v - v == 0.0; }
 
-// 1/x, and sqrt(x) with its reciprocal (x > 0).  GB300's FP64 pipe is the adjoint's bound: on the
-// device they are the hardware's approximation (about 20 bits) and one third-order Newton step,
-// with e = 1 - x r:  r (1 + e + e^2), and with e = 1 - x y^2:  y (1 + e/2 + 3 e^2 / 8), the root corrected
-// once; an ulp or so, at a third of the instructions of the IEEE operations.
-ADJ_HD inline double rcp(double x) {
-#ifdef __CUDA_ARCH__
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-#else
-  return 1.0 / x;
-#endif
-}
-ADJ_HD inline void root(double x, double &r, double &ir) {
-#ifdef __CUDA_ARCH__
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  y = fma(fma(0.375, e, 0.5), e * y, y);
-  const double g = x * y;
-  r = fma(fma(-g, g, x), 0.5 * y, g);
-  ir = y;
-#else
-  r = sqrt(x);
-  ir = 1.0 / r;
-#endif
-}
+// GB300's FP64 pipe is the adjoint's bound: reciprocals, roots and quotients by fp64_arith.h.
+ADJ_HD inline double rcp(double x) { return rcp64(x); }
+ADJ_HD inline void root(double x, double &r, double &ir) { root64(x, r, ir); }
 constexpr double kTinyR = 1e-145, kTinyR2 = 1e-290;  // smaller radii count as the axis
 
 // A load of a value another CTA may have written in the same launch (the pipelined steps):

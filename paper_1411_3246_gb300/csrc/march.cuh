@@ -29,6 +29,7 @@
 // wide type: FP64, or float-float pairs on the FP32 pipe.
 #pragma once
 
+#include "fp64_arith.h"
 #include "wake_common.cuh"
 #include <type_traits>
 
@@ -85,41 +86,22 @@ __device__ __forceinline__ long long wide_shfl_idx(long long a, int l) { return 
 template <>
 __device__ __forceinline__ long long wide_zero<long long>() { return 0; }
 
-// 1/x.  FP32: the unit's division (a reciprocal instruction in the fast units).  FP64: the
-// hardware's approximation (about 20 bits) and one third-order Newton step r (1 + e + e^2),
-// e = 1 - x r, which leaves about an ulp: three FP64 instructions after the seed, where GB300's
-// narrow FP64 pipe makes an IEEE division cost three times as many.
+// 1/x, and 1/sqrt(x) (x > 0) with sqrt(x).  FP32: the unit's division and square root; FP64: fp64_arith.h.
 __device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
-__device__ __forceinline__ double rcp_of(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
-// 1/sqrt(x) (x > 0) and sqrt(x).  FP32: the unit's square root and division.  FP64: the
-// hardware's approximation y and one third-order Newton step y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2;
-// the root x y is corrected once.
+__device__ __forceinline__ double rcp_of(double x) { return rcp64(x); }
 __device__ __forceinline__ void root_of(float x, float &r, float &ir) {
   r = sqrtf(x);
   ir = 1.0f / r;
 }
-__device__ __forceinline__ void root_of(double x, double &r, double &ir) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  y = fma(fma(0.375, e, 0.5), e * y, y);
-  const double g = x * y;
-  r = fma(fma(-g, g, x), 0.5 * y, g);
-  ir = y;
-}
+__device__ __forceinline__ void root_of(double x, double &r, double &ir) { root64(x, r, ir); }
 // The smallest square, and the smallest radius, that the reciprocals above take (FP64: the
 // approximations flush what is near the underflow; smaller counts as the axis).
 template <class R>
 __device__ __forceinline__ constexpr R tiny_r2() { return sizeof(R) == 8 ? (R)1e-290 : (R)0; }
 template <class R>
 __device__ __forceinline__ constexpr R tiny_r() { return sizeof(R) == 8 ? (R)1e-145 : (R)0; }
-// 1/a and 1/b: in FP64 from one reciprocal of the product (the FP64 pipe is the march's bound).
+// 1/a and 1/b: in FP64 from one reciprocal of the product (the FP64 pipe is the march's bound), three
+// roundings each.
 __device__ __forceinline__ void rcp_pair(float a, float b, float &ia, float &ib) {
   ia = rcp_of(a);
   ib = rcp_of(b);
