@@ -203,7 +203,7 @@ struct PolFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kPlain = false;
+  static constexpr bool kPlain = false, kStep = false;
   static constexpr int kScanE = 3;  // nodes per thread in the block scans: n1 <= kScanE * NT
 };
 struct PolMixed {
@@ -220,7 +220,7 @@ struct PolMixed {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kPlain = true;
+  static constexpr bool kPlain = true, kStep = false;
   static constexpr int kScanE = 3;
 };
 // The precision split in which only the particle arithmetic is FP32: each ring's push and its
@@ -241,7 +241,7 @@ struct PolMixed64 {
   static constexpr bool kWinGlobal = true;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = true;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kPlain = true;
+  static constexpr bool kPlain = true, kStep = false;
   static constexpr int kScanE = 3;
 };
 // The mixed arithmetic for boxes too large for one CTA's shared memory to hold the rings
@@ -261,7 +261,7 @@ struct PolWide {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kPlain = true;
+  static constexpr bool kPlain = true, kStep = false;
   static constexpr int kScanE = 5;
 };
 
@@ -282,13 +282,13 @@ struct PolWideFP64 {
   static constexpr bool kWinGlobal = false;
   static constexpr bool kSlab = false;  // geometry: see SlabOf
   static constexpr bool kDeferMisses = false;  // out-of-window rings deposited after the ring loops
-  static constexpr bool kPlain = false;
+  static constexpr bool kPlain = false, kStep = false;
   static constexpr int kScanE = 5;
 };
 // A policy in the pipelined beam steps.
 template <class P>
 struct StepOf : P {
-  static constexpr bool kPlain = false;
+  static constexpr bool kPlain = false, kStep = true;
 };
 // A policy marched by clusters of narrower CTAs (march_cluster_*.cu).
 template <class P>
@@ -305,12 +305,8 @@ struct SlabOf : P {
   static constexpr bool kSlab = true;
 };
 
-// Rows per lane of the tridiagonal solve (tri_solve_warp) of n rows, and the length of its arrays.
+// Rows per lane of the tridiagonal solve (tri_solve_warp) of n rows.
 __host__ __device__ constexpr int tri_per_lane(int n) { return (n + 31) >> 5; }
-__host__ __device__ constexpr int tri_len(int n) { return 33 * ((n + 31) >> 5); }
-// Entries of a tridiagonal row array for n1 nodes.
-template <class Pol>
-__host__ __device__ constexpr int row_len(int n1) { return Pol::kPlain ? n1 + 32 : tri_len(n1); }
 
 // Ring slot arrays: cell index, offset in the cell, u_r, the constants l_z, Gamma_0, w, and
 // the stage-1 Gamma and radial force kept for the full step; with ids, each slot also carries
@@ -348,6 +344,7 @@ struct MarchSmem {
   N *psi, *dpsi, *ez, *bth;                     // node fields
   R *nb0, *nb1;                                 // beam-density rows (double buffer)
   N *ta, *tb, *tc, *td;                         // tridiagonal rows (a, row sum, c, rhs)
+  int ts;                                       // their stride (tri_stride)
   N *invR, *invV, *alpha, *ga, *gb, *gc;        // tables (FP64 form; the mixed forms keep
                                                 // invR = 1/(m dr) and ga = 1/(j + 1/2) only)
   int *cnt;                                     // re-sort counts
@@ -355,13 +352,36 @@ struct MarchSmem {
   typename Pol::W *wtot;                        // block-scan warp totals
   RingSoA<R> rings;                             // ring slots (mixed form)
 
-  __host__ __device__ static size_t bytes(int n1, int slots, bool ids = false) {
+  // all but the tridiagonal rows
+  __host__ __device__ static size_t fixed_bytes(int n1, int slots, bool ids) {
     size_t b = sizeof(typename Pol::W) * 64 + sizeof(typename Pol::Q) * 2 * (size_t)n1 + sizeof(Acc) * 6 * (size_t)n1 +
-               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + sizeof(N) * 4 * (size_t)row_len<Pol>(n1) + 256;
+               sizeof(N) * 4 * (size_t)n1 + sizeof(R) * 2 * (size_t)n1 + 256;
     b += sizeof(N) * (Pol::kTables ? 6 : 2) * (size_t)n1;
     if (Pol::kSortEvery > 0) b += sizeof(int) * ((size_t)n1 + 32);
     if (Pol::kSmemRings) b += RingSoA<R>::bytes(slots, ids) + 32;
     return b + 64;
+  }
+  // What a pipelined step keeps in shared memory beside it: its field window (the tiles), control words.
+  __host__ __device__ static size_t step_bytes(int n1) {
+    return Pol::kStep ? 128 + (Pol::kSmemRings && !Pol::kWinGlobal ? sizeof(R) * 12 * (size_t)n1 : 0) : 0;
+  }
+  // One-warp solve: entries between rows of the same lane, 33, which spreads the rows' writers over the
+  // banks (TriAt), where that fits shared memory, else 32: the row arrays are then no longer than n1 +
+  // 32, so what fits does not hang on the padding.
+  __host__ __device__ static int tri_stride(int n1, int slots, bool ids) {
+    const size_t b = fixed_bytes(n1, slots, ids) + sizeof(N) * 4 * 33 * (size_t)tri_per_lane(n1 - 1);
+    return b + step_bytes(n1) <= kMaxSmemPerCta ? 33 : 32;
+  }
+  __host__ __device__ static int row_len(int n1, int slots, bool ids) {
+    return Pol::kPlain ? n1 + 32 : tri_stride(n1, slots, ids) * tri_per_lane(n1 - 1);
+  }
+  // Never less than for fewer nodes (a launch is sized for its largest simulation): all there is with
+  // the short stride.
+  __host__ __device__ static size_t bytes(int n1, int slots, bool ids = false) {
+    const size_t b = fixed_bytes(n1, slots, ids) + sizeof(N) * 4 * (size_t)row_len(n1, slots, ids);
+    if (Pol::kPlain || tri_stride(n1, slots, ids) == 33) return b;
+    const size_t most = kMaxSmemPerCta - step_bytes(n1);
+    return b < most ? most : b;
   }
   __device__ void carve(unsigned char *base, int n1, int slots, bool ids = false) {
     wtot = (typename Pol::W *)base;
@@ -380,10 +400,12 @@ struct MarchSmem {
     dpsi = rp; rp += n1;
     ez = rp; rp += n1;
     bth = rp; rp += n1;
-    ta = rp; rp += row_len<Pol>(n1);
-    tb = rp; rp += row_len<Pol>(n1);
-    tc = rp; rp += row_len<Pol>(n1);
-    td = rp; rp += row_len<Pol>(n1);
+    const int rl = row_len(n1, slots, ids);
+    ts = Pol::kPlain ? 0 : tri_stride(n1, slots, ids);
+    ta = rp; rp += rl;
+    tb = rp; rp += rl;
+    tc = rp; rp += rl;
+    td = rp; rp += rl;
     invR = invV = alpha = ga = gb = gc = nullptr;
     invR = rp; rp += n1;
     ga = rp; rp += n1;
@@ -409,7 +431,7 @@ struct MarchSmem {
   // The out-of-window ring queue: slot ids in the tridiagonal rows, which are free from the end
   // of one solve to the start of the next (a ring pass and the deposits that follow it)
   __device__ __forceinline__ int *queue() const { return (int *)ta; }
-  __device__ __forceinline__ int queue_cap(int n1) const { return (int)(4 * (size_t)row_len<Pol>(n1) * sizeof(N) / sizeof(int)); }
+  __device__ __forceinline__ int queue_cap() const { return (int)(4 * (size_t)(tb - ta) * sizeof(N) / sizeof(int)); }
 };
 
 // ---------------------------------------------------------------------------------------
@@ -567,28 +589,28 @@ __device__ __forceinline__ FF q_to_wide<long long, FF>(long long d) {
 // The two field solves of a slice, E_z scans and rows included, take 12.6k cycles at 257 nodes and
 // 7.1k at 129 (mixed); with the reduction over the block 18k at 513 nodes.
 //
-// Row q lies at tri_at(q) of each array: rows of the same index in consecutive lanes are adjacent,
-// 33 entries apart from the next index's, so the lanes' reads and the rows' writers (consecutive q)
-// both spread over the shared-memory banks.
+// Row q lies at TriAt(q) of each array: rows of the same index in consecutive lanes are adjacent, st
+// entries apart from the next index's (33: the lanes' reads and the rows' writers, consecutive q, both
+// spread over the shared-memory banks; 32 where that does not fit, MarchSmem::tri_stride).
 struct TriAt {
-  int E;
+  int E, st;
   unsigned m;  // ceil(2^32 / E): q / E for q < 2^16
-  __device__ __forceinline__ explicit TriAt(int n) : E(tri_per_lane(n)), m(0xffffffffu / (unsigned)tri_per_lane(n) + 1u) {}
+  __device__ __forceinline__ TriAt(int n, int stride) : E(tri_per_lane(n)), st(stride), m(0xffffffffu / (unsigned)tri_per_lane(n) + 1u) {}
   __device__ __forceinline__ int operator()(int q) const {
     const int lane = E == 1 ? q : (int)__umulhi((unsigned)q, m);
-    return (q - lane * E) * 33 + lane;
+    return (q - lane * E) * st + lane;
   }
 };
 
-// Called by one warp.  ta, ts, tc, td: the rows, 32 E of them (rows past n: a = c = d = 0, s = -1);
-// w: 3 tri_len(n) entries of scratch when E > 1.  out(q, x_q) receives the solution for q < n.
+// Called by one warp.  ta, ts, tc, td: the rows, 32 E of them (rows past n: a = c = d = 0, s = -1), st
+// their stride; w: 3 E st entries of scratch when E > 1.  out(q, x_q) receives the solution for q < n.
 template <class S, class Out>
-__device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S *tc, const S *td, S *w, int n, Out &&out) {
-  const int lane = threadIdx.x & 31, E = tri_per_lane(n), L = 33 * E;
+__device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S *tc, const S *td, S *w, int n, int st, Out &&out) {
+  const int lane = threadIdx.x & 31, E = tri_per_lane(n), L = st * E;
   S *wl = w, *wr = w + L, *wd = w + 2 * L;  // the downward rows: left coupling, 1/b, right-hand side
   S aq = ta[lane], sq = ts[lane], cq = tc[lane], dq = td[lane];
   if (E > 1) {
-    int u = (E - 2) * 33 + lane;  // the upward elimination starts at row E - 2
+    int u = (E - 2) * st + lane;  // the upward elimination starts at row E - 2
     S ua = ta[u], us = ts[u], ur = tc[u], ud = td[u], urb = rcp_of(us - ua - ur);
     S rb = rcp_of(sq - aq - cq);
     wl[lane] = aq;
@@ -597,7 +619,7 @@ __device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S
     int v = lane;
 #pragma unroll 2
     for (int e = 1; e < E; ++e) {
-      v += 33;
+      v += st;
       const S k = ta[v] * rb;
       sq = ts[v] - k * sq;
       dq = td[v] - k * dq;
@@ -608,7 +630,7 @@ __device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S
       wr[v] = rb;
       wd[v] = dq;
       if (e < E - 1) {
-        u -= 33;
+        u -= st;
         const S ku = tc[u] * urb;
         us = ts[u] - ku * us;
         ud = td[u] - ku * ud;
@@ -645,7 +667,7 @@ __device__ __forceinline__ void tri_solve_warp(const S *ta, const S *ts, const S
   if (q0 + E - 1 < n) out(q0 + E - 1, x);
 #pragma unroll 2
   for (int e = E - 2; e >= 0; --e) {
-    const int v = e * 33 + lane;
+    const int v = e * st + lane;
     x = (wd[v] - wl[v] * zl - tc[v] * x) * wr[v];
     if (q0 + e < n) out(q0 + e, x);
   }
@@ -879,7 +901,7 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
   // rows q = 0..nr-1 (node i = q + 1): central differences, a half cell at the wall; the one-warp
   // solve's rows past them up to whole lanes are -x = 0
   const R i2dr = (R)0.5 * inv_dr;
-  const TriAt at(nr);
+  const TriAt at(nr, sm.ts);
   const int nrows = Pol::kPlain ? nr : 32 * at.E;
   for (int q = tid; q < nrows; q += NT) {
     R a = (R)0, c = (R)0, s = (R)-1, rhs = (R)0;
@@ -903,12 +925,12 @@ __device__ __forceinline__ void solve_fields(MarchSmem<Pol> &sm, const NodeGeo<P
   }
   __syncthreads();
   // the solver's scratch reuses the six deposit arrays (contiguous, dead once the rows are set up,
-  // zeroed before the next pass B): the one-warp solve's 3 tri_len(nr) <= 6 (nr + 1) whenever nr > 32,
+  // zeroed before the next pass B): the one-warp solve's 99 ceil(nr / 32) <= 6 (nr + 1) whenever nr > 32,
   // the reduction's second buffer in four of them
   static_assert(sizeof(Acc) == sizeof(R), "the solver's scratch reuses the deposit arrays");
   auto out = [&](int q, R x) { sm.bth[q + 1] = x; };  // row q is node q + 1
   if constexpr (!Pol::kPlain) {
-    if (tid < 32) tri_solve_warp<R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, nr, out);
+    if (tid < 32) tri_solve_warp<R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, nr, sm.ts, out);
   } else if constexpr (Pol::kSmemRings) {
     pcr_rowsum_solve<NT, R>(sm.ta, sm.tb, sm.tc, sm.td, (R *)sm.jz, (R *)sm.chi, (R *)sm.T, (R *)sm.P, nr, out);
   } else {
@@ -1197,7 +1219,7 @@ __device__ __forceinline__ void queue_misses(MarchSmem<Pol> &sm, int n1, unsigne
     tot += __popc(mp[p]);
   }
   if (tot == 0) return;
-  const int lane = threadIdx.x & 31, cap = sm.queue_cap(n1);
+  const int lane = threadIdx.x & 31, cap = sm.queue_cap();
   int base = 0;
   if (lane == 0) base = atomicAdd(sm.qn, tot);
   base = __shfl_sync(kFull, base, 0);
@@ -1220,7 +1242,7 @@ __device__ __forceinline__ void queue_misses(MarchSmem<Pol> &sm, int n1, unsigne
 // ends the pass; contains a barrier when the queue is not empty.
 template <int NT, class Pol, class Fn>
 __device__ __forceinline__ void drain_queue(MarchSmem<Pol> &sm, int n1, Fn &&fn) {
-  const int n = min(*sm.qn, sm.queue_cap(n1));
+  const int n = min(*sm.qn, sm.queue_cap());
   if (n == 0) return;  // block-uniform
   constexpr int W = NT / 32;
   const int *q = sm.queue();

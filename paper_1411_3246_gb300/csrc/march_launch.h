@@ -10,8 +10,6 @@ namespace wake {
 
 struct PipeArgs;
 
-constexpr size_t kMaxSmemPerCta = 227 * 1024;
-
 // Precision forms, numbered as the library's WAKE_FP64, WAKE_MIXED and WAKE_MIXED64.
 enum Form : int { kFormFP64 = 0, kFormMixed = 1, kFormMixed64 = 2 };
 

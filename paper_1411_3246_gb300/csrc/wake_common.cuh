@@ -17,6 +17,9 @@ enum : int { ST_NUMERIC = 1, ST_ESCAPE = 2, ST_TIMEOUT = 4 };
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// Shared memory of one CTA at most (sm_103a).
+constexpr size_t kMaxSmemPerCta = 227 * 1024;
+
 // Everything one CTA needs about one simulation.  Grids are (nxi+1) x (nr+1), slice-major;
 // their element type is double (FP64) or float (mixed) as the kernel's policy says.
 struct SimDesc {
