@@ -64,7 +64,7 @@ def test_fp64_reciprocal_and_root(probe, lo, hi):
     """Against the IEEE division and root: the reciprocal and the root are the rounded value or its
     neighbour; the root's reciprocal is within two ulp of 1/sqrt, and numpy's, from a rounded root, within
     one: three."""
-    rng = np.random.default_rng(hi)
+    rng = np.random.default_rng(abs(hi))
     a = np.ldexp(rng.uniform(1, 2, 40000), rng.integers(lo, hi, 40000))
     a[:2000] = np.ldexp(1 + np.arange(-1000, 1000) * 2.0 ** -52, int(rng.integers(lo, hi)))  # around a power of two
     rcp, r, ir = _fp64(probe, a, np.ones_like(a))[:3]
