@@ -77,6 +77,7 @@ size_t ring_buf_bytes(int form);
 // Global field-window bytes per CTA the form's pipelined step needs (0: in shared memory).
 bool step_smem_ok(int form, int n1, int np);
 int step_max_ctas(int form, int n1, int np);
+int step_max_ctas_corners(int n1, int np);  // mixed, density grids by cells
 size_t step_global_window_bytes(int form, int n1);
 cudaError_t launch_step(int form, const PipeArgs &a, int np, int ctas, cudaStream_t stream);
 cudaError_t launch_step_mixed64(const PipeArgs &a, int np, int ctas, cudaStream_t stream);

@@ -37,9 +37,9 @@ static cudaError_t go_step(const PipeArgs &a, int ctas, cudaStream_t stream) {
   void *args[] = {&arg};
   return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(StepMixed::NT), args, smem, stream);
 }
-template <int PPT>
+template <int PPT, bool kCorn = false>
 static int ctas_step(int n1) {
-  auto kern = step_kernel<StepMixed, StepMixed::NT, PPT>;
+  auto kern = step_kernel<StepMixed, StepMixed::NT, PPT, kCorn>;
   const size_t smem = step_smem_bytes<StepMixed, StepMixed::NT, PPT>(n1);
   if (smem > 227 * 1024) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -99,6 +99,18 @@ int step_ctas_mixed(int n1, int np) {
     case 4: return ctas_step<4>(n1);
     case 8: return ctas_step<8>(n1);
     case 16: return ctas_step<16>(n1);
+    default: return 0;
+  }
+}
+
+// The same for the steps with density grids by cells (0: no such kernel).
+int step_max_ctas_corners(int n1, int np) {
+  if (step_bytes_for(n1, np) > 227 * 1024) return 0;
+  switch (ppt_for(np)) {
+    case 1: return ctas_step<1, true>(n1);
+    case 2: return ctas_step<2, true>(n1);
+    case 4: return ctas_step<4, true>(n1);
+    case 8: return ctas_step<8, true>(n1);
     default: return 0;
   }
 }

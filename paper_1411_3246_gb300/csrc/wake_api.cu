@@ -52,8 +52,8 @@ struct Sim {
   unsigned long long *slip = nullptr;  // largest xi slip rate of the beam (double bits)
   // pipelined steps: per-step beam-density grids, progress counters, per-CTA ring storage
   void *pgrids = nullptr;
-  int pgrid_cap = 0;
-  size_t pgrid_bytes = 0;  // of one of them
+  size_t pgrid_bytes = 0;  // all of them
+  int pstep_cap = 0;       // steps the progress and list counters hold
   int *progress = nullptr;
   void *pring = nullptr;
   size_t pring_bytes = 0;
@@ -211,6 +211,29 @@ int alloc_near(Sim &s, int cap, int ch) {
   const int rc = dalloc(&s.near_list, need);
   if (rc == WAKE_OK) s.near_bytes = need;
   return rc;
+}
+
+// Pipelined steps: at least `bytes` of density grids and counters for `steps` steps (they only grow: calls
+// of other lengths and other grid layouts share them).
+int alloc_steps(Sim &s, int steps, size_t bytes) {
+  int rc;
+  if (s.pgrid_bytes < bytes) {
+    if (s.pgrids) cudaFree(s.pgrids);
+    s.pgrids = nullptr;
+    s.pgrid_bytes = 0;
+    if ((rc = dalloc(&s.pgrids, bytes))) return rc;
+    s.pgrid_bytes = bytes;
+  }
+  if (s.pstep_cap < steps) {
+    if (s.progress) cudaFree(s.progress);
+    if (s.defer_cnt) cudaFree(s.defer_cnt);
+    s.progress = nullptr;
+    s.defer_cnt = nullptr;
+    s.pstep_cap = 0;
+    if ((rc = dalloc(&s.progress, sizeof(int) * steps)) || (rc = dalloc(&s.defer_cnt, 2 * sizeof(int) * steps))) return rc;
+    s.pstep_cap = steps;
+  }
+  return WAKE_OK;
 }
 
 // The beam arrays of simulation s for s.n_cap particles (any earlier ones freed).
@@ -1108,19 +1131,7 @@ int step_batch_pipelined(wake_sim *h, int nsteps) {
       Sim &s = h->sims[i];
       const size_t gbytes = sizeof(float) * s.ng;
       const int dcap = (int)std::min<int64_t>(s.p.n_beam, 4096);
-      if (s.pgrid_cap < ch + 1) {
-        void *old[] = {s.pgrids, s.progress, s.defer_cnt};
-        for (void *q : old)
-          if (q) cudaFree(q);
-        s.pgrids = nullptr;
-        s.progress = nullptr;
-        s.defer_cnt = nullptr;
-        s.pgrid_cap = 0;
-        if ((rc = dalloc(&s.pgrids, gbytes * (ch + 1))) || (rc = dalloc(&s.progress, sizeof(int) * ch)) ||
-            (rc = dalloc(&s.defer_cnt, 2 * sizeof(int) * ch)))
-          return rc;
-        s.pgrid_cap = ch + 1;
-      }
+      if ((rc = alloc_steps(s, ch, gbytes * (ch + 1)))) return rc;
       if (s.defer_bytes < sizeof(int2) * (size_t)dcap * ch) {
         if (s.defer_list) cudaFree(s.defer_list);
         s.defer_list = nullptr;
@@ -1311,19 +1322,27 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
   }
   const int fp64 = h->precision == WAKE_FP64;
   const size_t gs = gsize(h->precision);
-  // every step of a launch owns a density grid: up to a quarter of the free memory.  Mixed forms
-  // keep it by cells, four shares each (PipeArgs::corners), where the beam is dense enough for the
-  // deposits to count and a grid for every step fits: the OSIRIS set (5,000 particles per xi cell)
-  // takes 195 ms against 224 with four atomics a particle, the blowout run (512) 184 against 179 (a
-  // row read gathers four times the bytes).
+  // every step of a launch owns a density grid: up to a quarter of the free memory, the grids held from
+  // earlier calls counted as free, so that equal calls decide alike.  Mixed forms keep them by cells,
+  // four shares each (PipeArgs::corners), where the beam is dense enough for the deposits to count (a
+  // row read gathers four times the bytes) and a grid for every step fits.  170 steps with 500 / 1,000 /
+  // 1,500 / 2,000 / 2,600 / 3,500 / 5,000 particles per xi cell, four atomics against one: 128 x 600 cells
+  // 0.97 / 0.97 / 0.97 / 0.98 / 0.99 / 1.01 / 1.08 times as fast, 256 x 512 0.98 / 0.99 / 1.00 / 1.05 / 1.07 /
+  // 1.08 / 1.10, 200 x 500 0.98 / 0.99 / 1.04 / 1.07 / 1.09 / 1.12 / 1.14, 420 x 400 0.99 / 1.04 / 1.08 / 1.10 /
+  // 1.13 / 1.15 / 1.18: from 2,048 on.
   size_t free_b = 0, total_b = 0;
   CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-  const size_t cells = (size_t)s.p.nr * s.p.nxi;
-  const bool corners = h->precision == WAKE_MIXED && cn == 1 && !wide_nt && s.p.geometry != WAKE_SLAB && s.np <= 4096 &&
-                       s.p.n_beam >= (int64_t)2048 * s.p.nxi &&
-                       ((size_t)std::min(nsteps, 1024) + 1) * sizeof(float4) * cells <= free_b / 4;
+  const size_t grids_b = (free_b + s.pgrid_bytes) / 4, cells = (size_t)s.p.nr * s.p.nxi;
+  bool corners = h->precision == WAKE_MIXED && cn == 1 && !wide_nt && s.p.geometry != WAKE_SLAB &&
+                 s.p.n_beam >= (int64_t)2048 * s.p.nxi &&
+                 ((size_t)std::min(nsteps, 1024) + 1) * sizeof(float4) * cells <= grids_b;
+  if (corners) {
+    const int n = step_max_ctas_corners(s.p.nr + 1, s.np);  // of the kernel that is launched
+    corners = n > 0;
+    if (corners) ctas_max = std::min(ctas_max, n);
+  }
   const size_t gbytes = corners ? sizeof(float4) * cells : gs * s.ng;
-  const int chmax = (int)std::min<size_t>(1024, std::max<size_t>(1, free_b / 4 / gbytes - 1));
+  const int chmax = (int)std::min<size_t>(1024, std::max<size_t>(2, grids_b / gbytes) - 1);
   const int wnt = wide_nt;  // 0: the tiled step kernel
   const bool wide64 = wnt && fp64;  // the FP64 wide form: node arrays in the ring buffer
   const size_t rb = wnt && cn > 1 ? step_wide_cluster_ring_bytes(s.np, cn)  // per cluster
@@ -1359,21 +1378,8 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
     if (L < nsteps - done && L >= ctas_max) L = L / ctas_max * ctas_max;
     const int ch = (int)std::max<long long>(1, L);
     const int dcap = (int)dcap_l;
-    if (s.pgrid_cap < ch + 1 || s.pgrid_bytes != gbytes) {
-      void *old[] = {s.pgrids, s.progress, s.defer_cnt};
-      for (void *q : old)
-        if (q) cudaFree(q);
-      s.pgrids = nullptr;
-      s.progress = nullptr;
-      s.defer_cnt = nullptr;
-      s.pgrid_cap = 0;
-      const int cap = std::min(nsteps, chmax);
-      if ((rc = dalloc(&s.pgrids, gbytes * (cap + 1))) || (rc = dalloc(&s.progress, sizeof(int) * cap)) ||
-          (rc = dalloc(&s.defer_cnt, 2 * sizeof(int) * cap)))
-        return rc;
-      s.pgrid_cap = cap + 1;
-      s.pgrid_bytes = gbytes;
-    }
+    const int cap = std::min(nsteps, chmax);  // the call's longest launch
+    if ((s.pgrid_bytes < gbytes * (ch + 1) || s.pstep_cap < ch) && (rc = alloc_steps(s, cap, gbytes * (cap + 1)))) return rc;
     if (s.defer_bytes < sizeof(int2) * (size_t)dcap * ch) {
       if (s.defer_list) cudaFree(s.defer_list);
       s.defer_list = nullptr;
