@@ -389,25 +389,30 @@ int probe_tile(wake_sim *h, const Sim &s, const SimDesc &d, const TileFns &f, do
   return WAKE_OK;
 }
 
-// CTAs per simulation (or beam step) when `count` of them run at once: 1, or a cluster that shares
-// each one's rings.  The field solves are repeated by every CTA and the sums over the cluster cost
-// about 13k cycles a slice (8 CTAs), so a cluster pays where a CTA's ring passes cost more.  FP64 (its
-// pipe bounds the ring passes; linear march alone 20.1 ms with one CTA, 13.2 with 4, 13.1 with 8; 256
-// rings 15.6, 11.8 and 12.0 ms; 24 steps 103 ms, 48 with 4): as many CTAs as leave 64 rings to each and
-// fit the GPU at once.  Mixed (one march alone, 1 / 4 / 8 CTAs: 512 rings 2.8 / 3.5 / 3.6 ms, 1024 6.4 /
-// 5.8 / 6.0, 1536 8.7 / 7.7 / 6.4, 4096 69.5 / 58.8 / 41.8): 4 from 1024 rings and 8 from 1536, and only
-// while half of the SMs stay free for other streams' work, since a cluster does more work in all.
+// CTAs per simulation (FP64) or beam step (FP64, mixed) when `count` of them run at once: 1, or a
+// cluster that shares each one's rings.  The field solves are repeated by every CTA and the sums over the
+// cluster cost about 13k cycles a slice (8 CTAs), so a cluster pays where a CTA's ring passes cost more.
+// ms, 1 / 2 / 4 / 8 CTAs, by rings:
+//   FP64 march of 100 slices, alone: 128 rings 5.3 / 4.4 / 4.4 / 4.7, 256 6.4 / 5.2 / 5.0 / 5.1, 512 8.0 / 5.9 /
+//   5.2 / 5.2, 1024 12.6 / 8.3 / 6.0 / 5.5, 2048 22.1 / 13.7 / 9.3 / 7.1, 4096 38.4 / 21.8 / 13.9 / 9.6; 24 at
+//   once, each: 512 0.33 / 0.25 / 0.22 / 0.43, 2048 0.93 / 0.57 / 0.39 / 0.59
+//   9 FP64 steps: 256 21.3 / 16.4 / 14.9 / 14.7, 1024 41.1 / 27.2 / 19.1 / 17.4, 2048 68.4 / 44.0 / 28.9 / 21.6; 18:
+//   256 24.6 / 18.3 / 16.2 / 17.7, 2048 75.3 / 48.1 / 31.6 / 29.8
+//   9 mixed steps: 256 3.7 / 4.8 / 4.7 / 4.8, 1024 5.5 / 7.6 / 5.4 / 5.3, 2048 7.5 / 9.7 / 8.3 / 6.0, 4096 10.5 / 13.7
+//   / 10.9 / 9.6; 18: 1024 5.9 / 7.9 / 5.6 / 5.7, 2048 8.1 / 10.1 / 8.7 / 6.6
+// FP64: 2 CTAs from 128 rings, 4 from 256, 8 from 2048.  Mixed: 4 from 1024, 8 from 1536 (4 gain nothing
+// there).  8 of them, and the mixed forms', only while half of the SMs stay free for other streams' work.
 int pick_cluster(wake_sim *h, const wake_sim::TileClass &k, int count, bool step) {
   if (h->tile_nt_forced || h->precision == WAKE_MIXED64 || (h->precision == WAKE_MIXED && !step)) return 1;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
   const bool fp64 = h->precision == WAKE_FP64;
-  int cn = 1;
+  int cn;
   if (fp64)
-    for (int c = 8; c > 1 && cn == 1; c /= 2) cn = count * c <= sms && k.npmax >= 64 * c ? c : 1;
+    cn = k.npmax >= 2048 && count * 16 <= sms ? 8 : k.npmax >= 256 && count * 4 <= sms ? 4 : k.npmax >= 128 && count * 2 <= sms ? 2 : 1;
   else
-    cn = k.npmax >= 1536 && count * 16 <= sms ? 8 : (k.npmax >= 1024 && count * 8 <= sms ? 4 : 1);
+    cn = k.npmax >= 1536 ? (count * 16 <= sms ? 8 : 1) : k.npmax >= 1024 && count * 8 <= sms ? 4 : 1;
   return cn > 1 && cluster_max(h->precision, k.slab, step, k.n1max, k.npmax, cn) >= count ? cn : 1;
 }
 
