@@ -272,14 +272,13 @@ static __global__ void nb_from_corners_kernel(const float4 *__restrict__ g, floa
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x)
     nb[t] = corner_node(g, (int)(t / n1), (int)(t % n1), nr, nxi);
 }
-// The deposit of a launch's first step in that layout, divided by the hats' volumes.
+// The deposit of a launch's first step in that layout (cylinder), divided by the hats' volumes.
 static __global__ void beam_deposit_corners_kernel(BeamDesc b, float4 *g) {
   using W = BeamWide<float>;
-  const float inv_dr = (float)(1.0 / b.dr), wf = (float)(b.slab ? 1.0 / (b.dr * b.dxi) : 1.0 / (b.dr * b.dr * b.dxi));
+  const float inv_dr = (float)(1.0 / b.dr), wf = (float)(1.0 / (b.dr * b.dr * b.dxi));
   const W::Box bx = W::box(b.dxi, b.ximax, b.ffi, b.ffx);
   const int nr = b.nr;
-  auto iv = [&](int i) -> float {  // 1 / V_i in units of 1 / dr^2 (slab 1 / dx)
-    if (b.slab) return (i == 0 || i == nr) ? 2.f : 1.f;
+  auto iv = [&](int i) -> float {  // 1 / V_i in units of 1 / dr^2
     return i == 0 ? 6.f : (i == nr ? 1.f / (0.5f * nr - (float)(1.0 / 6.0)) : 1.f / (float)i);
   };
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < b.n_cap; j += (int64_t)gridDim.x * blockDim.x) {

@@ -959,8 +959,8 @@ __device__ __forceinline__ void move_ring(int c, R f, R r, R dx, R dy, R ux, R u
   R delta = (R)0;
   ex = (R)1;  // the direction of the new position in the frame
   ey = (R)0;
-  // the momentum by one division of the products, not through ex: x (1/x) falls short of 1 by a
-  // rounding, the same way every slice (the mixed linear march's error against 64 bits doubled)
+  // the momentum as the products' sum times 1/r', not through ex and ey: their roundings act the same way
+  // every slice (the mixed linear march's error against 64 bits doubled)
   if constexpr (sizeof(R) == 8) {
     if (r2 > tiny_r2<R>()) {
       R rr, irr;

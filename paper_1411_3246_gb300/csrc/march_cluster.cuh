@@ -73,22 +73,6 @@ struct ClusterForm {
     }
     return k;
   }
-  static void config(cudaLaunchConfig_t *c, cudaLaunchAttribute *at, int clusters, int cn, size_t bytes, bool coop,
-                     cudaStream_t stream) {
-    *c = cudaLaunchConfig_t{};
-    c->gridDim = dim3(clusters * cn);
-    c->blockDim = dim3(kClNT);
-    c->dynamicSmemBytes = bytes;
-    c->stream = stream;
-    at[0] = at[1] = cudaLaunchAttribute{};
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cn;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeCooperative;
-    at[1].val.cooperative = 1;
-    c->attrs = at;
-    c->numAttrs = coop ? 2 : 1;
-  }
   // Clusters of cn that the GPU holds at once (0: the form does not fit).
   static int max_clusters(bool slab, bool step, int n1, int np, int cn) {
     size_t bytes;
@@ -97,7 +81,7 @@ struct ClusterForm {
     if (!k) return 0;
     cudaLaunchConfig_t c;
     cudaLaunchAttribute at[2];
-    config(&c, at, 1, cn, bytes, false, nullptr);
+    cluster_config(&c, at, 1, cn, kClNT, bytes, false, nullptr);
     int n = 0;
     return cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess ? n : 0;
   }
@@ -108,7 +92,7 @@ struct ClusterForm {
     if (!k) return e != cudaSuccess ? e : cudaErrorInvalidValue;
     cudaLaunchConfig_t c;
     cudaLaunchAttribute at[2];
-    config(&c, at, clusters, cn, bytes, step, stream);
+    cluster_config(&c, at, clusters, cn, kClNT, bytes, step, stream);
     return cudaLaunchKernelExC(&c, k, args);
   }
 };

@@ -56,6 +56,25 @@ int batch_step_max_ctas(int max_n1, int bnt);
 size_t batch_ring_bytes(int max_np, int bnt);
 cudaError_t launch_batch_steps(const BatchArgs &b, int max_n1, int bnt, int ctas, cudaStream_t stream);
 
+// The configuration of a launch of `clusters` clusters of cn CTAs of nt threads (coop: all resident at
+// once).  at: two attributes that outlive the launch.
+inline void cluster_config(cudaLaunchConfig_t *c, cudaLaunchAttribute *at, int clusters, int cn, int nt, size_t bytes, bool coop,
+                           cudaStream_t stream) {
+  *c = cudaLaunchConfig_t{};
+  c->gridDim = dim3(clusters * cn);
+  c->blockDim = dim3(nt);
+  c->dynamicSmemBytes = bytes;
+  c->stream = stream;
+  at[0] = at[1] = cudaLaunchAttribute{};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cn;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;
+  at[1].val.cooperative = 1;
+  c->attrs = at;
+  c->numAttrs = coop ? 2 : 1;
+}
+
 // Clusters of cn = 2, 4 or 8 CTAs per simulation (FP64) or beam step (FP64, mixed; march_cluster.cuh):
 // how many the GPU holds at once (0: the form, grid or ring count has none), and the launches: `count`
 // simulations of at most n1 nodes and np rings, or the steps of `a` on `clusters` resident clusters.

@@ -96,22 +96,6 @@ cudaError_t launch_step_wide(const PipeArgs &a, int nt, int ctas, cudaStream_t s
 
 // The steps of clusters of cn CTAs of 512 threads: ring bytes of one cluster, clusters the GPU holds
 // at once (0: does not fit), launch.
-static void wide_cluster_config(cudaLaunchConfig_t *c, cudaLaunchAttribute *at, int clusters, int cn, size_t bytes, bool coop,
-                                cudaStream_t stream) {
-  *c = cudaLaunchConfig_t{};
-  c->gridDim = dim3(clusters * cn);
-  c->blockDim = dim3(kWideNT);
-  c->dynamicSmemBytes = bytes;
-  c->stream = stream;
-  at[0] = at[1] = cudaLaunchAttribute{};
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cn;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeCooperative;
-  at[1].val.cooperative = 1;
-  c->attrs = at;
-  c->numAttrs = coop ? 2 : 1;
-}
 size_t step_wide_cluster_ring_bytes(int np, int cn) {
   return (size_t)cn * wide_share_bytes<float, kWideNT, kWidePPT>((np + cn - 1) / cn);
 }
@@ -122,7 +106,7 @@ int step_wide_cluster_max(int n1, int cn) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   cudaLaunchConfig_t c;
   cudaLaunchAttribute at[2];
-  wide_cluster_config(&c, at, 1, cn, smem, false, nullptr);
+  cluster_config(&c, at, 1, cn, kWideNT, smem, false, nullptr);
   int n = 0;
   return cudaOccupancyMaxActiveClusters(&n, kern, &c) == cudaSuccess ? n : 0;
 }
@@ -133,7 +117,7 @@ cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cu
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t c;
   cudaLaunchAttribute at[2];
-  wide_cluster_config(&c, at, clusters, cn, smem, true, stream);
+  cluster_config(&c, at, clusters, cn, kWideNT, smem, true, stream);
   PipeArgs arg = a;
   void *args[] = {&arg};
   return cudaLaunchKernelExC(&c, (const void *)kern, args);
