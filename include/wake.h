@@ -224,6 +224,14 @@ int wake_step(wake_sim *s, int nsteps);
 int wake_tile(wake_sim *s, int sim, int *nt, int *ppt);
 
 /*
+ * The forms simulation `sim` last ran in: CTAs that share its plain march (0 before the first), CTAs that
+ * share each beam step of the last wake_step launch, and 1 in by_cells if that launch kept the beam density
+ * by cells (0 and 0 where the steps took the separate calls).  Instrumentation only: the paper has no
+ * counterpart.
+ */
+int wake_forms(wake_sim *s, int sim, int *march_ctas, int *step_ctas, int *by_cells);
+
+/*
  * Device time in milliseconds of the pipelined step kernels launched by the last wake_step
  * call (0 if it took the separate calls), measured with CUDA events on the handle's stream;
  * synchronous.  Instrumentation only: the paper has no counterpart.

@@ -54,6 +54,7 @@ struct Sim {
   void *pgrids = nullptr;
   size_t pgrid_bytes = 0;  // all of them
   int pstep_cap = 0;       // steps the progress and list counters hold
+  int step_ctas = 0, step_by_cells = 0;  // the last wake_step's forms (wake_forms)
   int *progress = nullptr;
   void *pring = nullptr;
   size_t pring_bytes = 0;
@@ -1258,6 +1259,7 @@ int step_batch_pipelined(wake_sim *h, int nsteps) {
       CUDA_TRY(cudaMemcpyAsync(s.nb, (char *)s.pgrids + sizeof(float) * s.ng * (ch - 1), sizeof(float) * s.ng,
                                cudaMemcpyDeviceToDevice, h->stream));
       s.marched = true;
+      s.step_ctas = 1;
     }
     done += ch;
   }
@@ -1495,6 +1497,8 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
                           : wide64 ? launch_step_wide_fp64(a, ctas, h->stream)
                                  : (wnt ? launch_step_wide(a, wnt, ctas, h->stream) : launch_step(h->precision, a, s.np, ctas, h->stream));
     if (e != cudaSuccess) return fail(WAKE_ECUDA, std::string("pipelined step launch: ") + cudaGetErrorString(e));
+    s.step_ctas = cn;
+    s.step_by_cells = corners;
     CUDA_TRY(cudaEventRecord(h->ev[h->ev_used].second, h->stream));
     ++h->ev_used;
     done += ch;
@@ -1519,6 +1523,7 @@ int wake_step(wake_sim *h, int nsteps) {
   if (!h || nsteps < 0) return fail(WAKE_EINVAL, "wake_step: null handle or nsteps < 0");
   h->ev_used = 0;
   if (nsteps == 0) return WAKE_OK;
+  for (auto &s : h->sims) s.step_ctas = s.step_by_cells = 0;
   if (h->n == 1 && h->sims[0].trap_gamma > 0.0) return step_sequential(h, nsteps);  // trapping: step by step
   if (h->n == 1 && h->sims[0].p.n_beam > 0) {
     Sim &s = h->sims[0];
@@ -1547,6 +1552,16 @@ int wake_tile(wake_sim *h, int sim, int *nt, int *ppt) {
     *nt = f.nt;
     *ppt = f.ppt;
   }
+  return WAKE_OK;
+}
+
+int wake_forms(wake_sim *h, int sim, int *march_ctas, int *step_ctas, int *by_cells) {
+  int rc = check_handle(h, sim);
+  if (rc) return rc;
+  if (!march_ctas || !step_ctas || !by_cells) return fail(WAKE_EINVAL, "wake_forms: null output");
+  *march_ctas = h->planned ? h->classes[h->tile_of[sim]].cluster : 0;
+  *step_ctas = h->sims[sim].step_ctas;
+  *by_cells = h->sims[sim].step_by_cells;
   return WAKE_OK;
 }
 

@@ -19,7 +19,7 @@ WAKE_CYLINDRICAL, WAKE_SLAB = 0, 1
 
 # every entry point the header declares
 EXPORTS = ["wake_init", "wake_load_plasma", "wake_load_beam", "wake_set_beam", "wake_beam_deposit", "wake_plasma_march",
-           "wake_plasma_march_traj", "wake_beam_push", "wake_beam_push_steps", "wake_bind_fields", "wake_step", "wake_tile", "wake_step_kernel_ms", "wake_get_fields", "wake_get_nb", "wake_get_beam",
+           "wake_plasma_march_traj", "wake_beam_push", "wake_beam_push_steps", "wake_bind_fields", "wake_step", "wake_tile", "wake_forms", "wake_step_kernel_ms", "wake_get_fields", "wake_get_nb", "wake_get_beam",
            "wake_diagnostics", "wake_status", "wake_set_trapping", "wake_trapped", "wake_beam_deposit_noalloc", "wake_adjoint_init",
            "wake_adjoint_forward", "wake_adjoint_backward", "wake_adjoint_destroy", "wake_last_error", "wake_destroy"]
 WAKE_NOALLOC_MAX_NODES = 524288
@@ -64,6 +64,7 @@ def lib():
         L.wake_step.argtypes = [vp, i32]
         L.wake_step_kernel_ms.argtypes = [vp, C.POINTER(C.c_float)]
         L.wake_tile.argtypes = [vp, i32, C.POINTER(C.c_int), C.POINTER(C.c_int)]
+        L.wake_forms.argtypes = [vp, i32, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
         L.wake_get_fields.argtypes = [vp, i32, vp, vp, vp, vp]
         L.wake_get_nb.argtypes = [vp, i32, vp]
         L.wake_get_beam.argtypes = [vp, i32, vp, vp]
@@ -161,6 +162,13 @@ def wake_bind_fields(h, sim, psi, ez, er, bth):
 
 def wake_step(h, nsteps):
     _check(lib().wake_step(h, nsteps))
+
+
+def wake_forms(h, sim):
+    """(CTAs sharing a march, CTAs sharing a pipelined step, density kept by cells) as last run."""
+    out = [C.c_int() for _ in range(3)]
+    _check(lib().wake_forms(h, sim, *[C.byref(v) for v in out]))
+    return tuple(v.value for v in out)
 
 
 def wake_tile(h, sim):
