@@ -49,6 +49,7 @@ cudaError_t launch_step_wide_fp64(const PipeArgs &a, int ctas, cudaStream_t stre
 // Pipelined steps in the wide form, one cluster of cn CTAs of 512 threads per step.
 size_t step_wide_cluster_ring_bytes(int np, int cn);
 int step_wide_cluster_max(int n1, int cn);
+int step_wide_chunks(int np, int cn);  // chunks of rings per CTA
 cudaError_t launch_step_wide_cluster(const PipeArgs &a, int cn, int clusters, cudaStream_t stream);
 // Pipelined steps of many simulations (pipeline.cuh batch_step_kernel), wide form.
 struct BatchArgs;

@@ -99,6 +99,7 @@ cudaError_t launch_step_wide(const PipeArgs &a, int nt, int ctas, cudaStream_t s
 size_t step_wide_cluster_ring_bytes(int np, int cn) {
   return (size_t)cn * wide_share_bytes<float, kWideNT, kWidePPT>((np + cn - 1) / cn);
 }
+int step_wide_chunks(int np, int cn) { return ((np + cn - 1) / cn + kWideNT * kWidePPT - 1) / (kWideNT * kWidePPT); }
 int step_wide_cluster_max(int n1, int cn) {
   auto kern = step_wide_cluster_kernel<StepWide, kWideNT, kWidePPT>;
   const size_t smem = step_wide_smem(n1);

@@ -393,28 +393,31 @@ int probe_tile(wake_sim *h, const Sim &s, const SimDesc &d, const TileFns &f, do
 // CTAs per simulation (FP64) or beam step (FP64, mixed) when `count` of them run at once: 1, or a
 // cluster that shares each one's rings.  The field solves are repeated by every CTA and the sums over the
 // cluster cost about 13k cycles a slice (8 CTAs), so a cluster pays where a CTA's ring passes cost more.
-// ms, 1 / 2 / 4 / 8 CTAs, by rings:
-//   FP64 march of 100 slices, alone: 128 rings 5.3 / 4.4 / 4.4 / 4.7, 256 6.4 / 5.2 / 5.0 / 5.1, 512 8.0 / 5.9 /
-//   5.2 / 5.2, 1024 12.6 / 8.3 / 6.0 / 5.5, 2048 22.1 / 13.7 / 9.3 / 7.1, 4096 38.4 / 21.8 / 13.9 / 9.6; 24 at
-//   once, each: 512 0.33 / 0.25 / 0.22 / 0.43, 2048 0.93 / 0.57 / 0.39 / 0.59
-//   9 FP64 steps: 256 21.3 / 16.4 / 14.9 / 14.7, 1024 41.1 / 27.2 / 19.1 / 17.4, 2048 68.4 / 44.0 / 28.9 / 21.6; 18:
-//   256 24.6 / 18.3 / 16.2 / 17.7, 2048 75.3 / 48.1 / 31.6 / 29.8
-//   9 mixed steps: 256 3.7 / 4.8 / 4.7 / 4.8, 1024 5.5 / 7.6 / 5.4 / 5.3, 2048 7.5 / 9.7 / 8.3 / 6.0, 4096 10.5 / 13.7
-//   / 10.9 / 9.6; 18: 1024 5.9 / 7.9 / 5.6 / 5.7, 2048 8.1 / 10.1 / 8.7 / 6.6
-// FP64: 2 CTAs from 128 rings, 4 from 256, 8 from 2048.  Mixed: 4 from 1024, 8 from 1536 (4 gain nothing
-// there).  8 of them, and the mixed forms', only while half of the SMs stay free for other streams' work.
+// ms alone / each of three such calls on three streams, with 1, 2, 4 and 8 CTAs:
+//   FP64 march of 60 slices: 128 cells, 128 rings 3.4/1.1, 3.0/1.0, 3.0/1.0, 3.2/1.1; 256 rings 3.8/1.3, 3.1/1.0,
+//   3.0/1.0, 3.1/1.0; 256 cells, 512 rings 5.2/1.7, 4.2/1.4, 3.7/1.2, 3.7/1.2; 512 cells, 1024 rings 8.7/2.9, 6.8/2.3,
+//   5.4/1.8, 5.1/1.7; 2048 rings 14.0/4.7, 9.5/3.2, 6.7/2.2, 5.5/1.8.  (24 simulations of 512 rings at once, 100
+//   slices, each: 0.33, 0.25, 0.22, 0.43.)
+//   FP64 steps, 512 cells, 512 rings: 9 steps 10.1/3.4, 9.4/3.1, 8.1/2.7, 8.0/6.8; 18 steps 12.9/4.3, 11.7/3.9, 10.1/5.0;
+//   36 steps 18.6/6.2, 16.4/8.0, 13.8/13.7.  2048 rings: 9 steps 19.7/6.6, 14.6/4.9, 10.4/3.5, 8.7/7.5.
+//   Mixed steps, 1 / 4 / 8 CTAs: 256 cells, 1024 rings, 9 steps 3.7/1.2, 4.0/1.3, 4.0/1.4; 1536 rings 4.7/1.6, 5.4/1.8,
+//   4.1/1.4; 384 cells 4.7/1.6, 5.7/1.8, 4.4/1.5; 512 cells 4.9/1.7, 6.0/2.0, 4.8/1.7; 768 cells 5.3/1.8, 6.5/2.1, 5.5/5.0;
+//   256 cells, 2048 rings, 9 steps 4.8/1.6, 5.6/1.8, 4.2/1.5, 18 steps 5.3/1.7, 6.0/2.0, 4.7/2.4.
+// FP64: 2 CTAs from 128 rings, 4 from 256, 8 from 2048 (the next more gains little for twice the SMs).  Mixed:
+// 8 from 1536 rings up to 384 cells, while half of the SMs stay free (4 lose to one CTA throughout).  And
+// only while the GPU holds three such launches, or the next stream's would wait for this one's.
 int pick_cluster(wake_sim *h, const wake_sim::TileClass &k, int count, bool step) {
   if (h->tile_nt_forced || h->precision == WAKE_MIXED64 || (h->precision == WAKE_MIXED && !step)) return 1;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
   const bool fp64 = h->precision == WAKE_FP64;
-  int cn;
-  if (fp64)
-    cn = k.npmax >= 2048 && count * 16 <= sms ? 8 : k.npmax >= 256 && count * 4 <= sms ? 4 : k.npmax >= 128 && count * 2 <= sms ? 2 : 1;
-  else
-    cn = k.npmax >= 1536 ? (count * 16 <= sms ? 8 : 1) : k.npmax >= 1024 && count * 8 <= sms ? 4 : 1;
-  return cn > 1 && cluster_max(h->precision, k.slab, step, k.n1max, k.npmax, cn) >= count ? cn : 1;
+  for (int cn = 8; cn > 1; cn /= 2) {
+    const bool pays = fp64 ? k.npmax >= (cn == 8 ? 2048 : cn == 4 ? 256 : 128)
+                           : cn == 8 && k.npmax >= 1536 && k.n1max <= 385 && 16 * count <= sms;
+    if (pays && count * cn <= sms && cluster_max(h->precision, k.slab, step, k.n1max, k.npmax, cn) >= 3 * count) return cn;
+  }
+  return 1;
 }
 
 // Choose a tile per simulation (the best probe score per distinct (Nr, Np); the only
@@ -1318,13 +1321,20 @@ int step_pipelined(wake_sim *h, int nsteps, int ctas_max, int wide_nt) {
     if (cn > 1) ctas_max = cluster_max(h->precision, k.slab, true, k.n1max, k.npmax, cn);
   }
   if (wide_nt == 512 && h->precision == WAKE_MIXED && !h->tile_nt_forced && !h->step_form) {
-    // wide form, a cluster per step while all steps run at once: the ring passes are nearly all of
-    // its time (8 steps of 2,048 cells and 65,536 rings: 126 ms with one CTA each)
+    // wide form, a cluster per step while all steps run at once: as many CTAs as still leave each fewer
+    // chunks of rings, and while the GPU holds three such launches (pick_cluster; from 32,768 rings one,
+    // their ring passes being nearly all of the time).  ms alone / each of three calls on three streams, 1 /
+    // 2 / 4 / 8 CTAs, 40 slices, 9 steps: 4,800 rings (2 chunks) 5.3/1.8, 4.7/1.6, 4.7/1.6, 4.7/3.8; 8,800 (3) 7.5/2.6,
+    // 7.5/2.5, 5.1/1.8, 5.1/4.1; 18,000 (5) 12.5/4.2, 10.9/3.7, 8.4/2.9, 5.9/4.8; 65,536 (16) 39.7/13.8, 27.4/9.5, 15.8/5.6,
+    // 10.2/8.3
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int launches = s.np >= 32768 ? 1 : 3;
     for (int c = 8; c > 1 && cn == 1; c /= 2)
-      if (nsteps * c <= sms && step_wide_cluster_max(s.p.nr + 1, c) >= nsteps) cn = c;
+      if (step_wide_chunks(s.np, c) < step_wide_chunks(s.np, c / 2) && nsteps * c <= sms &&
+          step_wide_cluster_max(s.p.nr + 1, c) >= launches * nsteps)
+        cn = c;
     if (cn > 1) ctas_max = nsteps;
   }
   const int fp64 = h->precision == WAKE_FP64;

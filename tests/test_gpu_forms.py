@@ -112,12 +112,15 @@ def test_fp64_slipping_steps_by_one_cta(wk, monkeypatch):
     assert np.array_equal(lost, bm["lost"] != 0)
 
 
-# (nr, nxi, ppc, n_beam, forced tile, form): one CTA with node grids, clusters of 4 and 8, wide clusters, grids by cells
+# (nr, nxi, ppc, n_beam, forced tile, form): one CTA with node grids, clusters of tiles, wide clusters, grids by cells
 @pytest.mark.parametrize("nr,nxi,ppc,n_beam,tile,forms", [
     (64, 64, 4, 20001, None, (1, 0)),
-    (128, 64, 8, 20001, None, (4, 0)),
+    (128, 64, 8, 20001, None, (1, 0)),
     (128, 64, 12, 20001, None, (8, 0)),
-    (800, 40, 6, 20001, None, (8, 0)),
+    (512, 40, 4, 20001, None, (1, 0)),
+    (800, 40, 6, 20001, None, (2, 0)),
+    (1030, 40, 20, 20001, None, (4, 0)),
+    (1030, 40, 32, 20001, None, (8, 0)),
     (64, 16, 4, 33001, None, (1, 1)),
     (140, 16, 8, 33001, "512", (1, 1)),
 ])
@@ -159,8 +162,8 @@ def test_density_by_cells_of_four_and_eight_rings_per_thread(wk, nr, ppc, monkey
     assert np.abs(nb - ref).max() <= (nr * 2.0 ** -24 + 1.2e-5) * np.abs(ref).max()
 
 
-@pytest.mark.parametrize("nr,ppc", [(128, 16), (800, 6)])
-def test_a_mixed_cluster_s_wait_runs_out(wk, nr, ppc, monkeypatch):
+@pytest.mark.parametrize("nr,ppc,ctas", [(128, 16, 8), (800, 6, 2), (1030, 32, 8)])
+def test_a_mixed_cluster_s_wait_runs_out(wk, nr, ppc, ctas, monkeypatch):
     """WAKE_SPIN_LIMIT=0, as in test_gpu_faults: the clusters (of tiles, of the wide form) give up together, the
     status says so, and a fresh handle runs."""
     cfg = synth.config_blowout(n_beam=1 << 14, nr=nr, nxi=64)
@@ -174,7 +177,7 @@ def test_a_mixed_cluster_s_wait_runs_out(wk, nr, ppc, monkeypatch):
             wk.wake_load_plasma(s.h, 0, _cuda(synth.plasma_normals(cfg)))
             wk.wake_load_beam(s.h, 0, _cuda(synth.beam_normals(cfg)))
             wk.wake_step(s.h, 6)
-            assert wk.wake_forms(s.h, 0)[1] == 8
+            assert wk.wake_forms(s.h, 0)[1] == ctas
             assert s.status(0) == status
             xyz, lost = s.beam(0)
         if limit is None:
